@@ -102,7 +102,7 @@ extern "C" abilu_status abilu_factors_create(abilu_pattern p, abilu_dtype dtype,
     const size_t ba = narrow ? rnd(sizeof(float) * BB * (size_t)v.nnzb) : 0;
     const size_t br = narrow ? rnd(sizeof(float) * BS * (size_t)v.n) : 0;
     const size_t bus = dtype == ABILU_F32 ? bu : 0;   // Dinv-scaled upper blocks
-    const size_t bcd = rnd(sizeof(int) * ((size_t)(v.nwork + 31) / 32 + 1));
+    const size_t bcd = rnd(sizeof(int) * (((size_t)v.nwork + 7) / 8 + 1));
     const size_t total = 2 * bl + 2 * bu + 3 * bd + 4 * bv + bc + bs + bp + ba + br + bus + bcd;
     abilu_factors f = new abilu_factors_s();
     memset(f, 0, sizeof *f);

@@ -1244,7 +1244,7 @@ static long long arena_bytes(const SrvCaps &c) {
     const long long bv = r(vt * BS * c.rows);
     b += 2 * bl + 2 * bu + 3 * bd + 4 * bv + r(8 * 8) + r((long long)solve_state_bytes()) +
          r(8LL * 66 * red_ctas()) + (narrow ? r(4 * BB * c.blocks) + r(4 * BS * c.rows) : 0) +
-         (c.dtype == ABILU_F32 ? bu : 0) + r(4 * ((c.work + 31) / 32 + 1));
+         (c.dtype == ABILU_F32 ? bu : 0) + r(4 * ((c.work + 7) / 8 + 1));
     return b;
 }
 

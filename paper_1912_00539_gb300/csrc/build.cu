@@ -413,7 +413,8 @@ k_build_blocks_sync(PatternView P, const float *__restrict__ A32, const T *__res
 // of the list, or 32 for sizes that are not multiples of 64) taken at a stride
 // of nchunks sub-chunks: sub-chunks c, c + nchunks, c + 2 nchunks, ...  Each
 // sub-chunk is done in steps of 8 blocks (one block per quad, consecutive
-// blocks, so a step stays within one kind).
+// blocks, so a step stays within one kind).  Small lists take tickets of
+// 8-block sub-chunks (SMALL_TICKET).
 //
 // Why the stride: the ILU fixed-point residual after a given number of sweeps
 // falls as the blocks in flight (resident warps x blocks per ticket) span
@@ -435,17 +436,32 @@ k_build_blocks_sync(PatternView P, const float *__restrict__ A32, const T *__res
 // completed sweeps, and publishes s + 1 after its writes.  A wait points only
 // to a smaller ticket, held by a resident warp, so every wait ends.  No bulk
 // copy is in flight in this kernel, so a warp that gives up can simply return.
-constexpr int WARP_CHUNK = 128;   // default work blocks per ticket (abilu_factors_set_build_chunk)
+constexpr int WARP_CHUNK = 128;   // largest default ticket (abilu_factors_set_build_chunk)
 
-// Sub-chunk size of a ticket of `wchunk` blocks (a multiple of 32) and the
-// number of tickets per sweep: the kernel and its launcher share this.
-__host__ __device__ __forceinline__ int build_sub(int wchunk) { return wchunk % 64 == 0 ? 64 : 32; }
-__host__ __device__ __forceinline__ long long build_tickets(int nwork, int wchunk) {
-    const int sub = build_sub(wchunk);
-    const long long nsub = (nwork + sub - 1) / sub;
+// Sub-chunk size of a ticket of `wchunk` blocks given by the caller (a
+// multiple of 32) and the number of tickets per sweep: the kernel and its
+// launcher share the latter.
+static int build_sub(int wchunk) { return wchunk % 64 == 0 ? 64 : 32; }
+__host__ __device__ __forceinline__ long long build_tickets(int nwork, int wchunk, int sub) {
+    const long long nsub = ((long long)nwork + sub - 1) / sub;
     const int per = wchunk / sub;
     return (nsub + per - 1) / per;
 }
+
+// Lists of at most SMALL_TICKET blocks per resident warp (6,080 warps at 40 per
+// SM: 389k blocks, 155k grid cells) take the smallest ticket of 8-block
+// sub-chunks that gives no more tickets than warps, so a sweep is at most one
+// ticket per warp.  Such lists are bound by the serial steps of a ticket: with
+// 128-block tickets a 20k-block list kept 160 warps busy for 16 dependent
+// steps per sweep.  Measured, 4 sweeps with the prepare pass (us, 128-block
+// tickets -> this rule): 2.4k blocks 80 -> 30, 20k 91 -> 34, 82k 96 -> 53, 144k
+// 105 -> 68, 327k 149 -> 124; 8 sweeps of 326k (wall-normal coupling 100x) 231 ->
+// 178.  Above the line the 64-block groups win: 737k blocks 253 against 286.
+// FGMRES iterations over those lists: the same or within one at the settings
+// used with them.  Fixing each warp's blocks for all sweeps (no tickets, no
+// flags) was faster still (20k: 22) but lets warps drift apart by sweeps:
+// FGMRES took 24 iterations where the ordered tickets take 7.
+constexpr int SMALL_TICKET = 64;
 
 template <typename T, bool ORDERED, int SUB>
 __global__ void __launch_bounds__(BUILD_THREADS, 5)   // 48 registers: measured fastest (4, 6 slower)
@@ -458,7 +474,7 @@ k_build_blocks_async(PatternView P, const float *__restrict__ A32, T *L, T *U, T
     __shared__ __align__(16) float sh_q[WORK_PER_CTA * QUAD_SCRATCH];
     // at most one warp per chunk: more would sweep the same blocks at once
     if (blockIdx.x * (BUILD_THREADS / 32) + (threadIdx.x >> 5) >= max_warps) return;
-    const long long nchunks = build_tickets(P.nwork, wchunk);
+    const long long nchunks = build_tickets(P.nwork, wchunk, SUB);
     const long long total = nchunks * nsweeps;
     const int stride = (int)nchunks * SUB;   // blocks between a ticket's sub-chunks
     const int lane = threadIdx.x & 31;
@@ -483,9 +499,9 @@ k_build_blocks_async(PatternView P, const float *__restrict__ A32, T *L, T *U, T
             if (!__shfl_sync(0xffffffffu, ok, 0)) return;
         }
         // step k: sub-chunk chunk + (k / steps) nchunks, its 8 blocks k mod
-        // steps (32-bit: block indices stay below (nsub + wchunk / 32) * 64,
+        // steps (32-bit: block indices stay below (nsub + wchunk / SUB) * SUB,
         // and nwork <= nnzb < 2^31 - 2^16)
-        constexpr int SSH = SUB == 64 ? 3 : 2;   // log2(steps per sub-chunk)
+        constexpr int SSH = SUB == 64 ? 3 : SUB == 32 ? 2 : 0;   // log2(steps per sub-chunk)
         const int base = chunk * SUB + (lane >> 2);
 #pragma unroll 1
         for (int k = 0; k < wchunk / 8; k++) {
@@ -688,9 +704,14 @@ static abilu_status block_sweeps_t(abilu_factors f, const float *A32, int nsweep
             per_sm_cache.store(per_sm, std::memory_order_relaxed);
         }
         ABILU_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        const int wc = f->build_chunk ? f->build_chunk : WARP_CHUNK;
-        const int wchunks = (int)build_tickets(P.nwork, wc);
         int warps = per_sm * sms * (BUILD_THREADS / 32);
+        const int resident = warps > 0 ? warps : 1;
+        int wc = f->build_chunk ? f->build_chunk : WARP_CHUNK, sub = build_sub(wc);
+        if (!f->build_chunk && (long long)P.nwork <= (long long)SMALL_TICKET * resident) {
+            wc = (int)(((long long)P.nwork + 8LL * resident - 1) / (8LL * resident)) * 8;
+            sub = 8;
+        }
+        const int wchunks = (int)build_tickets(P.nwork, wc, sub);
         if (warps > wchunks) warps = wchunks;
         if (warps < 1) warps = 1;
         const int ctas = (warps + BUILD_THREADS / 32 - 1) / (BUILD_THREADS / 32);
@@ -710,10 +731,11 @@ static abilu_status block_sweeps_t(abilu_factors f, const float *A32, int nsweep
         }
         const int c = f->cur;
         const unsigned long long lim = spin_limit_or_default(f->spin_limit);
-        auto kern = done ? (build_sub(wc) == 64 ? k_build_blocks_async<T, true, 64>
-                                                : k_build_blocks_async<T, true, 32>)
-                         : (build_sub(wc) == 64 ? k_build_blocks_async<T, false, 64>
-                                                : k_build_blocks_async<T, false, 32>);
+        auto kern = sub == 8 ? k_build_blocks_async<T, true, 8>   // one ticket per warp: always ordered
+                    : done ? (sub == 64 ? k_build_blocks_async<T, true, 64>
+                                        : k_build_blocks_async<T, true, 32>)
+                           : (sub == 64 ? k_build_blocks_async<T, false, 64>
+                                        : k_build_blocks_async<T, false, 32>);
         launch_pdl(kern, ctas, BUILD_THREADS, 0, st,
             P, A32, L[c], U[c], D[c], Ud, nsweeps, warps, f->ctr, f->ctr + 1, f->ctr + 4, done,
             lim, wc);

@@ -91,7 +91,7 @@ struct abilu_factors_s {
     void *Udiag;
     void *A32;                 // FP32 copy of A's non-constant blocks (FP32/BF16 factors)
     void *r32;                 // FP32 copy of the apply input (FP32/BF16 factors)
-    int *chunk_done;           // per 32-block chunk: completed sweeps (ordered async builds)
+    int *chunk_done;           // per ticket (at least 8 blocks): completed sweeps (ordered async builds)
     void *Us;                  // Dinv_i U_ij for every strictly upper block (FP32
                                // factors): the matrix of the upper sweeps, formed per build
     int cur;
@@ -119,7 +119,7 @@ struct abilu_factors_s {
     // chunk's rows start from A, 0 = from the factors in place (the systems of
     // a server step: new ones from A, continuing ones warm-started)
     const int *chunk_init;
-    int build_chunk;           // work blocks per ticket of the asynchronous block build (0: 128)
+    int build_chunk;           // work blocks per ticket of the asynchronous block build (0: by size)
     void *mem;
 };
 
