@@ -84,13 +84,19 @@ __device__ __forceinline__ VT dinv_times(const T *__restrict__ D, int i, VT t) {
     return dot4(d, tv);
 }
 
+// The application's FP64 result: z = v, or z += v when `zadd` (a smoothing
+// step's x += M^-1 r, which then needs no pass of its own over x and z)
+__device__ __forceinline__ void st_result(double *z, size_t o, double v, int zadd) {
+    z[o] = zadd ? z[o] + v : v;
+}
+
 // one Jacobi lower sweep; optionally x^1 = Dinv y fused (into x1 or, when
 // it is the last upper result, into z as FP64)
 template <typename T, typename VT>
 __global__ void __launch_bounds__(APPLY_THREADS)
 k_lower_sync(PatternView P, const T *__restrict__ L, const VT *__restrict__ r,
              const VT *__restrict__ yin, VT *__restrict__ yout, const T *__restrict__ D,
-             VT *__restrict__ x1, double *__restrict__ z, Skip skip) {
+             VT *__restrict__ x1, double *__restrict__ z, int zadd, Skip skip) {
     pdl_wait();
     pdl_trigger();
     if (skip_all(skip) || skip_chunk(skip, blockIdx.x)) return;
@@ -101,7 +107,7 @@ k_lower_sync(PatternView P, const T *__restrict__ L, const VT *__restrict__ r,
     if (x1 || z) {
         VT x = dinv_times<T, VT>(D, i, s);
         if (x1) x1[(size_t)i * BS + q] = x;
-        if (z) z[(size_t)i * BS + q] = to_f64v(x);
+        if (z) st_result(z, (size_t)i * BS + q, to_f64v(x), zadd);
     }
 }
 
@@ -109,7 +115,7 @@ k_lower_sync(PatternView P, const T *__restrict__ L, const VT *__restrict__ r,
 template <typename T, typename VT>
 __global__ void __launch_bounds__(APPLY_THREADS)
 k_diag_apply(PatternView P, const T *__restrict__ D, const VT *__restrict__ y,
-             VT *__restrict__ x1, double *__restrict__ z, Skip skip) {
+             VT *__restrict__ x1, double *__restrict__ z, int zadd, Skip skip) {
     pdl_wait();
     pdl_trigger();
     if (skip_all(skip) || skip_chunk(skip, blockIdx.x)) return;
@@ -118,7 +124,7 @@ k_diag_apply(PatternView P, const T *__restrict__ D, const VT *__restrict__ y,
     VT t = y[(size_t)i * BS + q];
     VT x = dinv_times<T, VT>(D, i, t);
     if (x1) x1[(size_t)i * BS + q] = x;
-    if (z) z[(size_t)i * BS + q] = to_f64v(x);
+    if (z) st_result(z, (size_t)i * BS + q, to_f64v(x), zadd);
 }
 
 // SCALED: U holds Us = Dinv U and y holds yh = Dinv y, so x = the row sum
@@ -126,7 +132,7 @@ template <typename T, typename VT, bool SCALED>
 __global__ void __launch_bounds__(APPLY_THREADS, sweep_min_ctas<VT>())
 k_upper_sync(PatternView P, const T *__restrict__ U, const T *__restrict__ D,
              const VT *__restrict__ y, const VT *__restrict__ xin, VT *__restrict__ xout,
-             double *__restrict__ z, Skip skip) {
+             double *__restrict__ z, int zadd, Skip skip) {
     pdl_wait();
     pdl_trigger();
     if (skip_all(skip) || skip_chunk(skip, blockIdx.x)) return;
@@ -137,7 +143,7 @@ k_upper_sync(PatternView P, const T *__restrict__ U, const T *__restrict__ D,
     if constexpr (SCALED) x = s;
     else x = dinv_times<T, VT>(D, i, s);
     if (xout) xout[(size_t)i * BS + q] = x;
-    if (z) z[(size_t)i * BS + q] = to_f64v(x);
+    if (z) st_result(z, (size_t)i * BS + q, to_f64v(x), zadd);
 }
 
 // ---------------------------------------------------------------- async
@@ -157,7 +163,7 @@ template <typename T, typename VT>
 __global__ void __launch_bounds__(APPLY_THREADS, sweep_min_ctas<VT>())
 k_lower_async(PatternView P, const T *__restrict__ L, const VT *__restrict__ r, VT *y,
               int nsweeps, const T *__restrict__ D, VT *__restrict__ x1, VT *__restrict__ yh,
-              double *__restrict__ z, unsigned long long *ticket, Skip skip) {
+              double *__restrict__ z, int zadd, unsigned long long *ticket, Skip skip) {
     pdl_wait();
     pdl_trigger();
     if (skip_all(skip)) return;
@@ -182,7 +188,7 @@ k_lower_async(PatternView P, const T *__restrict__ L, const VT *__restrict__ r, 
                 const VT x = dinv_times<T, VT>(D, i, s);
                 if (x1) x1[(size_t)i * BS + q] = x;
                 if (yh) yh[(size_t)i * BS + q] = x;
-                if (z) z[(size_t)i * BS + q] = to_f64v(x);
+                if (z) st_result(z, (size_t)i * BS + q, to_f64v(x), zadd);
             }
         }
     }
@@ -195,7 +201,7 @@ template <typename T, typename VT>
 __global__ void __launch_bounds__(APPLY_THREADS)
 k_async_start(PatternView P, const T *__restrict__ D, const VT *__restrict__ r,
               VT *__restrict__ y, VT *__restrict__ x1, VT *__restrict__ yh, double *__restrict__ z,
-              unsigned long long *tickets, Skip skip) {
+              int zadd, unsigned long long *tickets, Skip skip) {
     pdl_wait();
     pdl_trigger();
     if (skip_all(skip)) return;
@@ -209,7 +215,7 @@ k_async_start(PatternView P, const T *__restrict__ D, const VT *__restrict__ r,
         const VT x = dinv_times<T, VT>(D, i, b);
         if (x1) x1[(size_t)i * BS + q] = x;
         if (yh) yh[(size_t)i * BS + q] = x;
-        if (z) z[(size_t)i * BS + q] = to_f64v(x);
+        if (z) st_result(z, (size_t)i * BS + q, to_f64v(x), zadd);
     }
 }
 
@@ -219,7 +225,7 @@ k_async_start(PatternView P, const T *__restrict__ D, const VT *__restrict__ r,
 template <typename T, typename VT, bool SCALED>
 __global__ void __launch_bounds__(APPLY_THREADS)
 k_upper_async(PatternView P, const T *__restrict__ U, const T *__restrict__ D,
-              const VT *__restrict__ y, VT *x, double *__restrict__ z, int nsweeps,
+              const VT *__restrict__ y, VT *x, double *__restrict__ z, int zadd, int nsweeps,
               unsigned long long *ticket, Skip skip) {
     pdl_wait();
     pdl_trigger();
@@ -244,7 +250,7 @@ k_upper_async(PatternView P, const T *__restrict__ U, const T *__restrict__ D,
             if constexpr (SCALED) xi = s;
             else xi = dinv_times<T, VT>(D, i, s);
             st_vol(x + (size_t)i * BS + q, xi);
-            if (last) z[(size_t)i * BS + q] = to_f64v(xi);
+            if (last) st_result(z, (size_t)i * BS + q, to_f64v(xi), zadd);
         }
     }
 }
@@ -289,7 +295,7 @@ template <bool UPPER, bool SCALED, bool SYNC, typename T>
 __global__ void __launch_bounds__(PIPE_THREADS, 7)   // 7 x 288 threads per SM: 32 registers
 k_tri_staged(PatternView P, const T *__restrict__ F, const T *__restrict__ D,
              const float *__restrict__ rhs, const float *vin, float *v, int nsweeps, int sync_last,
-             float *__restrict__ x1, float *__restrict__ yh, double *__restrict__ z,
+             float *__restrict__ x1, float *__restrict__ yh, double *__restrict__ z, int zadd,
              unsigned long long *ticket, unsigned long long *err, Skip skip,
              unsigned long long limit) {
     pdl_wait();
@@ -410,12 +416,12 @@ k_tri_staged(PatternView P, const T *__restrict__ F, const T *__restrict__ D,
             }
             if (last) {
                 if constexpr (UPPER) {
-                    if (z) z[(size_t)i * BS + q] = to_f64v(xi);
+                    if (z) st_result(z, (size_t)i * BS + q, to_f64v(xi), zadd);
                 } else if (x1 || yh || z) {
                     const float x = dinv_times<T, float>(D, i, acc);
                     if (x1) x1[(size_t)i * BS + q] = x;
                     if (yh) yh[(size_t)i * BS + q] = x;
-                    if (z) z[(size_t)i * BS + q] = to_f64v(x);
+                    if (z) st_result(z, (size_t)i * BS + q, to_f64v(x), zadd);
                 }
             }
         }
@@ -477,7 +483,7 @@ template <bool UPPER, bool SCALED, bool SYNC, typename T> static int staged_ctas
 template <typename T>
 static abilu_status apply_t(abilu_factors f, const double *r, const float *r32_in, double *z,
                             int nl, int nu, abilu_mode mode, cudaStream_t st, Skip skip,
-                            bool y_ready = false) {
+                            bool y_ready = false, int zadd = 0) {
     using VT = typename ApplyArith<T>::VT;
     const PatternView &P = f->p->v;
     const int c = f->cur;
@@ -510,6 +516,7 @@ static abilu_status apply_t(abilu_factors f, const double *r, const float *r32_i
     const T *UU = SC ? reinterpret_cast<const T *>(f->Us) : U;
     const long long n4 = (long long)P.n * BS;
     if (nl == 0 || nu == 0) {  // y = 0, or no upper update: z = x^0 = 0
+        if (zadd) return ABILU_OK;
         k_zero<double><<<counted((int)((n4 + 255) / 256)), 256, 0, st>>>(z, n4, skip);
         ABILU_LAUNCH_CHECK("apply");
         return ABILU_OK;
@@ -524,7 +531,7 @@ static abilu_status apply_t(abilu_factors f, const double *r, const float *r32_i
         if (!(y_ready && sizeof(VT) == 4 && nl >= 2)) {
             launch_pdl(k_async_start<T, VT>, grid, APPLY_THREADS, 0, st,
                 P, D, rv, y[0], nl == 1 ? x1 : nullptr, nl == 1 ? yh : nullptr, nl == 1 ? z1 : nullptr,
-                tk, skip);
+                zadd, tk, skip);
             ABILU_LAUNCH_CHECK("k_async_start");
         }
         unsigned long long *err = f->ctr + 4;
@@ -534,12 +541,12 @@ static abilu_status apply_t(abilu_factors f, const double *r, const float *r32_i
                 const int c = staged_ctas<false, false, false, T>();
                 const int g = (int)(c < nchunks ? c : nchunks);
                 launch_pdl(k_tri_staged<false, false, false, T>, g, PIPE_THREADS, 0, st,
-                    P, L, D, rv, nullptr, y[0], nl - 1, 0, x1, yh, z1, tk, err, skip, lim);
+                    P, L, D, rv, nullptr, y[0], nl - 1, 0, x1, yh, z1, zadd, tk, err, skip, lim);
             } else {
                 const int ctas_l = lower_async_ctas<T, VT>();
                 const int g = (int)(ctas_l < nchunks ? ctas_l : nchunks);
                 launch_pdl(k_lower_async<T, VT>, g, APPLY_THREADS, 0, st, P, L, rv, y[0], nl - 1, D,
-                    x1, yh, z1, tk, skip);
+                    x1, yh, z1, zadd, tk, skip);
             }
             ABILU_LAUNCH_CHECK("lower async");
         }
@@ -548,13 +555,13 @@ static abilu_status apply_t(abilu_factors f, const double *r, const float *r32_i
                 const int c = staged_ctas<true, SC, false, T>();
                 const int g = (int)(c < nchunks ? c : nchunks);
                 launch_pdl(k_tri_staged<true, SC, false, T>, g, PIPE_THREADS, 0, st,
-                    P, UU, D, SC ? y[1] : y[0], nullptr, x[0], nu - 1, 0, nullptr, nullptr, z, tk + 1,
+                    P, UU, D, SC ? y[1] : y[0], nullptr, x[0], nu - 1, 0, nullptr, nullptr, z, zadd, tk + 1,
                     err, skip, lim);
             } else {
                 const int ctas_u = upper_async_ctas<T, VT>();
                 const int g = (int)(ctas_u < nchunks ? ctas_u : nchunks);
                 launch_pdl(k_upper_async<T, VT, SC>, g, APPLY_THREADS, 0, st,
-                    P, UU, D, SC ? y[1] : y[0], x[0], z, nu - 1, tk + 1, skip);
+                    P, UU, D, SC ? y[1] : y[0], x[0], z, zadd, nu - 1, tk + 1, skip);
             }
             ABILU_LAUNCH_CHECK("upper async");
         }
@@ -570,7 +577,7 @@ static abilu_status apply_t(abilu_factors f, const double *r, const float *r32_i
     if (nl == 1) {      // no lower sweep runs: x^1 = Dinv r
         VT *x1 = nu >= 2 ? (SC ? y[0] : x[1]) : nullptr;
         launch_pdl(k_diag_apply<T, VT>, grid, APPLY_THREADS, 0, st, P, D, rv, x1,
-            nu == 1 ? z : nullptr, skip);
+            nu == 1 ? z : nullptr, zadd, skip);
         ABILU_LAUNCH_CHECK("k_diag_apply");
         yfin = SC ? y[0] : rv;
         xfirst = x1;
@@ -584,7 +591,7 @@ static abilu_status apply_t(abilu_factors f, const double *r, const float *r32_i
             // (the staged form was measured slower for this sweep: 19.3 vs 17.1 us)
             launch_pdl(k_lower_sync<T, VT>, grid, APPLY_THREADS, 0, st,
                 P, L, rv, yprev, (last && SC) ? nullptr : yout, D, last ? x1 : nullptr,
-                (last && nu == 1) ? z : nullptr, skip);
+                (last && nu == 1) ? z : nullptr, zadd, skip);
             ABILU_LAUNCH_CHECK("lower sync");
             yprev = yout;
         }
@@ -599,10 +606,10 @@ static abilu_status apply_t(abilu_factors f, const double *r, const float *r32_i
             const int g = c < grid ? c : grid;
             launch_pdl(k_tri_staged<true, SC, true, T>, g, PIPE_THREADS, 0, st,
                 P, UU, D, yfin, xin, last ? nullptr : x[s & 1], 1, last ? 1 : 0, nullptr, nullptr,
-                last ? z : nullptr, nullptr, f->ctr + 4, skip, spin_limit_or_default(f->spin_limit));
+                last ? z : nullptr, zadd, nullptr, f->ctr + 4, skip, spin_limit_or_default(f->spin_limit));
         } else {
             launch_pdl(k_upper_sync<T, VT, SC>, grid, APPLY_THREADS, 0, st,
-                P, UU, D, yfin, xin, last ? nullptr : x[s & 1], last ? z : nullptr, skip);
+                P, UU, D, yfin, xin, last ? nullptr : x[s & 1], last ? z : nullptr, zadd, skip);
         }
         ABILU_LAUNCH_CHECK("upper sync");
     }
@@ -639,6 +646,17 @@ abilu_status apply_dispatch(abilu_factors f, const double *r, const float *r32, 
     case ABILU_BF16: return apply_t<__nv_bfloat16>(f, r, r32, z, nl, nu, mode, st, skip);
     }
     return fail(ABILU_EINVAL, "apply: bad dtype");
+}
+
+// x += M^-1 r in the same launches (block factors)
+abilu_status apply_add_dispatch(abilu_factors f, const double *r, const float *r32, double *x,
+                                int nl, int nu, abilu_mode mode, cudaStream_t st, Skip skip) {
+    if (!f->scalar) switch (f->dtype) {
+    case ABILU_F64: return apply_t<double>(f, r, r32, x, nl, nu, mode, st, skip, false, 1);
+    case ABILU_F32: return apply_t<float>(f, r, r32, x, nl, nu, mode, st, skip, false, 1);
+    case ABILU_BF16: return apply_t<__nv_bfloat16>(f, r, r32, x, nl, nu, mode, st, skip, false, 1);
+    }
+    return fail(ABILU_EINVAL, "apply: block factors needed");
 }
 
 // The application when apply_y_ready(f, nl, mode) holds and the caller wrote

@@ -33,7 +33,8 @@
 //   steps.  The first step from x = 0 is x = M^{-1} b (no residual pass).
 //   Kernels: the residual (the SpMV's FMA chain, spmv.cuh; a quad per row,
 //   coalesced), the restriction (a quad per aggregate summing its cells'
-//   residuals in ascending order), the prolongation, x += z.
+//   residuals in ascending order), the prolongation; x += z happens in the
+//   application's last sweep.
 #include <string.h>
 
 #include <algorithm>
@@ -48,6 +49,8 @@ abilu_status build_dispatch(abilu_factors f, const double *A, int nsweeps, abilu
                             abilu_init init, cudaStream_t st);
 abilu_status apply_dispatch(abilu_factors f, const double *r, const float *r32, double *z,
                             int nl, int nu, abilu_mode mode, cudaStream_t st, Skip skip);
+abilu_status apply_add_dispatch(abilu_factors f, const double *r, const float *r32, double *x,
+                                int nl, int nu, abilu_mode mode, cudaStream_t st, Skip skip);
 abilu_status fgmres_run(const PatternView &P, const double *A, abilu_factors ws, const Precond &pc,
                         const double *b, double *x, const fgmres_opts *opts, fgmres_result *res,
                         cudaStream_t st, abilu_factors const *cnt, int ncnt);
@@ -74,21 +77,29 @@ k_block_norm2(const double *__restrict__ A, long long nnzb, double *__restrict__
     w[p] = s;
 }
 
-// Ac[c] = sum of A[gidx[t]], t = gptr[c] .. gptr[c+1]-1 (ascending fine
-// positions); a quad per coarse block, thread q sums row q.  Up to four fine
-// blocks are loaded before they are added (in list order), so the gathers of
-// a coarse block overlap instead of forming a chain.
+// Ac[c] = sum of A[gidx[t]], t = t0 .. t0+len-1 (ascending fine positions),
+// from the records (c, t0, len); a quad per coarse block, thread q sums row q.
+// Up to four fine blocks are loaded before they are added (in list order), so
+// the gathers of a coarse block overlap instead of forming a chain.
+//
+// The records are sorted by list length (stable, so neighbours in memory stay
+// close): an FP64 add holds this GPU's FP64 pipe for 16 cycles whatever lanes
+// are active, and with the coarse blocks in storage order the eight quads of a
+// warp waited for its one diagonal block's ten or so entries.  The first entry
+// starts the sum (one add per entry fewer).  512x512 cells x 2, finest level
+// (274 MB read, 26 M adds): 347 us in storage order, 124 sorted (level 2: 112 -> 53).
 __global__ void __launch_bounds__(MG_THREADS)
-k_galerkin(long long nnzb_c, const int *__restrict__ gptr, const int *__restrict__ gidx,
+k_galerkin(long long nnzb_c, const int4 *__restrict__ grec, const int *__restrict__ gidx,
            const double *__restrict__ A, double *__restrict__ Ac) {
     pdl_wait();
     pdl_trigger();
-    const long long c = ((long long)blockIdx.x * MG_THREADS + threadIdx.x) >> 2;
+    const long long k = ((long long)blockIdx.x * MG_THREADS + threadIdx.x) >> 2;
     const int q = threadIdx.x & 3;
-    if (c >= nnzb_c) return;
+    if (k >= nnzb_c) return;
+    const int4 rec = __ldg(grec + k);
     double s[4] = {0.0, 0.0, 0.0, 0.0};
-    const int t1 = gptr[c + 1];
-    for (int t = gptr[c]; t < t1; t += 4) {
+    const int t1 = rec.y + rec.z;
+    for (int t = rec.y; t < t1; t += 4) {
         double v[4][4];
 #pragma unroll
         for (int u = 0; u < 4; u++)
@@ -96,32 +107,44 @@ k_galerkin(long long nnzb_c, const int *__restrict__ gptr, const int *__restrict
 #pragma unroll
         for (int u = 0; u < 4; u++)
             if (t + u < t1) {
+                if (u == 0 && t == rec.y) {
 #pragma unroll
-                for (int k = 0; k < 4; k++) s[k] = __dadd_rn(s[k], v[u][k]);
+                    for (int e = 0; e < 4; e++) s[e] = v[0][e];
+                } else {
+#pragma unroll
+                    for (int e = 0; e < 4; e++) s[e] = __dadd_rn(s[e], v[u][e]);
+                }
             }
     }
-    st_row(Ac + (size_t)c * BB + q * BS, s);
+    st_row(Ac + (size_t)rec.x * BB + q * BS, s);
 }
 
-// r = b - A x, a quad per block row
+// r = b - A x, a quad per block row; into r, or rounded into r32 when only the
+// FP32 right-hand side of a smoothing step is wanted (r NULL)
 __global__ void __launch_bounds__(MG_THREADS)
 k_mg_residual(PatternView P, const double *__restrict__ A, const double *__restrict__ b,
-              const double *__restrict__ x, double *__restrict__ r, Skip skip) {
+              const double *__restrict__ x, double *__restrict__ r, float *__restrict__ r32,
+              Skip skip) {
     pdl_wait();
     pdl_trigger();
     if (skip_all(skip)) return;
     const int i = blockIdx.x * MG_ROWS + (threadIdx.x >> 2), q = threadIdx.x & 3;
     if (i >= P.n) return;
     const size_t o = (size_t)i * BS + q;
-    r[o] = b[o] - row_dot_blocks(P, A, x, i, q);
+    const double v = b[o] - row_dot_blocks(P, A, x, i, q);
+    if (r) r[o] = v;
+    else r32[o] = to_f32_int(v);
 }
 
 // Restriction bc = P^T r: bc[I] = sum over the cells i of aggregate I, in
 // ascending order, of r_i.  A quad per aggregate, thread q sums component q;
 // up to four members' entries are loaded before they are added in order.
+// b32 (NULL: none): the FP32 copy that the coarse level's first smoothing
+// step reads.
 __global__ void __launch_bounds__(MG_THREADS)
 k_mg_restrict(const double *__restrict__ r, const int *__restrict__ mptr,
-              const int *__restrict__ mem, int nc, double *__restrict__ bc, Skip skip) {
+              const int *__restrict__ mem, int nc, double *__restrict__ bc,
+              float *__restrict__ b32, Skip skip) {
     pdl_wait();
     pdl_trigger();
     if (skip_all(skip)) return;
@@ -139,6 +162,7 @@ k_mg_restrict(const double *__restrict__ r, const int *__restrict__ mptr,
             if (t + u < t1) s += v[u];
     }
     bc[(size_t)I * BS + q] = s;
+    if (b32) b32[(size_t)I * BS + q] = to_f32_int(s);
 }
 
 // x_i += x_c[agg(i)] (ASSIGN: x_i = x_c[agg(i)], x was zero)
@@ -157,21 +181,6 @@ k_mg_prolong(const int *__restrict__ agg, const double *__restrict__ xc, double 
     }
 }
 
-// x += z
-__global__ void __launch_bounds__(MG_THREADS)
-k_mg_axpy(double *__restrict__ x, const double *__restrict__ z, long long n2, Skip skip) {
-    pdl_wait();
-    pdl_trigger();
-    if (skip_all(skip)) return;
-    double2 *x2 = reinterpret_cast<double2 *>(x);
-    const double2 *z2 = reinterpret_cast<const double2 *>(z);
-    for (long long e = (long long)blockIdx.x * MG_THREADS + threadIdx.x; e < n2;
-         e += (long long)gridDim.x * MG_THREADS) {
-        const double2 a = x2[e], d = z2[e];
-        x2[e] = make_double2(a.x + d.x, a.y + d.y);
-    }
-}
-
 // ------------------------------------------------------------------ handle
 
 struct MgLevel {
@@ -184,10 +193,13 @@ struct MgLevel {
     // transfer to the next level (all NULL on the coarsest)
     int *agg = nullptr;          // [n] aggregate of each cell
     int *mptr = nullptr, *mem = nullptr;   // [nc+1], [n]: cells of each aggregate, ascending
-    int *gptr = nullptr, *gidx = nullptr;  // [nnzb_c+1], [nnzb]: fine blocks of each coarse block
+    // fine blocks of each coarse block: [nnzb_c] (coarse block, start, length),
+    // by length, and the lists [nnzb]
+    int4 *grec = nullptr;
+    int *gidx = nullptr;
     // vectors, double[n][4]: right-hand side and solution (coarse levels; level
-    // 0 uses the caller's), residual and smoother correction
-    double *b = nullptr, *x = nullptr, *r = nullptr, *z = nullptr;
+    // 0 uses the caller's), residual
+    double *b = nullptr, *x = nullptr, *r = nullptr;
 };
 
 }  // namespace abilu
@@ -265,7 +277,8 @@ static int aggregate_host(int n, const std::vector<int> &rowptr, const std::vect
 struct Coarse {
     std::vector<int> rowptr, colind;   // coarse pattern
     std::vector<int> mptr, mem;        // cells of each aggregate
-    std::vector<int> gptr, gidx;       // fine blocks summed into each coarse block
+    std::vector<int> gidx;             // fine blocks summed into each coarse block
+    std::vector<int4> grec;            // (coarse block, start in gidx, length), by length
 };
 
 static void coarse_host(int n, const std::vector<int> &rowptr, const std::vector<int> &colind,
@@ -307,12 +320,27 @@ static void coarse_host(int n, const std::vector<int> &rowptr, const std::vector
             cpos[p] = (int)(std::lower_bound(b0, b1, agg[colind[p]]) - c.colind.data());
     }
     const int nnzc = (int)c.colind.size();
-    c.gptr.assign(nnzc + 1, 0);
-    for (long long p = 0; p < nnzb; p++) c.gptr[cpos[p] + 1]++;
-    for (int k = 0; k < nnzc; k++) c.gptr[k + 1] += c.gptr[k];
+    std::vector<int> gptr(nnzc + 1, 0);
+    for (long long p = 0; p < nnzb; p++) gptr[cpos[p] + 1]++;
+    int longest = 0;
+    for (int k = 0; k < nnzc; k++) {
+        longest = std::max(longest, gptr[k + 1]);
+        gptr[k + 1] += gptr[k];
+    }
     c.gidx.resize(nnzb);
-    std::vector<int> fill(c.gptr.begin(), c.gptr.end() - 1);
-    for (long long p = 0; p < nnzb; p++) c.gidx[fill[cpos[p]]++] = (int)p;
+    {
+        std::vector<int> pos(gptr.begin(), gptr.end() - 1);
+        for (long long p = 0; p < nnzb; p++) c.gidx[pos[cpos[p]]++] = (int)p;
+    }
+    // the records of k_galerkin: a stable counting sort by list length
+    std::vector<int> at(longest + 2, 0);
+    for (int k = 0; k < nnzc; k++) at[gptr[k + 1] - gptr[k] + 1]++;
+    for (int l = 0; l <= longest; l++) at[l + 1] += at[l];
+    c.grec.resize(nnzc);
+    for (int k = 0; k < nnzc; k++) {
+        const int len = gptr[k + 1] - gptr[k];
+        c.grec[at[len]++] = make_int4(k, gptr[k], len, 0);
+    }
 }
 
 template <typename T>
@@ -330,7 +358,7 @@ static int grid_of(long long threads) { return (int)((threads + MG_THREADS - 1) 
 static abilu_status galerkin_values(abilu_mg mg, int l, cudaStream_t st) {
     MgLevel &F = mg->L[l], &Cl = mg->L[l + 1];
     if (Cl.nnzb == 0) return ABILU_OK;
-    launch_pdl(k_galerkin, grid_of(4 * Cl.nnzb), MG_THREADS, 0, st, Cl.nnzb, F.gptr, F.gidx, F.A, Cl.Ac);
+    launch_pdl(k_galerkin, grid_of(4 * Cl.nnzb), MG_THREADS, 0, st, Cl.nnzb, F.grec, F.gidx, F.A, Cl.Ac);
     ABILU_LAUNCH_CHECK("k_galerkin");
     return ABILU_OK;
 }
@@ -341,59 +369,65 @@ static abilu_status galerkin_values(abilu_mg mg, int l, cudaStream_t st) {
 
 namespace abilu {
 
+// the FP32 right-hand side of level l's smoother (NULL: FP64 factors read FP64)
+static float *level_r32(abilu_mg mg, int l) { return reinterpret_cast<float *>(mg->L[l].f->r32); }
+
 // `steps` smoothing steps x += M^{-1}(b - A x) on level l; *xzero says x is
-// (still) zero and not yet written: the first step is then x = M^{-1} b
-static abilu_status smooth(abilu_mg mg, int l, int steps, const double *b, double *x, bool *xzero,
-                           cudaStream_t st, Skip skip) {
+// (still) zero and not yet written: the first step is then x = M^{-1} b, from
+// b32, the FP32 copy of b, when a kernel before it wrote one.  The later steps'
+// residual goes straight into the FP32 right-hand side (FP32/BF16 factors) and
+// their last sweep adds into x: no conversion pass, no x += z pass.
+static abilu_status smooth(abilu_mg mg, int l, int steps, const double *b, const float *b32,
+                           double *x, bool *xzero, cudaStream_t st, Skip skip) {
     MgLevel &L = mg->L[l];
     const abilu_mg_opts &o = mg->o;
     const abilu_mode mode = (abilu_mode)o.mode;
+    float *r32 = level_r32(mg, l);
     for (int k = 0; k < steps; k++) {
         abilu_status s;
         if (*xzero) {
-            s = apply_dispatch(L.f, b, nullptr, x, o.apply_sweeps_lower, o.apply_sweeps_upper, mode,
+            s = apply_dispatch(L.f, b, b32, x, o.apply_sweeps_lower, o.apply_sweeps_upper, mode,
                                st, skip);
             if (s != ABILU_OK) return s;
             *xzero = false;
             continue;
         }
-        launch_pdl(k_mg_residual, grid_of(4LL * L.n), MG_THREADS, 0, st, L.p->v, L.A, b, x, L.r, skip);
+        launch_pdl(k_mg_residual, grid_of(4LL * L.n), MG_THREADS, 0, st, L.p->v, L.A, b, x,
+                   r32 ? nullptr : L.r, r32, skip);
         ABILU_LAUNCH_CHECK("k_mg_residual");
-        s = apply_dispatch(L.f, L.r, nullptr, L.z, o.apply_sweeps_lower, o.apply_sweeps_upper, mode,
-                           st, skip);
+        s = apply_add_dispatch(L.f, L.r, r32, x, o.apply_sweeps_lower, o.apply_sweeps_upper, mode,
+                               st, skip);
         if (s != ABILU_OK) return s;
-        const long long n2 = 2LL * L.n;
-        launch_pdl(k_mg_axpy, grid_of(n2), MG_THREADS, 0, st, x, L.z, n2, skip);
-        ABILU_LAUNCH_CHECK("k_mg_axpy");
     }
     return ABILU_OK;
 }
 
-// x = the V-cycle from level l applied to b
-static abilu_status vcycle(abilu_mg mg, int l, const double *b, double *x, cudaStream_t st,
-                           Skip skip) {
+// x = the V-cycle from level l applied to b (b32: its FP32 copy or NULL)
+static abilu_status vcycle(abilu_mg mg, int l, const double *b, const float *b32, double *x,
+                           cudaStream_t st, Skip skip) {
     MgLevel &L = mg->L[l];
     const abilu_mg_opts &o = mg->o;
     bool xzero = true;
     abilu_status s;
     if (l == mg->nlevels - 1) {
-        s = smooth(mg, l, o.coarse_smooth, b, x, &xzero, st, skip);
+        s = smooth(mg, l, o.coarse_smooth, b, b32, x, &xzero, st, skip);
         if (s == ABILU_OK && xzero)
             ABILU_CUDA(cudaMemsetAsync(x, 0, sizeof(double) * 4 * (size_t)L.n, st));
         return s;
     }
     MgLevel &Cl = mg->L[l + 1];
-    if ((s = smooth(mg, l, o.pre_smooth, b, x, &xzero, st, skip)) != ABILU_OK) return s;
+    if ((s = smooth(mg, l, o.pre_smooth, b, b32, x, &xzero, st, skip)) != ABILU_OK) return s;
     const double *rf = b;   // the fine residual: b itself while x = 0
     if (!xzero) {
-        launch_pdl(k_mg_residual, grid_of(4LL * L.n), MG_THREADS, 0, st, L.p->v, L.A, b, x, L.r, skip);
+        launch_pdl(k_mg_residual, grid_of(4LL * L.n), MG_THREADS, 0, st, L.p->v, L.A, b, x, L.r,
+                   nullptr, skip);
         ABILU_LAUNCH_CHECK("k_mg_residual");
         rf = L.r;
     }
     launch_pdl(k_mg_restrict, grid_of(4LL * Cl.n), MG_THREADS, 0, st, rf, L.mptr, L.mem, Cl.n, Cl.b,
-        skip);
+        level_r32(mg, l + 1), skip);
     ABILU_LAUNCH_CHECK("k_mg_restrict");
-    if ((s = vcycle(mg, l + 1, Cl.b, Cl.x, st, skip)) != ABILU_OK) return s;
+    if ((s = vcycle(mg, l + 1, Cl.b, level_r32(mg, l + 1), Cl.x, st, skip)) != ABILU_OK) return s;
     const long long n4 = 4LL * L.n;
     if (xzero)
         launch_pdl(k_mg_prolong<true>, grid_of(n4), MG_THREADS, 0, st, L.agg, Cl.x, x, n4, skip);
@@ -401,13 +435,13 @@ static abilu_status vcycle(abilu_mg mg, int l, const double *b, double *x, cudaS
         launch_pdl(k_mg_prolong<false>, grid_of(n4), MG_THREADS, 0, st, L.agg, Cl.x, x, n4, skip);
     ABILU_LAUNCH_CHECK("k_mg_prolong");
     xzero = false;
-    return smooth(mg, l, o.post_smooth, b, x, &xzero, st, skip);
+    return smooth(mg, l, o.post_smooth, b, nullptr, x, &xzero, st, skip);
 }
 
-static abilu_status mg_pc(void *ctx, const double *v, const float *, double *z, cudaStream_t st,
+static abilu_status mg_pc(void *ctx, const double *v, const float *v32, double *z, cudaStream_t st,
                           Skip skip) {
     abilu_mg mg = static_cast<abilu_mg>(ctx);
-    return vcycle(mg, 0, v, z, st, skip);
+    return vcycle(mg, 0, v, v32, z, st, skip);
 }
 
 static abilu_status mg_setup(abilu_mg mg, const double *A, cudaStream_t st) {
@@ -457,7 +491,7 @@ static abilu_status mg_build_hierarchy(abilu_mg mg, abilu_pattern p, const doubl
         if ((s = upload(mg, &F.agg, agg, st)) != ABILU_OK) return s;
         if ((s = upload(mg, &F.mptr, c.mptr, st)) != ABILU_OK) return s;
         if ((s = upload(mg, &F.mem, c.mem, st)) != ABILU_OK) return s;
-        if ((s = upload(mg, &F.gptr, c.gptr, st)) != ABILU_OK) return s;
+        if ((s = upload(mg, &F.grec, c.grec, st)) != ABILU_OK) return s;
         if ((s = upload(mg, &F.gidx, c.gidx, st)) != ABILU_OK) return s;
         int *rpd = nullptr, *cid = nullptr;
         if ((s = upload(mg, &rpd, c.rowptr, st)) != ABILU_OK) return s;
@@ -479,7 +513,6 @@ static abilu_status mg_build_hierarchy(abilu_mg mg, abilu_pattern p, const doubl
         if ((s = abilu_factors_create(L.p, (abilu_dtype)o.factor_dtype, &L.f)) != ABILU_OK) return s;
         const size_t nv = 4 * (size_t)L.n;
         if ((s = mg_alloc(mg, &L.r, nv)) != ABILU_OK) return s;
-        if ((s = mg_alloc(mg, &L.z, nv)) != ABILU_OK) return s;
         if (l > 0) {
             if ((s = mg_alloc(mg, &L.b, nv)) != ABILU_OK) return s;
             if ((s = mg_alloc(mg, &L.x, nv)) != ABILU_OK) return s;
@@ -547,7 +580,7 @@ extern "C" abilu_status abilu_mg_apply(abilu_mg mg, const double *r, double *z, 
     if (r == z) return fail(ABILU_EINVAL, "abilu_mg_apply: r and z must be distinct");
     if (!aligned16(r) || !aligned16(z))
         return fail(ABILU_EINVAL, "abilu_mg_apply: vectors must be 16-byte aligned");
-    return vcycle(mg, 0, r, z, S(stream), Skip{});
+    return vcycle(mg, 0, r, nullptr, z, S(stream), Skip{});
 }
 
 extern "C" abilu_status abilu_mg_levels(abilu_mg mg, int64_t *out) {
@@ -602,7 +635,7 @@ extern "C" abilu_status fgmres_solve_mg(abilu_mg mg, const double *A, const doub
         cnt[l]->spin_limit = (unsigned long long)opts->spin_limit;
     }
     if (!opts->build || (s = mg_setup(mg, A, st)) == ABILU_OK) {
-        const Precond pc{mg_pc, mg, nullptr};
+        const Precond pc{mg_pc, mg, level_r32(mg, 0)};
         s = fgmres_run(mg->L[0].p->v, A, mg->L[0].f, pc, b, x, opts, res, st, cnt, mg->nlevels);
     }
     for (int l = 0; l < mg->nlevels; l++) cnt[l]->spin_limit = keep[l];
