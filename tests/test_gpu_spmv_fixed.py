@@ -1,0 +1,103 @@
+"""The FP64 block product's integer sums (third and fourth block of a row)."""
+from fractions import Fraction
+
+import numpy as np
+import pytest
+
+
+def _system(blocks, seed, fill):
+    """Rows of 1 .. `blocks` blocks; `fill(rng, n)` draws n values."""
+    rng = np.random.default_rng(seed)
+    n = 40
+    rows = []
+    for i in range(n):
+        others = [j for j in range(n) if j != i]
+        rng.shuffle(others)
+        rows.append(sorted([i] + others[:i % blocks]))
+    rowptr = np.cumsum([0] + [len(r) for r in rows]).astype(np.int32)
+    colind = np.concatenate(rows).astype(np.int32)
+    A = fill(rng, rowptr[-1] * 16).reshape(-1, 4, 4)
+    return rowptr, colind, A, fill(rng, n * 4).reshape(n, 4)
+
+
+def _run(rowptr, colind, A, x):
+    import torch
+    import paper_1912_00539_gb300.abilu as ab
+    pat = ab.Pattern(torch.from_numpy(rowptr).cuda(), torch.from_numpy(colind).cuda())
+    y = torch.empty(x.shape, dtype=torch.float64, device="cuda")
+    ab.bsr_spmv(pat, torch.from_numpy(A).cuda(), torch.from_numpy(x).cuda(), y)
+    return y.cpu().numpy()
+
+
+def _normal(rng, n):
+    return rng.standard_normal(n)
+
+
+def _wide(rng, n):
+    return np.ldexp(rng.standard_normal(n), rng.integers(-300, 300, n))
+
+
+def _tiny(rng, n):   # every product below the integer range, many subnormal
+    return np.ldexp(rng.standard_normal(n), rng.integers(-560, -480, n))
+
+
+def _huge(rng, n):   # operands above the integer range
+    return np.ldexp(rng.standard_normal(n), rng.integers(478, 505, n))
+
+
+def _zeros(rng, n):
+    v = rng.standard_normal(n) * (rng.random(n) < 0.4)
+    v[rng.random(n) < 0.1] = -0.0
+    v[rng.random(n) < 0.1] = 5e-324
+    return v
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("fill", [_normal, _wide, _tiny, _huge, _zeros])
+@pytest.mark.parametrize("blocks", [1, 2, 3, 4, 7])
+def test_product_against_exact_sums(blocks, fill):
+    """Each entry within k u (sum |a x|) of the exact sum, k the number of
+    products (u = 2^-53): the bound of a sum of FMAs, which the integer part
+    (3 x 8 units of 2^-58 of the largest product, one rounding) keeps; products
+    below the normal range add half a subnormal unit each."""
+    rowptr, colind, A, x = _system(blocks, 3 * blocks, fill)
+    y = _run(rowptr, colind, A, x)
+    for i in range(x.shape[0]):
+        for q in range(4):
+            s, m, k = Fraction(0), Fraction(0), 0
+            for p in range(rowptr[i], rowptr[i + 1]):
+                for c in range(4):
+                    t = Fraction(float(A[p, q, c])) * Fraction(float(x[colind[p], c]))
+                    s, m, k = s + t, m + abs(t), k + 1
+            err = abs(Fraction(float(y[i, q])) - s)
+            assert err <= k * m / 2**53 + k * Fraction(5e-324), (i, q)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("bad", [np.inf, -np.inf, np.nan])
+def test_infinities_and_nans_pass_through(bad):
+    rowptr, colind, A, x = _system(4, 1, _normal)
+    x[7, 2] = bad
+    x[9, 1] = 0.0
+    p = rowptr[11] + 3
+    A[p, 1, 1] = bad
+    y = _run(rowptr, colind, A, x)
+    want = np.zeros_like(y)
+    with np.errstate(invalid="ignore"):
+        for i in range(x.shape[0]):
+            for q in range(rowptr[i], rowptr[i + 1]):
+                want[i] += A[q] @ x[colind[q]]
+    assert np.array_equal(np.isfinite(y), np.isfinite(want))
+    assert np.array_equal(np.isnan(y), np.isnan(want))
+    inf = np.isinf(want)
+    assert np.array_equal(y[inf], want[inf])
+
+
+@pytest.mark.gpu
+def test_integers_are_exact():
+    rowptr, colind, A, x = _system(5, 2, lambda r, n: r.integers(-2**20, 2**20, n).astype(np.float64))
+    y = _run(rowptr, colind, A, x)
+    for i in range(x.shape[0]):
+        for q in range(4):
+            s = sum(int(A[p, q, c]) * int(x[colind[p], c]) for p in range(rowptr[i], rowptr[i + 1]) for c in range(4))
+            assert y[i, q] == float(s)
