@@ -74,6 +74,46 @@ __device__ __forceinline__ VT row_sweep_sum(VT s, const T *__restrict__ F,
     return s;
 }
 
+// The FP64 form: one FMA per entry into the running sum (five operations per
+// block as a separate dot product and subtraction, on the pipe that bounds these
+// sweeps).
+template <bool VOL>
+__device__ __forceinline__ double row_sweep_sum(double s, const double *__restrict__ F,
+                                                const int32_t *__restrict__ col, int l0, int l1,
+                                                const double *v) {
+    const int q = threadIdx.x & 3;
+    for (int l = l0; l < l1; l++) {
+        double a[4], b[4];
+        ld_row(F + (size_t)l * BB + q * BS, a);
+        ld_row_sel<VOL>(v + (size_t)col[l] * BS, b);
+#pragma unroll
+        for (int c = 0; c < 4; c++) s = fma(-a[c], b[c], s);
+    }
+    return s;
+}
+
+// The row of this quad among the 64 rows from row0 (n or more: none) and its
+// blocks l0 .. l1-1: in order, or for FP64 by decreasing block count
+// (row_by_work).  512x512, one sweep (us): lower 63 -> 37, upper 73 -> 52 (upper with its Dinv product).
+template <typename VT>
+__device__ __forceinline__ int sweep_row(const int32_t *__restrict__ ptr, int row0, int n, int &l0, int &l1) {
+    if constexpr (sizeof(VT) == 8) {
+        __shared__ unsigned char sh[APPLY_THREADS];
+        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        const int base = row0 + (warp >> 2) * 32, r = base + lane;
+        const int a = r < n ? ptr[r] : 0, b = r < n ? ptr[r + 1] : 0;
+        const int off = row_by_work(b - a, sh + warp * 32);
+        l0 = __shfl_sync(0xffffffffu, a, off);
+        l1 = __shfl_sync(0xffffffffu, b, off);
+        return base + off;
+    } else {
+        const int i = row0 + (threadIdx.x >> 2);
+        l0 = i < n ? ptr[i] : 0;
+        l1 = i < n ? ptr[i + 1] : 0;
+        return i;
+    }
+}
+
 // x_i = Dinv_i t_i where thread q holds t_i[q]; returns x_i[q]
 template <typename T, typename VT>
 __device__ __forceinline__ VT dinv_times(const T *__restrict__ D, int i, VT t) {
@@ -100,9 +140,11 @@ k_lower_sync(PatternView P, const T *__restrict__ L, const VT *__restrict__ r,
     pdl_wait();
     pdl_trigger();
     if (skip_all(skip) || skip_chunk(skip, blockIdx.x)) return;
-    const int i = blockIdx.x * APPLY_ROWS + (threadIdx.x >> 2), q = threadIdx.x & 3;
+    const int q = threadIdx.x & 3;
+    int l0, l1;
+    const int i = sweep_row<VT>(P.lrow, blockIdx.x * APPLY_ROWS, P.n, l0, l1);
     if (i >= P.n) return;
-    const VT s = row_sweep_sum<false>(r[(size_t)i * BS + q], L, P.lcol, P.lrow[i], P.lrow[i + 1], yin);
+    const VT s = row_sweep_sum<false>(r[(size_t)i * BS + q], L, P.lcol, l0, l1, yin);
     if (yout) yout[(size_t)i * BS + q] = s;
     if (x1 || z) {
         VT x = dinv_times<T, VT>(D, i, s);
@@ -136,9 +178,11 @@ k_upper_sync(PatternView P, const T *__restrict__ U, const T *__restrict__ D,
     pdl_wait();
     pdl_trigger();
     if (skip_all(skip) || skip_chunk(skip, blockIdx.x)) return;
-    const int i = blockIdx.x * APPLY_ROWS + (threadIdx.x >> 2), q = threadIdx.x & 3;
+    const int q = threadIdx.x & 3;
+    int l0, l1;
+    const int i = sweep_row<VT>(P.urow, blockIdx.x * APPLY_ROWS, P.n, l0, l1);
     if (i >= P.n) return;
-    const VT s = row_sweep_sum<false>(y[(size_t)i * BS + q], U, P.ucol, P.urow[i], P.urow[i + 1], xin);
+    const VT s = row_sweep_sum<false>(y[(size_t)i * BS + q], U, P.ucol, l0, l1, xin);
     VT x;
     if constexpr (SCALED) x = s;
     else x = dinv_times<T, VT>(D, i, s);
@@ -179,10 +223,10 @@ k_lower_async(PatternView P, const T *__restrict__ L, const VT *__restrict__ r, 
         if (t >= total) break;
         const bool last = t / nchunks == nsweeps - 1;
         const int chunk = (int)(t % nchunks);
-        const int i = chunk * APPLY_ROWS + (threadIdx.x >> 2);
+        int l0, l1;
+        const int i = sweep_row<VT>(P.lrow, chunk * APPLY_ROWS, P.n, l0, l1);
         if (i < P.n && !skip_chunk(skip, chunk)) {  // quads of a row stay together
-            const VT s = row_sweep_sum<true>(r[(size_t)i * BS + q], L, P.lcol, P.lrow[i],
-                                             P.lrow[i + 1], (const VT *)y);
+            const VT s = row_sweep_sum<true>(r[(size_t)i * BS + q], L, P.lcol, l0, l1, (const VT *)y);
             st_vol(y + (size_t)i * BS + q, s);
             if (last && (x1 || z)) {
                 const VT x = dinv_times<T, VT>(D, i, s);
@@ -242,10 +286,10 @@ k_upper_async(PatternView P, const T *__restrict__ U, const T *__restrict__ D,
         if (t >= total) break;
         const bool last = t / nchunks == nsweeps - 1;
         const int chunk = (int)(nchunks - 1 - t % nchunks);
-        const int i = chunk * APPLY_ROWS + (threadIdx.x >> 2);
+        int l0, l1;
+        const int i = sweep_row<VT>(P.urow, chunk * APPLY_ROWS, P.n, l0, l1);
         if (i < P.n && !skip_chunk(skip, chunk)) {  // quads of a row stay together
-            const VT s = row_sweep_sum<true>(y[(size_t)i * BS + q], U, P.ucol, P.urow[i],
-                                             P.urow[i + 1], (const VT *)x);
+            const VT s = row_sweep_sum<true>(y[(size_t)i * BS + q], U, P.ucol, l0, l1, (const VT *)x);
             VT xi;
             if constexpr (SCALED) xi = s;
             else xi = dinv_times<T, VT>(D, i, s);

@@ -7,11 +7,11 @@
 // work item, Sec. 3.3), blocks of the row in ascending column order with a
 // local accumulator and one write per block.
 //
-// Thread mapping: 4 threads ("a quad") per block row; thread q of the quad
+// Thread mapping: 4 threads ("a quad") per block; thread q of the quad
 // owns row q of every 4x4 block, so a block is read with four 16/32-byte row
 // loads that are contiguous across the quad (fully used sectors), and the 4x4
-// products exchange rows through quad shuffles.  The inversion of U_ii is done
-// by one thread per block out of shared memory (FP64 adjugate), because FP64
+// products exchange rows through quad shuffles.  The FP64 inversion of U_ii
+// is done by one thread per block out of shared memory (adjugate), because FP64
 // throughput is scarce on this GPU: no FP64 work is duplicated across lanes.
 //
 // Precision: A is FP64.  In FP64 factor mode everything is FP64.  In FP32/BF16
@@ -207,83 +207,30 @@ __device__ __forceinline__ void st_row_sel(T *p, const C v[4]) {
     }
 }
 
-// One block row i handled by one quad.  Writes the row's L and U blocks and
-// returns row q of U_ii in udiag.
-template <typename T, bool VOL, typename AT>
-__device__ __forceinline__ void build_row_products(const PatternView &P, int i,
-                                                   const AT *__restrict__ A, const T *Lin,
-                                                   const T *Uin, const T *Din, T *Lout, T *Uout,
-                                                   typename BuildArith<T>::C udiag[4]) {
-    using C = typename BuildArith<T>::C;
-    const int q = threadIdx.x & 3;
-    const int p0 = P.rowptr[i], p1 = P.rowptr[i + 1], dp = P.diagpos[i];
-    const int lb = P.lrow[i], ub = P.urow[i];
-    for (int p = p0; p < p1; p++) {
-        const int t0 = P.pair_ptr[p], t1 = P.pair_ptr[p + 1];
-        // U_ij with no product pair equals A_ij in every sweep: written once
-        // per build by k_build_prepare into every buffer, skipped here
-        if (p > dp && t0 == t1) continue;
-        const int j = P.colind[p];
-        C s[4];
-        ld_row(A + (size_t)p * BB + q * BS, s);
-        for (int t = t0; t < t1; t++) {
-            const int2 pr = P.pairs[t];
-            C l[4], u[4];
-            ld_row_sel<VOL>(Lin + (size_t)pr.x * BB + q * BS, l);  // row q of L_ik
-            ld_row_sel<VOL>(Uin + (size_t)pr.y * BB + q * BS, u);  // row q of U_kj
-            C acc[4] = {0, 0, 0, 0};
-#pragma unroll
-            for (int k = 0; k < 4; k++)
-#pragma unroll
-                for (int c = 0; c < 4; c++) acc[c] += l[k] * qshfl(u[c], k);
-#pragma unroll
-            for (int c = 0; c < 4; c++) s[c] -= acc[c];
-        }
-        if (j < i) {  // L_ij = S Dinv_j
-            C d[4];
-            ld_row_sel<VOL>(Din + (size_t)j * BB + q * BS, d);
-            C o[4];
-#pragma unroll
-            for (int c = 0; c < 4; c++) {
-                // o[c] = sum_k s[k] * Dinv_j[k][c]; row k of Dinv_j lives in thread k
-                C d0 = qshfl(d[c], 0), d1 = qshfl(d[c], 1), d2 = qshfl(d[c], 2), d3 = qshfl(d[c], 3);
-                o[c] = s[0] * d0 + s[1] * d1 + s[2] * d2 + s[3] * d3;
-            }
-            st_row_sel<VOL>(Lout + (size_t)(lb + (p - p0)) * BB + q * BS, o);
-        } else if (j == i) {
-            udiag[0] = s[0]; udiag[1] = s[1]; udiag[2] = s[2]; udiag[3] = s[3];
-        } else {
-            st_row_sel<VOL>(Uout + (size_t)(ub + (p - dp - 1)) * BB + q * BS, s);
-        }
-    }
-}
-
-// Inversion phase: one thread per row of the CTA inverts its U_ii from shared
-// memory and writes Dinv_i (and U_ii if requested) with coalesced row stores
-// done by the quads afterwards.
+// Inversion phase: one thread per row of the CTA inverts its U_ii in shared
+// memory (blocks INV_LD entries apart: an odd count, so the threads of a warp
+// read distinct banks), then the quads write Dinv_i with coalesced row stores.
+// Every thread of the CTA calls it.
+constexpr int INV_LD = BB + 1;
 template <typename T, bool VOL>
-__device__ __forceinline__ void build_cta_invert(int row0, int n, T *Dout, T *Udiag,
-                                                 double *sh_u, double *sh_d,
+__device__ __forceinline__ void build_cta_invert(int row0, int n, T *Dout, double *sh_u,
                                                  unsigned long long *nsing) {
     __syncthreads();
     const int r = threadIdx.x;
     if (r < BUILD_ROWS && row0 + r < n) {
         double a[16], inv[16];
 #pragma unroll
-        for (int k = 0; k < 16; k++) a[k] = sh_u[r * BB + k];
+        for (int k = 0; k < 16; k++) a[k] = sh_u[r * INV_LD + k];
         if (inv4_adj(a, inv)) atomicAdd(nsing, 1ull);
 #pragma unroll
-        for (int k = 0; k < 16; k++) sh_d[r * BB + k] = inv[k];
+        for (int k = 0; k < 16; k++) sh_u[r * INV_LD + k] = inv[k];
     }
     __syncthreads();
     const int i = row0 + (threadIdx.x >> 2), q = threadIdx.x & 3;
     if (i < n) {
-        const double *d = sh_d + (threadIdx.x >> 2) * BB + q * BS;
-        st_row_sel<VOL>(Dout + (size_t)i * BB + q * BS, d);
-        if (Udiag) {
-            const double *u = sh_u + (threadIdx.x >> 2) * BB + q * BS;
-            st_row_sel<false>(Udiag + (size_t)i * BB + q * BS, u);
-        }
+        const double *d = sh_u + (threadIdx.x >> 2) * INV_LD + q * BS;
+        const double v[4] = {d[0], d[1], d[2], d[3]};
+        st_row_sel<VOL>(Dout + (size_t)i * BB + q * BS, v);
     }
 }
 
@@ -291,8 +238,8 @@ __device__ __forceinline__ void build_cta_invert(int row0, int n, T *Dout, T *Ud
 // U_ii held by thread q of each row's quad.  Every thread of the CTA calls it.
 template <typename T, bool VOL>
 __device__ __forceinline__ void build_finish_rows(int row0, int n, const typename BuildArith<T>::C u[4],
-                                                  T *Dout, T *Udiag, double *sh_u, double *sh_d,
-                                                  float *sh_q, unsigned long long *nsing) {
+                                                  T *Dout, T *Udiag, double *sh_u, float *sh_q,
+                                                  unsigned long long *nsing) {
     const int i = row0 + (threadIdx.x >> 2), q = threadIdx.x & 3;
     if constexpr (sizeof(T) < 8) {
         if (i < n) {
@@ -307,16 +254,17 @@ __device__ __forceinline__ void build_finish_rows(int row0, int n, const typenam
         }
     } else {
         if (i < n) {
-            double *su = sh_u + (threadIdx.x >> 2) * BB + q * BS;
+            double *su = sh_u + (threadIdx.x >> 2) * INV_LD + q * BS;
             su[0] = u[0]; su[1] = u[1]; su[2] = u[2]; su[3] = u[3];
+            if (Udiag) st_row_sel<false>(Udiag + (size_t)i * BB + q * BS, u);
         }
-        build_cta_invert<T, VOL>(row0, n, Dout, Udiag, sh_u, sh_d, nsing);
+        build_cta_invert<T, VOL>(row0, n, Dout, sh_u, nsing);
     }
 }
 
 // shared memory of the build kernels: FP64 inversion scratch or FP32 quad scratch
 template <typename T> struct BuildShared {
-    static constexpr int D = sizeof(T) == 8 ? BUILD_ROWS * BB : 1;
+    static constexpr int D = sizeof(T) == 8 ? BUILD_ROWS * INV_LD : 1;
     static constexpr int F = sizeof(T) == 8 ? 1 : BUILD_ROWS * QUAD_SCRATCH;
 };
 
@@ -515,35 +463,137 @@ k_build_blocks_async(PatternView P, const float *__restrict__ A32, T *L, T *U, T
     }
 }
 
-template <typename T, typename AT>
-__global__ void __launch_bounds__(BUILD_THREADS)
-k_build_sync(PatternView P, const AT *__restrict__ A, const T *__restrict__ Lin,
-             const T *__restrict__ Uin, const T *__restrict__ Din, T *__restrict__ Lout,
-             T *__restrict__ Uout, T *__restrict__ Dout, T *__restrict__ Udiag,
-             unsigned long long *nsing) {
+// ---- FP64 factors: 64 rows per CTA
+// The FP64 pipe bounds these sweeps (16 cycles per warp-wide instruction
+// whatever lanes are active), so every quad of a warp gets the same work: the
+// rows' L blocks as one list (they are contiguous in the compact array; the
+// row of each by a search in shared memory), then the diagonal blocks of each
+// 32 rows by decreasing number of product pairs (row_by_work), then the U blocks
+// with pairs, again as one list, and the inverses one thread per row.  A quad
+// per block row, its blocks in turn, ran the L update, the diagonal update and
+// each pair count of its eight rows one after the other.  Products subtract by
+// FMA from the block itself.  512x512, one sweep: 473 -> 351 us (the FP64
+// instructions alone: about 300).
+//
+// VOL (in place, Algorithm 4 with blocks): reads are volatile, and a barrier
+// puts the rows' new L blocks before their diagonal and U updates.
+struct F64Rows {
+    double u[BUILD_ROWS * INV_LD];      // U_ii, then Dinv_i
+    int lr[BUILD_ROWS + 1], ur[BUILD_ROWS + 1];
+    unsigned char ord[BUILD_THREADS];
+};
+
+// the row r of the CTA's rows whose list range ptr[r] .. ptr[r+1]-1 holds t
+__device__ __forceinline__ int list_row(const int *ptr, int rows, int t) {
+    int a = 0, b = rows;
+    while (b - a > 1) {
+        const int h = (a + b) >> 1;
+        if (ptr[h] <= t) a = h; else b = h;
+    }
+    return a;
+}
+
+// s -= sum over product pairs t0 .. t1-1 of L_ik U_kj (row q of the block)
+template <bool VOL>
+__device__ __forceinline__ void sub_pairs_f64(const PatternView &P, int t0, int t1, const double *Lin,
+                                              const double *Uin, double s[4]) {
+    const int q = threadIdx.x & 3;
+    for (int t = t0; t < t1; t++) {
+        const int2 pr = P.pairs[t];
+        double l[4], u[4];
+        ld_row_sel<VOL>(Lin + (size_t)pr.x * BB + q * BS, l);  // row q of L_ik
+        ld_row_sel<VOL>(Uin + (size_t)pr.y * BB + q * BS, u);  // row q of U_kj
+#pragma unroll
+        for (int k = 0; k < 4; k++)
+#pragma unroll
+            for (int c = 0; c < 4; c++) s[c] = fma(-l[k], qshfl(u[c], k), s[c]);
+    }
+}
+
+template <bool VOL>
+__device__ __forceinline__ void build_rows_f64(const PatternView &P, int row0,
+                                               const double *__restrict__ A, const double *Lin,
+                                               const double *Uin, const double *Din, double *Lout,
+                                               double *Uout, double *Dout, double *Udiag,
+                                               F64Rows &sh, unsigned long long *nsing) {
+    const int q = threadIdx.x & 3, quad = threadIdx.x >> 2;
+    const int rows = min(BUILD_ROWS, P.n - row0);
+    if (threadIdx.x <= rows) {
+        sh.lr[threadIdx.x] = P.lrow[row0 + threadIdx.x];
+        sh.ur[threadIdx.x] = P.urow[row0 + threadIdx.x];
+    }
+    __syncthreads();
+    for (int t = sh.lr[0] + quad; t < sh.lr[rows]; t += BUILD_ROWS) {   // L_ij = S Dinv_j
+        const int r = list_row(sh.lr, rows, t);
+        const int p = P.rowptr[row0 + r] + (t - sh.lr[r]);
+        double s[4], d[4], o[4];
+        ld_row_sel<VOL>(Din + (size_t)P.lcol[t] * BB + q * BS, d);
+        ld_row(A + (size_t)p * BB + q * BS, s);
+        sub_pairs_f64<VOL>(P, P.pair_ptr[p], P.pair_ptr[p + 1], Lin, Uin, s);
+#pragma unroll
+        for (int c = 0; c < 4; c++) {   // row k of Dinv_j lives in thread k
+            const double d0 = qshfl(d[c], 0), d1 = qshfl(d[c], 1), d2 = qshfl(d[c], 2), d3 = qshfl(d[c], 3);
+            o[c] = s[0] * d0 + s[1] * d1 + s[2] * d2 + s[3] * d3;
+        }
+        st_row_sel<VOL>(Lout + (size_t)t * BB + q * BS, o);
+    }
+    if constexpr (VOL) __syncthreads();
+    {   // U_ii = S
+        const int lane = threadIdx.x & 31, base = row0 + (threadIdx.x >> 7) * 32, mine = base + lane;
+        int dp = 0, t0 = 0, t1 = 0;
+        if (mine < P.n) {
+            dp = P.diagpos[mine];
+            t0 = P.pair_ptr[dp];
+            t1 = P.pair_ptr[dp + 1];
+        }
+        const int off = row_by_work(t1 - t0, sh.ord + (threadIdx.x & ~31));
+        dp = __shfl_sync(0xffffffffu, dp, off);
+        t0 = __shfl_sync(0xffffffffu, t0, off);
+        t1 = __shfl_sync(0xffffffffu, t1, off);
+        const int i = base + off;
+        if (i < P.n) {
+            double s[4];
+            ld_row(A + (size_t)dp * BB + q * BS, s);
+            sub_pairs_f64<VOL>(P, t0, t1, Lin, Uin, s);
+            double *su = sh.u + (i - row0) * INV_LD + q * BS;
+            su[0] = s[0]; su[1] = s[1]; su[2] = s[2]; su[3] = s[3];
+            if (Udiag) st_row(Udiag + (size_t)i * BB + q * BS, s);
+        }
+    }
+    // U_ij with no product pair equals A_ij in every sweep: written once per
+    // build by k_build_prepare into every buffer, not touched here
+    for (int t = sh.ur[0] + quad; t < sh.ur[rows]; t += BUILD_ROWS) {
+        const int r = list_row(sh.ur, rows, t);
+        const int p = P.diagpos[row0 + r] + 1 + (t - sh.ur[r]);
+        const int t0 = P.pair_ptr[p], t1 = P.pair_ptr[p + 1];
+        if (t0 == t1) continue;
+        double s[4];
+        ld_row(A + (size_t)p * BB + q * BS, s);
+        sub_pairs_f64<VOL>(P, t0, t1, Lin, Uin, s);
+        st_row_sel<VOL>(Uout + (size_t)t * BB + q * BS, s);
+    }
+    build_cta_invert<double, VOL>(row0, P.n, Dout, sh.u, nsing);
+}
+
+__global__ void __launch_bounds__(BUILD_THREADS, 4)
+k_build_sync(PatternView P, const double *__restrict__ A, const double *__restrict__ Lin,
+             const double *__restrict__ Uin, const double *__restrict__ Din,
+             double *__restrict__ Lout, double *__restrict__ Uout, double *__restrict__ Dout,
+             double *__restrict__ Udiag, unsigned long long *nsing) {
     pdl_wait();
     pdl_trigger();
-    __shared__ double sh_u[BuildShared<T>::D];
-    __shared__ double sh_d[BuildShared<T>::D];
-    __shared__ __align__(16) float sh_q[BuildShared<T>::F];
-    const int row0 = blockIdx.x * BUILD_ROWS;
-    const int i = row0 + (threadIdx.x >> 2);
-    typename BuildArith<T>::C u[4] = {0, 0, 0, 0};
-    if (i < P.n) build_row_products<T, false>(P, i, A, Lin, Uin, Din, Lout, Uout, u);
-    build_finish_rows<T, false>(row0, P.n, u, Dout, Udiag, sh_u, sh_d, sh_q, nsing);
+    __shared__ F64Rows sh;
+    build_rows_f64<false>(P, blockIdx.x * BUILD_ROWS, A, Lin, Uin, Din, Lout, Uout, Dout, Udiag, sh, nsing);
 }
 
 // Persistent in-place kernel: tickets t = 0 .. nsweeps*nchunks-1 taken in
 // order from ctr; ticket t is chunk (t mod nchunks) in sweep (t / nchunks).
-template <typename T, typename AT>
-__global__ void __launch_bounds__(BUILD_THREADS)
-k_build_async(PatternView P, const AT *__restrict__ A, T *L, T *U, T *D, T *Udiag,
-              int nsweeps, unsigned long long *nsing, unsigned long long *ticket) {
+__global__ void __launch_bounds__(BUILD_THREADS, 4)
+k_build_async(PatternView P, const double *__restrict__ A, double *L, double *U, double *D,
+              double *Udiag, int nsweeps, unsigned long long *nsing, unsigned long long *ticket) {
     pdl_wait();
     pdl_trigger();
-    __shared__ double sh_u[BuildShared<T>::D];
-    __shared__ double sh_d[BuildShared<T>::D];
-    __shared__ __align__(16) float sh_q[BuildShared<T>::F];
+    __shared__ F64Rows sh;
     __shared__ unsigned long long s_t;
     const long long nchunks = (P.n + BUILD_ROWS - 1) / BUILD_ROWS;
     const long long total = nchunks * nsweeps;
@@ -554,12 +604,8 @@ k_build_async(PatternView P, const AT *__restrict__ A, T *L, T *U, T *D, T *Udia
         __syncthreads();
         if (t >= total) break;
         const int sweep = (int)(t / nchunks);
-        const int row0 = (int)(t % nchunks) * BUILD_ROWS;
-        const int i = row0 + (threadIdx.x >> 2);
-        typename BuildArith<T>::C u[4] = {0, 0, 0, 0};
-        if (i < P.n) build_row_products<T, true>(P, i, A, L, U, D, L, U, u);
-        build_finish_rows<T, true>(row0, P.n, u, D, sweep == nsweeps - 1 ? Udiag : nullptr,
-                                   sh_u, sh_d, sh_q, nsing);
+        build_rows_f64<true>(P, (int)(t % nchunks) * BUILD_ROWS, A, L, U, D, L, U, D,
+                             sweep == nsweeps - 1 ? Udiag : nullptr, sh, nsing);
     }
 }
 
@@ -582,7 +628,6 @@ k_build_prepare(PatternView P, const double *__restrict__ A, float *__restrict__
     // a CTA's 64 rows are one chunk of a server's arena (BUILD_ROWS = 64)
     const int init_from_a = chunk_init ? chunk_init[blockIdx.x] : init_all;
     __shared__ double sh_u[BuildShared<T>::D];
-    __shared__ double sh_d[BuildShared<T>::D];
     __shared__ __align__(16) float sh_q[BuildShared<T>::F];
     const int row0 = blockIdx.x * BUILD_ROWS;
     const int i = row0 + (threadIdx.x >> 2), q = threadIdx.x & 3;
@@ -624,7 +669,7 @@ k_build_prepare(PatternView P, const double *__restrict__ A, float *__restrict__
             }
         }
     }
-    if (init_from_a) build_finish_rows<T, false>(row0, P.n, ud, D, Udiag, sh_u, sh_d, sh_q, nsing);
+    if (init_from_a) build_finish_rows<T, false>(row0, P.n, ud, D, Udiag, sh_u, sh_q, nsing);
 }
 
 // Us_ij = Dinv_i U_ij for every strictly upper block (FP32 factors), once per
@@ -744,18 +789,17 @@ static abilu_status block_sweeps_t(abilu_factors f, const float *A32, int nsweep
     return ABILU_OK;
 }
 
-template <typename T, typename AT>
-static abilu_status sweeps_t(abilu_factors f, const AT *Asrc, int nsweeps, abilu_mode mode,
-                             cudaStream_t st) {
+static abilu_status sweeps_f64(abilu_factors f, const double *Asrc, int nsweeps, abilu_mode mode,
+                               cudaStream_t st) {
     const PatternView &P = f->p->v;
     const int grid = (P.n + BUILD_ROWS - 1) / BUILD_ROWS;
-    T **L = reinterpret_cast<T **>(f->L), **U = reinterpret_cast<T **>(f->U);
-    T **D = reinterpret_cast<T **>(f->D);
-    T *Ud = reinterpret_cast<T *>(f->Udiag);
+    double **L = reinterpret_cast<double **>(f->L), **U = reinterpret_cast<double **>(f->U);
+    double **D = reinterpret_cast<double **>(f->D);
+    double *Ud = reinterpret_cast<double *>(f->Udiag);
     if (mode == ABILU_SYNC) {
         for (int s = 0; s < nsweeps; s++) {
             const int c = f->cur, o = 1 - f->cur;
-            launch_pdl(k_build_sync<T, AT>, grid, BUILD_THREADS, 0, st,
+            launch_pdl(k_build_sync, grid, BUILD_THREADS, 0, st,
                 P, Asrc, L[c], U[c], D[c], L[o], U[o], D[o], s == nsweeps - 1 ? Ud : nullptr,
                 f->ctr);
             ABILU_LAUNCH_CHECK("k_build_sync");
@@ -766,7 +810,7 @@ static abilu_status sweeps_t(abilu_factors f, const AT *Asrc, int nsweeps, abilu
         int dev = 0, sms = 0, per_sm = per_sm_cache.load(std::memory_order_relaxed);
         cudaGetDevice(&dev);
         if (per_sm < 0) {
-            ABILU_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_build_async<T, AT>,
+            ABILU_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_build_async,
                                                                      BUILD_THREADS, 0));
             per_sm_cache.store(per_sm, std::memory_order_relaxed);
         }
@@ -777,7 +821,7 @@ static abilu_status sweeps_t(abilu_factors f, const AT *Asrc, int nsweeps, abilu
         if (ctas < 1) ctas = 1;
         ABILU_CUDA(cudaMemsetAsync(f->ctr + 1, 0, sizeof(unsigned long long), st));
         const int c = f->cur;
-        launch_pdl(k_build_async<T, AT>, ctas, BUILD_THREADS, 0, st, P, Asrc, L[c], U[c], D[c], Ud,
+        launch_pdl(k_build_async, ctas, BUILD_THREADS, 0, st, P, Asrc, L[c], U[c], D[c], Ud,
             nsweeps, f->ctr, f->ctr + 1);
         ABILU_LAUNCH_CHECK("k_build_async");
     }
@@ -829,7 +873,7 @@ static abilu_status build_t(abilu_factors f, const double *A, int nsweeps, abilu
     } else {
         if (nsweeps == 0) return ABILU_OK;
         abilu_status s = timing_mark(f, 0, st);
-        if (s == ABILU_OK) s = sweeps_t<T, double>(f, A, nsweeps, mode, st);
+        if (s == ABILU_OK) s = sweeps_f64(f, A, nsweeps, mode, st);
         if (s == ABILU_OK) s = timing_mark(f, 1, st);
         return s;
     }

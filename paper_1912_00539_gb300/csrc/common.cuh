@@ -381,4 +381,27 @@ __device__ __forceinline__ C qshfl(C v, int src_q) {
     return __shfl_sync(quad_mask(), v, (int)(lane & ~3u) + src_q);
 }
 
+// Rows by work.  An FP64 instruction holds this GPU's FP64 pipe for 16 cycles
+// whatever lanes are active, so a warp whose eight quads loop over 0 to 3 blocks
+// pays for 3 in every row.  Groups of four warps (32 rows) therefore hand their
+// rows to quads by decreasing block count.  `key` is the work of row base + lane
+// of the group; returns the offset in the group of this quad's row.  `sh` is the
+// warp's 32 bytes of shared memory; every lane calls it.
+__device__ __forceinline__ int row_by_work(int key, unsigned char *sh) {
+    const int lane = threadIdx.x & 31;
+    const int c = min(key, 4);
+    int above = 0, rank = 0;
+#pragma unroll
+    for (int v = 4; v >= 0; v--) {
+        const unsigned m = __ballot_sync(0xffffffffu, c == v);
+        if (c == v) rank = above + __popc(m & ((1u << lane) - 1u));
+        above += __popc(m);
+    }
+    sh[rank] = (unsigned char)lane;
+    __syncwarp();
+    const int off = sh[((threadIdx.x >> 5) & 3) * 8 + (lane >> 2)];
+    __syncwarp();
+    return off;
+}
+
 }  // namespace abilu
