@@ -38,7 +38,13 @@ int red_ctas() {
 
 static inline bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
+// the solve's workspace: made by the first solve (a handle that only builds,
+// exports or applies needs none), grown by a longer restart
 abilu_status ensure_krylov(abilu_factors f, int m) {
+    if (!f->host_status) {
+        ABILU_CUDA(cudaHostAlloc(&f->host_status, host_status_bytes(), cudaHostAllocMapped));
+        memset(f->host_status, 0, host_status_bytes());
+    }
     if (f->krylov && f->krylov_m >= m) return ABILU_OK;
     if (f->krylov) cudaFree(f->krylov);
     f->krylov = nullptr;
@@ -131,9 +137,7 @@ extern "C" abilu_status abilu_factors_create(abilu_pattern p, abilu_dtype dtype,
     f->Us = bus ? m : nullptr; m += bus;
     f->chunk_done = reinterpret_cast<int *>(m); m += bcd;
     e = cudaMemset(f->mem, 0, total);
-    if (e == cudaSuccess) e = cudaHostAlloc(&f->host_status, host_status_bytes(), cudaHostAllocMapped);
     if (e != cudaSuccess) { factors_free(f); return cuda_fail(e, "factors_create"); }
-    memset(f->host_status, 0, host_status_bytes());
     f->cur = 0;
     *out = f;
     return ABILU_OK;

@@ -17,7 +17,7 @@
 // from the same analysis as A's.  Pattern work on the device: a thread per row
 // merges the upper parts of the rows its L blocks name (sorted, at most
 // PLU_MAX_ROW blocks per row); values move between patterns by a per-row merge
-// of the sorted columns; the selection threshold is found by bisection on the
+// of the sorted columns; the selection threshold is found byte by byte on the
 // bit patterns of the non-negative keys (integer counts, exact).
 #include <string.h>
 
@@ -127,30 +127,74 @@ k_import(PatternView P, const double *__restrict__ X, const double *__restrict__
     st_row(D + (size_t)i * BB + q * BS, d);
 }
 
-// cnt[0] += strictly lower blocks with key bits >= tl, cnt[1] += strictly
-// upper ones with key bits >= tu (keys: squared norms, non-negative, so the
-// bit patterns order like the values)
+// Selection of the (budget+1)-th largest key of each side (0: strictly lower
+// blocks, 1: strictly upper; keys are squared norms, non-negative, so their bit
+// patterns order like the values): eight passes of one byte each, from the top.
+// A pass counts, among the keys that agree with the bytes found so far, the 256
+// values of the next byte; its last CTA walks the counts down from 255 to the
+// value that holds the wanted rank, and clears them for the next pass.  Integer
+// counts, so exact and independent of the order.  (A bisection on the host, 64
+// counting passes with a round trip each, took 1.4 ms of a 9 ms call.)
+struct Select {
+    unsigned long long key[2];     // bytes found so far; after the last pass the threshold
+    long long rank[2];             // wanted rank among the keys that agree (from 1)
+    unsigned hist[2][256];
+    unsigned done;
+};
+
+__global__ void k_select_init(Select *s, long long rl, long long ru) {
+    for (int t = threadIdx.x; t < 512; t += blockDim.x) s->hist[t >> 8][t & 255] = 0u;
+    if (threadIdx.x == 0) {
+        s->key[0] = s->key[1] = 0ull;
+        s->rank[0] = rl;
+        s->rank[1] = ru;
+        s->done = 0u;
+    }
+}
+
 __global__ void __launch_bounds__(256)
-k_count_at_least(int n, const int32_t *__restrict__ rowptr, const int32_t *__restrict__ colind,
-                 const unsigned long long *__restrict__ key, unsigned long long tl,
-                 unsigned long long tu, unsigned long long *cnt) {
+k_select_pass(int n, const int32_t *__restrict__ rowptr, const int32_t *__restrict__ diagpos,
+              const unsigned long long *__restrict__ key, int shift, Select *s) {
+    __shared__ unsigned h[2][256];
+    __shared__ bool last;
+    h[0][threadIdx.x] = h[1][threadIdx.x] = 0u;
+    __syncthreads();
     const int i = blockIdx.x * 256 + threadIdx.x;
-    unsigned long long cl = 0, cu = 0;
     if (i < n) {
-        for (int p = rowptr[i]; p < rowptr[i + 1]; p++) {
-            const int j = colind[p];
-            if (j < i) cl += key[p] >= tl;
-            else if (j > i) cu += key[p] >= tu;
+        const int dp = diagpos[i], p1 = rowptr[i + 1];
+        for (int p = rowptr[i]; p < p1; p++) {
+            if (p == dp) continue;
+            const int side = p > dp;
+            const unsigned long long k = key[p];
+            // the bytes above this one (none in the first pass)
+            if (shift == 56 || (k >> (shift + 8)) == (s->key[side] >> (shift + 8)))
+                atomicAdd(&h[side][(unsigned)(k >> shift) & 255u], 1u);
         }
     }
-    for (int o = 16; o > 0; o >>= 1) {
-        cl += __shfl_down_sync(0xffffffffu, cl, o);
-        cu += __shfl_down_sync(0xffffffffu, cu, o);
+    __syncthreads();
+    for (int side = 0; side < 2; side++)
+        if (h[side][threadIdx.x]) atomicAdd(&s->hist[side][threadIdx.x], h[side][threadIdx.x]);
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(&s->done, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    // thread v: does value v of the byte hold the rank?
+    for (int side = 0; side < 2; side++) {
+        h[side][threadIdx.x] = __ldcg(&s->hist[side][threadIdx.x]);
+        s->hist[side][threadIdx.x] = 0u;
     }
-    if ((threadIdx.x & 31) == 0 && (cl | cu)) {
-        atomicAdd(cnt, cl);
-        atomicAdd(cnt + 1, cu);
+    __syncthreads();
+    if (threadIdx.x < 2) {
+        const int side = threadIdx.x;
+        long long r = s->rank[side];
+        int v = 255;
+        while (v > 0 && r > (long long)h[side][v]) r -= h[side][v--];
+        s->key[side] |= (unsigned long long)v << shift;
+        s->rank[side] = r;
     }
+    if (threadIdx.x == 0) s->done = 0u;
 }
 
 // kept blocks of row i: diagonal, lower with key bits > tl, upper with > tu
@@ -158,13 +202,14 @@ k_count_at_least(int n, const int32_t *__restrict__ rowptr, const int32_t *__res
 template <bool FILL>
 __global__ void __launch_bounds__(PLU_THREADS)
 k_compact(int n, const int32_t *__restrict__ rowptr, const int32_t *__restrict__ colind,
-          const unsigned long long *__restrict__ key, unsigned long long tl, unsigned long long tu,
-          int keep_all_l, int keep_all_u, int32_t *__restrict__ cnt,
+          const unsigned long long *__restrict__ key, const Select *__restrict__ sel, int keep_all_l, int keep_all_u,
+          int32_t *__restrict__ cnt,
           const int32_t *__restrict__ out_ptr, int32_t *__restrict__ out_col,
           const double *__restrict__ X, const double *__restrict__ A, double *__restrict__ X_out,
           double *__restrict__ A_out) {
     const int i = blockIdx.x * (PLU_THREADS / 4) + (threadIdx.x >> 2), q = threadIdx.x & 3;
     if (i >= n) return;
+    const unsigned long long tl = sel->key[0], tu = sel->key[1];
     int o = FILL ? out_ptr[i] : 0;
     for (int p = rowptr[i]; p < rowptr[i + 1]; p++) {
         const int j = colind[p];
@@ -191,7 +236,8 @@ namespace abilu {
 
 namespace {
 
-// device allocations released at scope exit
+// device allocations released at scope exit; several arrays share one (carve):
+// an allocation with its release costs this call tens of microseconds
 struct DevBufs {
     std::vector<void *> p;
     ~DevBufs() {
@@ -206,6 +252,28 @@ struct DevBufs {
         return ABILU_OK;
     }
 };
+
+// arrays of one allocation, each on a 256-byte boundary
+struct Carve {
+    char *base = nullptr;
+    size_t at = 0;
+    template <typename T> T *take(size_t count) {
+        T *q = base ? reinterpret_cast<T *>(base + at) : nullptr;
+        at += (sizeof(T) * (count > 0 ? count : 1) + 255) & ~(size_t)255;
+        return q;
+    }
+};
+
+// `lay` takes its arrays from a Carve: once to size the allocation, once on it
+template <typename F> abilu_status carve(DevBufs &bufs, F lay) {
+    Carve c;
+    lay(c);
+    abilu_status s = bufs.get(&c.base, c.at);
+    if (s != ABILU_OK) return s;
+    c.at = 0;
+    lay(c);
+    return ABILU_OK;
+}
 
 struct PatternGuard {
     abilu_pattern p = nullptr;
@@ -249,34 +317,15 @@ static abilu_status factors_from(abilu_pattern p, const double *X, const double 
     return ABILU_OK;
 }
 
-// largest t with #{keys of the side >= t} >= budget + 1, both sides at once,
-// by bisection on the 64-bit patterns (64 counting passes)
-static abilu_status select_thresholds(int n, const int32_t *rowptr, const int32_t *colind,
+// the (budget+1)-th largest keys of both sides into *sel (a side that keeps
+// every block does not use its own)
+static abilu_status select_thresholds(int n, const int32_t *rowptr, const int32_t *diagpos,
                                       const unsigned long long *key, long long bl, long long bu,
-                                      bool need_l, bool need_u, unsigned long long *cnt,
-                                      cudaStream_t st, unsigned long long *tl,
-                                      unsigned long long *tu) {
-    unsigned long long lo[2] = {0ull, 0ull}, hi[2] = {~0ull, ~0ull};
-    const long long need[2] = {bl + 1, bu + 1};
-    const bool act[2] = {need_l, need_u};
-    for (int step = 0; step < 64; step++) {
-        unsigned long long mid[2];
-        for (int k = 0; k < 2; k++) mid[k] = lo[k] + (hi[k] - lo[k]) / 2 + ((hi[k] - lo[k]) & 1);
-        ABILU_CUDA(cudaMemsetAsync(cnt, 0, 2 * sizeof(unsigned long long), st));
-        k_count_at_least<<<counted(grid_rows(n, 256)), 256, 0, st>>>(n, rowptr, colind, key, mid[0],
-                                                                     mid[1], cnt);
-        ABILU_LAUNCH_CHECK("k_count_at_least");
-        unsigned long long h[2];
-        ABILU_CUDA(cudaMemcpyAsync(h, cnt, sizeof h, cudaMemcpyDeviceToHost, st));
-        ABILU_CUDA(cudaStreamSynchronize(st));
-        for (int k = 0; k < 2; k++) {
-            if (!act[k] || lo[k] == hi[k]) continue;
-            if ((long long)h[k] >= need[k]) lo[k] = mid[k];
-            else hi[k] = mid[k] - 1;
-        }
-    }
-    *tl = lo[0];
-    *tu = lo[1];
+                                      Select *sel, cudaStream_t st) {
+    k_select_init<<<counted(1), 256, 0, st>>>(sel, bl + 1, bu + 1);
+    for (int shift = 56; shift >= 0; shift -= 8)
+        k_select_pass<<<counted(grid_rows(n, 256)), 256, 0, st>>>(n, rowptr, diagpos, key, shift, sel);
+    ABILU_LAUNCH_CHECK("k_select_pass");
     return ABILU_OK;
 }
 
@@ -348,20 +397,25 @@ extern "C" abilu_status abilu_parilut(abilu_pattern pA, const double *A,
     const long long bl = (long long)(o->fill * (double)VA.nl), bu = (long long)(o->fill * (double)VA.nu);
     DevBufs bufs;
     unsigned *err = nullptr;
-    unsigned long long *cnt = nullptr;
+    Select *sel = nullptr;
     long long *scratch = nullptr;
-    int32_t *rowcnt = nullptr;
-    double *D = nullptr;
-    abilu_status s;
-    if ((s = bufs.get(&err, 1)) != ABILU_OK || (s = bufs.get(&cnt, 2)) != ABILU_OK ||
-        (s = bufs.get(&scratch, (size_t)n / 4096 + 2)) != ABILU_OK ||
-        (s = bufs.get(&rowcnt, (size_t)n)) != ABILU_OK || (s = bufs.get(&D, (size_t)n * BB)) != ABILU_OK)
-        return s;
+    int32_t *rowcnt = nullptr, *rp2 = nullptr, *rp3 = nullptr;
+    double *D = nullptr, *X = nullptr;
+    abilu_status s = carve(bufs, [&](Carve &c) {
+        err = c.take<unsigned>(1);
+        sel = c.take<Select>(1);
+        scratch = c.take<long long>((size_t)n / 4096 + 2);
+        rowcnt = c.take<int32_t>(n);
+        rp2 = c.take<int32_t>((size_t)n + 1);
+        rp3 = c.take<int32_t>((size_t)n + 1);
+        D = c.take<double>((size_t)n * BB);
+        if (o->iters > 0) X = c.take<double>((size_t)VA.nnzb * BB);
+    });
+    if (s != ABILU_OK) return s;
     ABILU_CUDA(cudaMemsetAsync(err, 0, sizeof(unsigned), st));
 
     // start: X = A, `sweeps` synchronous sweeps on A's pattern
     PatternGuard pcur;   // the current pattern when owned (NULL: A's)
-    double *X = nullptr;
     {
         FactorsGuard f0;
         if ((s = abilu_factors_create(pA, ABILU_F64, &f0.f)) != ABILU_OK) return s;
@@ -389,28 +443,31 @@ extern "C" abilu_status abilu_parilut(abilu_pattern pA, const double *A,
             fo.f = nullptr;
             return ABILU_OK;
         }
-        if ((s = bufs.get(&X, (size_t)VA.nnzb * BB)) != ABILU_OK) return s;
         if ((s = export_dispatch(f0.f, X, D, st)) != ABILU_OK) return s;
         ABILU_CUDA(cudaStreamSynchronize(st));
     }
     for (int it = 0; it < o->iters; it++) {
         const PatternView &VC = pcur.p ? pcur.p->v : VA;
         // fill: the pattern of L U
-        int32_t *rp2 = nullptr, *ci2 = nullptr;
-        if ((s = bufs.get(&rp2, (size_t)n + 1)) != ABILU_OK) return s;
         k_lu_pattern<false><<<counted(grid_rows(n, PLU_THREADS)), PLU_THREADS, 0, st>>>(
             n, VC.rowptr, VC.colind, VC.diagpos, rowcnt, nullptr, nullptr, err);
         ABILU_LAUNCH_CHECK("k_lu_pattern");
         if ((s = scan_i32(rowcnt, rp2, n, scratch, err, st)) != ABILU_OK) return s;
         int32_t nnz2 = 0;
         if ((s = read_total(rp2 + n, err, st, &nnz2)) != ABILU_OK) return s;
-        if ((s = bufs.get(&ci2, (size_t)nnz2)) != ABILU_OK) return s;
+        int32_t *ci2 = nullptr;
+        double *X2 = nullptr, *A2 = nullptr;
+        unsigned long long *key = nullptr;
+        s = carve(bufs, [&](Carve &c) {
+            ci2 = c.take<int32_t>((size_t)nnz2);
+            X2 = c.take<double>((size_t)nnz2 * BB);
+            A2 = c.take<double>((size_t)nnz2 * BB);
+            key = c.take<unsigned long long>((size_t)nnz2);
+        });
+        if (s != ABILU_OK) return s;
         k_lu_pattern<true><<<counted(grid_rows(n, PLU_THREADS)), PLU_THREADS, 0, st>>>(
             n, VC.rowptr, VC.colind, VC.diagpos, nullptr, rp2, ci2, err);
         ABILU_LAUNCH_CHECK("k_lu_pattern");
-        double *X2 = nullptr, *A2 = nullptr;
-        if ((s = bufs.get(&X2, (size_t)nnz2 * BB)) != ABILU_OK) return s;
-        if ((s = bufs.get(&A2, (size_t)nnz2 * BB)) != ABILU_OK) return s;
         k_map_blocks<<<counted(grid_rows(n, PLU_THREADS / 4)), PLU_THREADS, 0, st>>>(
             n, rp2, ci2, VC.rowptr, VC.colind, X, VA.rowptr, VA.colind, A, X2, A2);
         ABILU_LAUNCH_CHECK("k_map_blocks");
@@ -424,31 +481,30 @@ extern "C" abilu_status abilu_parilut(abilu_pattern pA, const double *A,
         }
         // drop: the largest strictly lower and strictly upper blocks
         const PatternView &V2 = p2.p->v;
-        unsigned long long *key = nullptr;
-        if ((s = bufs.get(&key, (size_t)nnz2)) != ABILU_OK) return s;
         k_block_norm2<<<counted(grid_rows(nnz2, 256)), 256, 0, st>>>(X2, nnz2, reinterpret_cast<double *>(key));
         ABILU_LAUNCH_CHECK("k_block_norm2");
         const bool all_l = (long long)V2.nl <= bl, all_u = (long long)V2.nu <= bu;
-        unsigned long long tl = 0, tu = 0;
         if (!all_l || !all_u) {
-            s = select_thresholds(n, V2.rowptr, V2.colind, key, bl, bu, !all_l, !all_u, cnt, st, &tl, &tu);
+            s = select_thresholds(n, V2.rowptr, V2.diagpos, key, bl, bu, sel, st);
             if (s != ABILU_OK) return s;
         }
-        int32_t *rp3 = nullptr, *ci3 = nullptr;
-        if ((s = bufs.get(&rp3, (size_t)n + 1)) != ABILU_OK) return s;
         k_compact<false><<<counted(grid_rows(n, PLU_THREADS / 4)), PLU_THREADS, 0, st>>>(
-            n, V2.rowptr, V2.colind, key, tl, tu, all_l, all_u, rowcnt, nullptr, nullptr, nullptr,
+            n, V2.rowptr, V2.colind, key, sel, all_l, all_u, rowcnt, nullptr, nullptr, nullptr,
             nullptr, nullptr, nullptr);
         ABILU_LAUNCH_CHECK("k_compact");
         if ((s = scan_i32(rowcnt, rp3, n, scratch, err, st)) != ABILU_OK) return s;
         int32_t nnz3 = 0;
         if ((s = read_total(rp3 + n, err, st, &nnz3)) != ABILU_OK) return s;
+        int32_t *ci3 = nullptr;
         double *X3 = nullptr, *A3 = nullptr;
-        if ((s = bufs.get(&ci3, (size_t)nnz3)) != ABILU_OK) return s;
-        if ((s = bufs.get(&X3, (size_t)nnz3 * BB)) != ABILU_OK) return s;
-        if ((s = bufs.get(&A3, (size_t)nnz3 * BB)) != ABILU_OK) return s;
+        s = carve(bufs, [&](Carve &c) {
+            ci3 = c.take<int32_t>((size_t)nnz3);
+            X3 = c.take<double>((size_t)nnz3 * BB);
+            A3 = c.take<double>((size_t)nnz3 * BB);
+        });
+        if (s != ABILU_OK) return s;
         k_compact<true><<<counted(grid_rows(n, PLU_THREADS / 4)), PLU_THREADS, 0, st>>>(
-            n, V2.rowptr, V2.colind, key, tl, tu, all_l, all_u, nullptr, rp3, ci3, X2, A2, X3, A3);
+            n, V2.rowptr, V2.colind, key, sel, all_l, all_u, nullptr, rp3, ci3, X2, A2, X3, A3);
         ABILU_LAUNCH_CHECK("k_compact");
         PatternGuard p3;
         if ((s = abilu_pattern_create(n, nnz3, rp3, ci3, stream, &p3.p)) != ABILU_OK) return s;

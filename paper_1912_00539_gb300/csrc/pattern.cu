@@ -312,10 +312,22 @@ extern "C" abilu_status abilu_pattern_create(int32_t n, int32_t nnzb, const int3
     auto allocs = new std::vector<void *>();
     p->mem = allocs;
     cudaGetDevice(&p->device);
-    auto alloc = [&](void **ptr, size_t bytes) -> abilu_status {
-        cudaError_t e = cudaMalloc(ptr, bytes < 16 ? 16 : bytes);
+    // two allocations hold every array: one for what n and nnzb size (the
+    // strictly lower and upper blocks share nnzb - n columns), one for the pairs
+    // and the work list.  (One per array, 22 of them, took most of this call:
+    // about 36 us each with its share of the release.)
+    size_t bytes = 0;
+    auto room = [&](size_t b) {
+        const size_t at = bytes;
+        bytes += (b + 255) & ~(size_t)255;
+        return at;
+    };
+    auto alloc = [&](char **ptr) -> abilu_status {
+        void *q = nullptr;
+        cudaError_t e = cudaMalloc(&q, bytes);
         if (e != cudaSuccess) return cuda_fail(e, "pattern_create: cudaMalloc");
-        allocs->push_back(*ptr);
+        allocs->push_back(q);
+        *ptr = static_cast<char *>(q);
         return ABILU_OK;
     };
 #define TRY(x)                                   \
@@ -323,24 +335,27 @@ extern "C" abilu_status abilu_pattern_create(int32_t n, int32_t nnzb, const int3
         abilu_status s_ = (x);                   \
         if (s_ != ABILU_OK) { pattern_free(p); return s_; } \
     } while (0)
-    int32_t *d_rowptr, *d_colind, *diagpos, *lcnt, *ucnt, *lrow, *urow, *pair_cnt, *pair_ptr;
-    long long *scratch;
-    unsigned *err;
-    int *max_row;
-    int ntiles = (nnzb + SCAN_TILE - 1) / SCAN_TILE + 1;
-    TRY(alloc((void **)&d_rowptr, sizeof(int32_t) * (n + 1)));
-    TRY(alloc((void **)&d_colind, sizeof(int32_t) * nnzb));
-    TRY(alloc((void **)&diagpos, sizeof(int32_t) * n));
-    TRY(alloc((void **)&lcnt, sizeof(int32_t) * n));
-    TRY(alloc((void **)&ucnt, sizeof(int32_t) * n));
+    const int ntiles = (nnzb + SCAN_TILE - 1) / SCAN_TILE + 1;
+    const size_t w4 = sizeof(int32_t), nn = (size_t)n, nb = (size_t)nnzb;
+    const size_t o_rowptr = room(w4 * (nn + 1)), o_colind = room(w4 * nb), o_diag = room(w4 * nn);
+    const size_t o_lcnt = room(w4 * nn), o_ucnt = room(w4 * nn);
     // +68 entries: a sweep copies rowptr windows of 68 entries per 64-row chunk
-    TRY(alloc((void **)&lrow, sizeof(int32_t) * (n + 1 + 68)));
-    TRY(alloc((void **)&urow, sizeof(int32_t) * (n + 1 + 68)));
-    TRY(alloc((void **)&pair_cnt, sizeof(int32_t) * nnzb));
-    TRY(alloc((void **)&pair_ptr, sizeof(int32_t) * (nnzb + 1)));
-    TRY(alloc((void **)&scratch, sizeof(long long) * ntiles));
-    TRY(alloc((void **)&err, sizeof(unsigned) * 4));
-    max_row = reinterpret_cast<int *>(err + 2);
+    const size_t o_lrow = room(w4 * (nn + 1 + 68)), o_urow = room(w4 * (nn + 1 + 68));
+    const size_t o_pcnt = room(w4 * nb), o_pptr = room(w4 * (nb + 1));
+    const size_t o_wptr = room(w4 * (nn + 1)), o_wpos = room(w4 * nb);
+    // padded to whole 16-byte groups (+16 bytes each): the sweeps copy index
+    // ranges rounded out to 16-byte boundaries with bulk asynchronous copies
+    const size_t o_cols = room(w4 * (nb - nn + 16));
+    const size_t o_scratch = room(sizeof(long long) * (size_t)ntiles), o_err = room(sizeof(unsigned) * 4);
+    char *m = nullptr;
+    TRY(alloc(&m));
+    auto i32 = [&](size_t at) { return reinterpret_cast<int32_t *>(m + at); };
+    int32_t *d_rowptr = i32(o_rowptr), *d_colind = i32(o_colind), *diagpos = i32(o_diag);
+    int32_t *lcnt = i32(o_lcnt), *ucnt = i32(o_ucnt), *lrow = i32(o_lrow), *urow = i32(o_urow);
+    int32_t *pair_cnt = i32(o_pcnt), *pair_ptr = i32(o_pptr), *wptr = i32(o_wptr), *wpos = i32(o_wpos);
+    long long *scratch = reinterpret_cast<long long *>(m + o_scratch);
+    unsigned *err = reinterpret_cast<unsigned *>(m + o_err);
+    int *max_row = reinterpret_cast<int *>(err + 2);
     auto cu = [&](cudaError_t e, const char *w) -> abilu_status {
         return e == cudaSuccess ? ABILU_OK : cuda_fail(e, w);
     };
@@ -363,45 +378,40 @@ extern "C" abilu_status abilu_pattern_create(int32_t n, int32_t nnzb, const int3
     }
     TRY(scan_i32(lcnt, lrow, n, scratch, err, st));
     TRY(scan_i32(ucnt, urow, n, scratch, err, st));
-    int32_t nl_nu[2];
-    TRY(cu(cudaMemcpyAsync(&nl_nu[0], lrow + n, 4, cudaMemcpyDeviceToHost, st), "read nl"));
-    TRY(cu(cudaMemcpyAsync(&nl_nu[1], urow + n, 4, cudaMemcpyDeviceToHost, st), "read nu"));
-    TRY(cu(cudaStreamSynchronize(st), "sync"));
-    int32_t *lcol, *ucol;
-    // padded to whole 16-byte groups (+16 bytes): the sweeps copy index ranges
-    // rounded out to 16-byte boundaries with bulk asynchronous copies
-    TRY(alloc((void **)&lcol, sizeof(int32_t) * ((nl_nu[0] + 3) / 4 * 4 + 4)));
-    TRY(alloc((void **)&ucol, sizeof(int32_t) * ((nl_nu[1] + 3) / 4 * 4 + 4)));
-    k_pat_cols<<<counted(gb), 256, 0, st>>>(n, d_rowptr, d_colind, diagpos, lrow, urow, lcol, ucol);
     k_pat_pairs<false><<<counted(gb), 256, 0, st>>>(n, d_rowptr, d_colind, diagpos, lrow, urow, pair_cnt,
                                            nullptr, nullptr);
     TRY(cu(cudaGetLastError(), "k_pat_pairs count"));
     TRY(scan_i32(pair_cnt, pair_ptr, nnzb, scratch, err, st));
-    int32_t npairs;
+    int32_t *wcnt = lcnt;   // lcnt is free again: the work list's counts
+    k_pat_work<false><<<counted(gb), 256, 0, st>>>(n, d_rowptr, d_colind, diagpos, lrow, urow,
+                                                   pair_ptr, wcnt, nullptr, nullptr);
+    TRY(cu(cudaGetLastError(), "k_pat_work count"));
+    TRY(scan_i32(wcnt, wptr, n, scratch, err, st));
+    int32_t nl_nu[2], npairs, nwork;
+    TRY(cu(cudaMemcpyAsync(&nl_nu[0], lrow + n, 4, cudaMemcpyDeviceToHost, st), "read nl"));
+    TRY(cu(cudaMemcpyAsync(&nl_nu[1], urow + n, 4, cudaMemcpyDeviceToHost, st), "read nu"));
     TRY(cu(cudaMemcpyAsync(&npairs, pair_ptr + nnzb, 4, cudaMemcpyDeviceToHost, st), "read npairs"));
+    TRY(cu(cudaMemcpyAsync(&nwork, wptr + n, 4, cudaMemcpyDeviceToHost, st), "read nwork"));
     TRY(cu(cudaMemcpyAsync(herr, err, sizeof herr, cudaMemcpyDeviceToHost, st), "read err"));
     TRY(cu(cudaStreamSynchronize(st), "sync"));
     if (herr[0] & (1u << 8)) {
         pattern_free(p);
         return fail(ABILU_EINVAL, "pattern_create: more than 2^31 product pairs");
     }
-    int2 *pairs;
-    TRY(alloc((void **)&pairs, sizeof(int2) * (npairs > 0 ? npairs : 1)));
+    int32_t *lcol = i32(o_cols), *ucol = lcol + ((nl_nu[0] + 3) / 4 * 4 + 4);
+    k_pat_cols<<<counted(gb), 256, 0, st>>>(n, d_rowptr, d_colind, diagpos, lrow, urow, lcol, ucol);
+    bytes = 0;
+    const size_t o_pairs = room(sizeof(int2) * (npairs > 0 ? npairs : 1));
+    const size_t o_work = room(sizeof(int4) * (nwork > 0 ? nwork : 1));
+    const size_t o_items = room(sizeof(WorkItem) * (nwork > 0 ? nwork : 1));
+    char *m2 = nullptr;
+    TRY(alloc(&m2));
+    int2 *pairs = reinterpret_cast<int2 *>(m2 + o_pairs);
+    int4 *work = reinterpret_cast<int4 *>(m2 + o_work);
+    WorkItem *items = reinterpret_cast<WorkItem *>(m2 + o_items);
     k_pat_pairs<true><<<counted(gb), 256, 0, st>>>(n, d_rowptr, d_colind, diagpos, lrow, urow, nullptr,
                                           pair_ptr, pairs);
     TRY(cu(cudaGetLastError(), "k_pat_pairs fill"));
-    // work list of the build sweeps
-    int32_t *wcnt = lcnt, *wptr;  // lcnt is free again: reuse it for the counts
-    TRY(alloc((void **)&wptr, sizeof(int32_t) * (n + 1)));
-    k_pat_work<false><<<counted(gb), 256, 0, st>>>(n, d_rowptr, d_colind, diagpos, lrow, urow,
-                                                   pair_ptr, wcnt, nullptr, nullptr);
-    TRY(cu(cudaGetLastError(), "k_pat_work count"));
-    TRY(scan_i32(wcnt, wptr, n, scratch, err, st));
-    int32_t nwork;
-    TRY(cu(cudaMemcpyAsync(&nwork, wptr + n, 4, cudaMemcpyDeviceToHost, st), "read nwork"));
-    TRY(cu(cudaStreamSynchronize(st), "sync"));
-    int4 *work;
-    TRY(alloc((void **)&work, sizeof(int4) * (nwork > 0 ? nwork : 1)));
     k_pat_work<true><<<counted(gb), 256, 0, st>>>(n, d_rowptr, d_colind, diagpos, lrow, urow,
                                                   pair_ptr, nullptr, wptr, work);
     TRY(cu(cudaGetLastError(), "k_pat_work fill"));
@@ -412,10 +422,6 @@ extern "C" abilu_status abilu_pattern_create(int32_t n, int32_t nnzb, const int3
             TRY(cu(cudaGetLastError(), "k_pat_work_sort"));
         }
     }
-    int32_t *wpos;
-    WorkItem *items;
-    TRY(alloc((void **)&wpos, sizeof(int32_t) * nnzb));
-    TRY(alloc((void **)&items, sizeof(WorkItem) * (nwork > 0 ? nwork : 1)));
     TRY(cu(cudaMemsetAsync(wpos, 0xFF, sizeof(int32_t) * nnzb, st), "memset wpos"));
     if (nwork > 0) {
         k_pat_work_items<<<counted((nwork + 255) / 256), 256, 0, st>>>(nwork, work, pair_ptr, pairs,
