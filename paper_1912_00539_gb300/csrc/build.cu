@@ -631,7 +631,8 @@ k_build_prepare(PatternView P, const double *__restrict__ A, float *__restrict__
     __shared__ __align__(16) float sh_q[BuildShared<T>::F];
     const int row0 = blockIdx.x * BUILD_ROWS;
     const int i = row0 + (threadIdx.x >> 2), q = threadIdx.x & 3;
-    typename BuildArith<T>::C ud[4] = {0, 0, 0, 0};
+    using C = typename BuildArith<T>::C;
+    C ud[4] = {0, 0, 0, 0};
     if (i < P.n) {
         const int p0 = P.rowptr[i], p1 = P.rowptr[i + 1], dp = P.diagpos[i];
         const int lb = P.lrow[i], ub = P.urow[i];
@@ -650,21 +651,25 @@ k_build_prepare(PatternView P, const double *__restrict__ A, float *__restrict__
             for (int k = 0; k < 4; k++) {
                 const int p = pb + k;
                 if (p >= p1) break;
+                C v[4];   // converted once, stored where it goes
+                if constexpr (sizeof(T) == 8) {
+#pragma unroll
+                    for (int c = 0; c < 4; c++) v[c] = a[k][c];
+                } else {
+                    to_f32x4(a[k], v);
+                }
                 if (p > dp && wp[k] < 0) {  // not a work item: a constant U block
-                    st_row(U + (size_t)(ub + p - dp - 1) * BB + q * BS, a[k]);
-                    if (Uother) st_row(Uother + (size_t)(ub + p - dp - 1) * BB + q * BS, a[k]);
+                    st_row(U + (size_t)(ub + p - dp - 1) * BB + q * BS, v);
+                    if (Uother) st_row(Uother + (size_t)(ub + p - dp - 1) * BB + q * BS, v);
                     continue;
                 }
-                if (A32) st_row(A32 + (size_t)wp[k] * BB + q * BS, a[k]);  // work order
+                if constexpr (sizeof(T) < 8) st_row(A32 + (size_t)wp[k] * BB + q * BS, v);  // work order
                 if (!init_from_a) continue;
-                if (p < dp) st_row(L + (size_t)(lb + p - p0) * BB + q * BS, a[k]);
-                else if (p > dp) st_row(U + (size_t)(ub + p - dp - 1) * BB + q * BS, a[k]);
+                if (p < dp) st_row(L + (size_t)(lb + p - p0) * BB + q * BS, v);
+                else if (p > dp) st_row(U + (size_t)(ub + p - dp - 1) * BB + q * BS, v);
                 else {
 #pragma unroll
-                    for (int c = 0; c < 4; c++) {
-                        if constexpr (sizeof(T) == 8) ud[c] = a[k][c];
-                        else ud[c] = to_f32(a[k][c]);
-                    }
+                    for (int c = 0; c < 4; c++) ud[c] = v[c];
                 }
             }
         }

@@ -241,20 +241,82 @@ __device__ __forceinline__ double to_f64(float x) {
     return __hiloint2double((int)hi, (int)lo);
 }
 
+// FP32 -> FP64 with every case in integer instructions
+__device__ __forceinline__ double to_f64_int(float x) {
+    const unsigned u = __float_as_uint(x), sign = u & 0x80000000u;
+    unsigned ex = (u >> 23) & 0xFFu, m = u & 0x7FFFFFu;
+    if (ex == 0xFFu)   // Inf; NaN made quiet
+        return __hiloint2double((int)(sign | 0x7FF00000u | (m ? 0x80000u : 0u) | (m >> 3)), (int)((m & 7u) << 29));
+    unsigned e = ex + (1023u - 127u);
+    if (ex == 0u) {
+        if (m == 0u) return __hiloint2double((int)sign, 0);
+        const int z = __clz((int)m) - 8;   // subnormal: shift the leading bit to bit 23
+        m = (m << z) & 0x7FFFFFu;
+        e = 1023u - 126u - (unsigned)z;
+    }
+    return __hiloint2double((int)(sign | (e << 20) | (m >> 3)), (int)((m & 7u) << 29));
+}
+
+// Four conversions at once, the rows' form: the normal cases of all four in a
+// few integer instructions each, everything else (zeros among them) behind one
+// branch.  The scalar forms above issue their hardware fallback for every
+// element, predicated off, and it takes FP64-pipe cycles all the same: the
+// build's prepare pass (16 conversions a thread) had that pipe 77% busy without
+// an FP64 operation of its own.
+__device__ __forceinline__ void to_f32x4(const double d[4], float f[4]) {
+    unsigned u[4], bad = 0u;
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+        const unsigned hi = (unsigned)__double2hiint(d[k]), lo = (unsigned)__double2loint(d[k]);
+        // exponent field and 23 mantissa bits, rebased by -896 (mod 2^32)
+        unsigned t = __funnelshift_l(lo, hi, 3) + 0x40000000u;
+        t += ((lo & 0x1FFFFFFFu) + 0x0FFFFFFFu + (t & 1u)) >> 29;   // nearest even
+        u[k] = (t & 0x7FFFFFFFu) | (hi & 0x80000000u);
+        // FP64 exponents 897 .. 1150 are FP32's 1 .. 254 (rounding up to Inf included)
+        bad |= (((hi >> 20) & 0x7FFu) - 897u) > 253u;
+    }
+    if (!bad) {
+#pragma unroll
+        for (int k = 0; k < 4; k++) f[k] = __uint_as_float(u[k]);
+    } else {
+#pragma unroll
+        for (int k = 0; k < 4; k++) f[k] = to_f32_int(d[k]);
+    }
+}
+
+__device__ __forceinline__ void to_f64x4(const float x[4], double d[4]) {
+    unsigned bad = 0u;
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+        const unsigned u = __float_as_uint(x[k]);
+        bad |= (((u >> 23) & 0xFFu) - 1u) > 253u;   // zero, subnormal, Inf, NaN
+        d[k] = __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7FFFFFFFu) >> 3) + (896u << 20))),
+                                (int)(u << 29));
+    }
+    if (bad) {
+        d[0] = to_f64_int(x[0]);
+        d[1] = to_f64_int(x[1]);
+        d[2] = to_f64_int(x[2]);
+        d[3] = to_f64_int(x[3]);
+    }
+}
+
 __device__ __forceinline__ void ld_row(const double *p, double v[4]) {
     double2 a = reinterpret_cast<const double2 *>(p)[0];
     double2 b = reinterpret_cast<const double2 *>(p)[1];
     v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
 }
 __device__ __forceinline__ void ld_row(const float *p, double v[4]) {
-    float4 a = *reinterpret_cast<const float4 *>(p);
-    v[0] = to_f64(a.x); v[1] = to_f64(a.y); v[2] = to_f64(a.z); v[3] = to_f64(a.w);
+    const float4 a = *reinterpret_cast<const float4 *>(p);
+    const float w[4] = {a.x, a.y, a.z, a.w};
+    to_f64x4(w, v);
 }
 __device__ __forceinline__ void ld_row(const __nv_bfloat16 *p, double v[4]) {
     uint2 u = *reinterpret_cast<const uint2 *>(p);
     float2 a = __bfloat1622float2(*reinterpret_cast<__nv_bfloat162 *>(&u.x));
     float2 b = __bfloat1622float2(*reinterpret_cast<__nv_bfloat162 *>(&u.y));
-    v[0] = to_f64(a.x); v[1] = to_f64(a.y); v[2] = to_f64(b.x); v[3] = to_f64(b.y);
+    const float w[4] = {a.x, a.y, b.x, b.y};
+    to_f64x4(w, v);
 }
 __device__ __forceinline__ void ld_row(const float *p, float v[4]) {
     float4 a = *reinterpret_cast<const float4 *>(p);
@@ -269,7 +331,7 @@ __device__ __forceinline__ void ld_row(const __nv_bfloat16 *p, float v[4]) {
 __device__ __forceinline__ void ld_row(const double *p, float v[4]) {
     double w[4];
     ld_row(p, w);
-    v[0] = to_f32(w[0]); v[1] = to_f32(w[1]); v[2] = to_f32(w[2]); v[3] = to_f32(w[3]);
+    to_f32x4(w, v);
 }
 
 // volatile (relaxed, uncached-in-L1) loads for data other threads may be
@@ -316,21 +378,26 @@ __device__ __forceinline__ void st_row(double *p, const double v[4]) {
     reinterpret_cast<double2 *>(p)[1] = make_double2(v[2], v[3]);
 }
 __device__ __forceinline__ void st_row(float *p, const double v[4]) {
-    *reinterpret_cast<float4 *>(p) = make_float4(to_f32(v[0]), to_f32(v[1]), to_f32(v[2]), to_f32(v[3]));
+    float f[4];
+    to_f32x4(v, f);
+    *reinterpret_cast<float4 *>(p) = make_float4(f[0], f[1], f[2], f[3]);
 }
 __device__ __forceinline__ void st_row(float *p, const float v[4]) {
     *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
 }
 __device__ __forceinline__ void st_row(__nv_bfloat16 *p, const double v[4]) {
-    __nv_bfloat162 a = __floats2bfloat162_rn(to_f32(v[0]), to_f32(v[1]));
-    __nv_bfloat162 b = __floats2bfloat162_rn(to_f32(v[2]), to_f32(v[3]));
+    float f[4];
+    to_f32x4(v, f);
+    __nv_bfloat162 a = __floats2bfloat162_rn(f[0], f[1]);
+    __nv_bfloat162 b = __floats2bfloat162_rn(f[2], f[3]);
     uint2 u;
     u.x = *reinterpret_cast<unsigned *>(&a);
     u.y = *reinterpret_cast<unsigned *>(&b);
     *reinterpret_cast<uint2 *>(p) = u;
 }
 __device__ __forceinline__ void st_row(double *p, const float v[4]) {
-    double w[4] = {to_f64(v[0]), to_f64(v[1]), to_f64(v[2]), to_f64(v[3])};
+    double w[4];
+    to_f64x4(v, w);
     st_row(p, w);
 }
 __device__ __forceinline__ void st_row(__nv_bfloat16 *p, const float v[4]) {
