@@ -281,13 +281,33 @@ constexpr int WORK_PER_CTA = BUILD_THREADS / 4;
 static_assert(WORK_PER_CTA == WORK_CHUNK, "work list chunks are sorted per CTA");
 static_assert(sizeof(WorkItem) == 32, "work records are two 16-byte loads");
 
-// s -= L_ik U_kj for the quad's block (thread q: row q); u's row k lives in thread k
-__device__ __forceinline__ void sub_product(float s[4], const float l[4], const float u[4]) {
-    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+// The quad's rows of one block through shared memory: thread q stores row q,
+// after the barrier every thread reads the four rows (one 16-byte store and four
+// broadcast loads; 16 shuffles before, which had the load/store unit 41% and
+// the L1 73% busy, and spilled at 48 and 40 registers; at 40 registers and six
+// CTAs per SM the in-place sweeps now run without: 6 sweeps at 512x512 397 -> 379
+// us, the synchronous ones unchanged at 66 us each)
+__device__ __forceinline__ void put_row(float *sh, const float u[4]) {
+    reinterpret_cast<float4 *>(sh)[threadIdx.x & 3] = make_float4(u[0], u[1], u[2], u[3]);
+}
+
+// o = s M (row q of the product) with M's rows in shared memory
+__device__ __forceinline__ void row_times(float o[4], const float s[4], const float *sh) {
 #pragma unroll
-    for (int k = 0; k < 4; k++)
-#pragma unroll
-        for (int c = 0; c < 4; c++) acc[c] += l[k] * qshfl(u[c], k);
+    for (int k = 0; k < 4; k++) {
+        const float4 r = reinterpret_cast<const float4 *>(sh)[k];
+        if (k == 0) {
+            o[0] = s[0] * r.x; o[1] = s[0] * r.y; o[2] = s[0] * r.z; o[3] = s[0] * r.w;
+        } else {
+            o[0] += s[k] * r.x; o[1] += s[k] * r.y; o[2] += s[k] * r.z; o[3] += s[k] * r.w;
+        }
+    }
+}
+
+// s -= l U (row q) with U's rows in shared memory
+__device__ __forceinline__ void sub_product(float s[4], const float l[4], const float *sh) {
+    float acc[4];
+    row_times(acc, l, sh);
 #pragma unroll
     for (int c = 0; c < 4; c++) s[c] -= acc[c];
 }
@@ -298,45 +318,53 @@ __device__ __forceinline__ void build_block(const PatternView &P, int w,
                                             const T *Uin, const T *Din, T *Lout, T *Uout, T *Dout,
                                             T *Udiag, float *sh_q, unsigned long long *nsing) {
     const int q = threadIdx.x & 3;
+    const unsigned m = quad_mask();
     const WorkItem it = P.work[w];
     float s[4], d[4];
     ld_row(A32 + (size_t)w * BB + q * BS, s);
     const int kind = it.kind_np & 3, np = it.kind_np >> 2, dst = it.dst;
     if (kind == WORK_L) ld_row_sel<VOL>(Din + (size_t)it.j * BB + q * BS, d);
     if (np > 0) {  // products in pair order (ascending k)
-        float l0[4], u0[4], l1[4], u1[4];
+        float l0[4], u[4], l1[4];
         ld_row_sel<VOL>(Lin + (size_t)it.pr[0].x * BB + q * BS, l0);  // row q of L_ik
-        ld_row_sel<VOL>(Uin + (size_t)it.pr[0].y * BB + q * BS, u0);  // row q of U_kj
+        ld_row_sel<VOL>(Uin + (size_t)it.pr[0].y * BB + q * BS, u);   // row q of U_kj
         if (np > 1) {
+            float u1[4];
             ld_row_sel<VOL>(Lin + (size_t)it.pr[1].x * BB + q * BS, l1);
             ld_row_sel<VOL>(Uin + (size_t)it.pr[1].y * BB + q * BS, u1);
+            put_row(sh_q + 16, u1);
         }
-        sub_product(s, l0, u0);
-        if (np > 1) sub_product(s, l1, u1);
+        put_row(sh_q, u);
+        __syncwarp(m);
+        sub_product(s, l0, sh_q);
+        if (np > 1) sub_product(s, l1, sh_q + 16);
         for (int t = 2; t < np; t++) {
             const int2 pr = P.pairs[it.t0 + t];
             ld_row_sel<VOL>(Lin + (size_t)pr.x * BB + q * BS, l0);
-            ld_row_sel<VOL>(Uin + (size_t)pr.y * BB + q * BS, u0);
-            sub_product(s, l0, u0);
+            ld_row_sel<VOL>(Uin + (size_t)pr.y * BB + q * BS, u);
+            __syncwarp(m);   // every thread has read the previous rows
+            put_row(sh_q, u);
+            __syncwarp(m);
+            sub_product(s, l0, sh_q);
         }
     }
-    if (kind == WORK_L) {  // L_ij = S Dinv_j; row k of Dinv_j lives in thread k
+    if (kind == WORK_L) {  // L_ij = S Dinv_j
         float o[4];
-#pragma unroll
-        for (int c = 0; c < 4; c++) {
-            float d0 = qshfl(d[c], 0), d1 = qshfl(d[c], 1), d2 = qshfl(d[c], 2), d3 = qshfl(d[c], 3);
-            o[c] = s[0] * d0 + s[1] * d1 + s[2] * d2 + s[3] * d3;
-        }
+        put_row(sh_q + 32, d);
+        __syncwarp(m);
+        row_times(o, s, sh_q + 32);
         st_row_sel<VOL>(Lout + (size_t)dst * BB + q * BS, o);
     } else if (kind == WORK_U) {
         st_row_sel<VOL>(Uout + (size_t)dst * BB + q * BS, s);
     } else {  // U_ii = S, Dinv_i = inv(U_ii), refined only in a build's last sweep, in
               // either mode (Udiag passed): earlier inverses only feed the next updates
         float x[4];
+        __syncwarp(m);   // the products' rows are read
         if (quad_inv4_refined(s, x, sh_q, Udiag != nullptr) && q == 0) atomicAdd(nsing, 1ull);
         st_row_sel<VOL>(Dout + (size_t)dst * BB + q * BS, x);
         if (Udiag) st_row_sel<false>(Udiag + (size_t)dst * BB + q * BS, s);
     }
+    __syncwarp(m);   // the scratch is free for the quad's next block
 }
 
 template <typename T>
@@ -396,12 +424,12 @@ __host__ __device__ __forceinline__ long long build_tickets(int nwork, int wchun
     return (nsub + per - 1) / per;
 }
 
-// Lists of at most SMALL_TICKET blocks per resident warp (6,080 warps at 40 per
-// SM: 389k blocks, 155k grid cells) take the smallest ticket of 8-block
+// Lists of at most SMALL_TICKET blocks per resident warp (7,296 warps at 48 per
+// SM: 467k blocks, 187k grid cells) take the smallest ticket of 8-block
 // sub-chunks that gives no more tickets than warps, so a sweep is at most one
 // ticket per warp.  Such lists are bound by the serial steps of a ticket: with
 // 128-block tickets a 20k-block list kept 160 warps busy for 16 dependent
-// steps per sweep.  Measured, 4 sweeps with the prepare pass (us, 128-block
+// steps per sweep.  Measured, 4 sweeps with the prepare pass, 40 warps per SM (us, 128-block
 // tickets -> this rule): 2.4k blocks 80 -> 30, 20k 91 -> 34, 82k 96 -> 53, 144k
 // 105 -> 68, 327k 149 -> 124; 8 sweeps of 326k (wall-normal coupling 100x) 231 ->
 // 178.  Above the line the 64-block groups win: 737k blocks 253 against 286.
@@ -412,7 +440,7 @@ __host__ __device__ __forceinline__ long long build_tickets(int nwork, int wchun
 constexpr int SMALL_TICKET = 64;
 
 template <typename T, bool ORDERED, int SUB>
-__global__ void __launch_bounds__(BUILD_THREADS, 5)   // 48 registers: measured fastest (4, 6 slower)
+__global__ void __launch_bounds__(BUILD_THREADS, 6)   // 40 registers; 512x512, 6 sweeps: 379 us (5: 398, 4: 428, 7: 416)
 k_build_blocks_async(PatternView P, const float *__restrict__ A32, T *L, T *U, T *D, T *Udiag,
                      int nsweeps, int max_warps, unsigned long long *nsing,
                      unsigned long long *ticket, unsigned long long *err, int *done,
@@ -712,12 +740,22 @@ __global__ void k_export(PatternView P, const T *__restrict__ L, const T *__rest
     if (X) {
         const int p0 = P.rowptr[i], p1 = P.rowptr[i + 1], dp = P.diagpos[i];
         const int lb = P.lrow[i], ub = P.urow[i];
-        for (int p = p0; p < p1; p++) {
-            double v[4];
-            if (p < dp) ld_row(L + (size_t)(lb + p - p0) * BB + q * BS, v);
-            else if (p > dp) ld_row(U + (size_t)(ub + p - dp - 1) * BB + q * BS, v);
-            else ld_row(Udiag + (size_t)i * BB + q * BS, v);
-            st_row(X + (size_t)p * BB + q * BS, v);
+        // four blocks of the row at a time, every load issued before any store
+        for (int pb = p0; pb < p1; pb += 4) {
+            typename BuildArith<T>::C v[4][4];
+#pragma unroll
+            for (int k = 0; k < 4; k++) {
+                const int p = pb + k;
+                if (p >= p1) break;
+                const T *src = p < dp ? L + (size_t)(lb + p - p0) * BB
+                               : p > dp ? U + (size_t)(ub + p - dp - 1) * BB : Udiag + (size_t)i * BB;
+                ld_row(src + q * BS, v[k]);
+            }
+#pragma unroll
+            for (int k = 0; k < 4; k++) {
+                if (pb + k >= p1) break;
+                st_row(X + (size_t)(pb + k) * BB + q * BS, v[k]);
+            }
         }
     }
     if (Dinv) {

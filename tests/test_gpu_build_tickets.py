@@ -6,10 +6,10 @@ import abilu_inputs as gen
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("nx,ny", [(1, 1), (2, 3), (98, 99), (99, 100), (278, 279), (280, 281)])
+@pytest.mark.parametrize("nx,ny", [(1, 1), (2, 3), (107, 108), (109, 108), (304, 306), (306, 307)])
 def test_default_tickets_reach_the_sequential_factors(nx, ny):
     """One block, a ragged last ticket, both sides of one step per warp (8
-    blocks on each of 6,080 resident warps) and of the line to 128-block
+    blocks on each of 7,296 resident warps) and of the line to 128-block
     tickets (64 blocks per warp): the in-place build reaches sequential block
     ILU(0).  The bound is the FP32 one of the other ticket sizes."""
     import torch
