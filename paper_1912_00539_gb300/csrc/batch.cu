@@ -11,7 +11,7 @@
 // the small ones across the GPU).  The padding makes every 64-row chunk belong
 // to one system, so the Krylov kernels below keep a separate FGMRES state per
 // system: per-system dot products and norms (each CTA of a reducing kernel
-// sums a run of up to 16 of one system's chunks, and the partials of a
+// sums a run of up to 8 of one system's chunks, and the partials of a
 // system's runs are summed in order by the last of them to finish),
 // per-system Hessenberg, Givens rotations and convergence.  The systems iterate
 // in lockstep; a system that has converged (or left its cycle) skips its
@@ -62,11 +62,14 @@ struct BConf {
 
 // The reducing kernels (residual, Gram-Schmidt dots, norms) give each CTA a
 // super-chunk: up to SUPER_CHUNKS consecutive 64-row chunks of one system, so
-// one block reduction covers up to 4,096 values (one per 256 values made the
+// one block reduction covers up to 2,048 values (one per 256 values made the
 // reductions' latency, not memory, bound those kernels).  A system's
 // super-chunks split its chunks from its first one, whatever its place in
-// the batch, so its reductions are the same alone and in any batch.
-constexpr int SUPER_CHUNKS = 16;
+// the batch, so its reductions are the same alone and in any batch.  Eight
+// chunks: the fused product and dots of 2.6 M rows take 334 us (16 chunks: 330,
+// 4: 357, 2: 446), those of a four-system server step, whose 16-chunk
+// super-chunks left one CTA per SM, 35 us (51, 37, 38).
+constexpr int SUPER_CHUNKS = 8;
 struct BTab {
     const int *sc_first;   // [nsc + 1] first chunk of each super-chunk
     const int *sc_sys;     // [nsc] its system
@@ -729,7 +732,7 @@ extern "C" abilu_status abilu_batch_counts(abilu_batch b, int64_t *out) {
 // ---- copies between the caller's arrays and the concatenation
 //
 // Up to COPY_SEGS arrays in one launch: one wave of CTAs takes tiles of 1,024
-// 16-byte words, four words in flight per thread.  (A copy-engine-free
+// 16-byte words, four words in flight per thread.  (A
 // cudaMemcpyAsync per array moved a 10 MB array at 2.3 TB/s, read and write
 // together, and cost a launch each; 64 systems set and read back, 2.8 GB: about
 // 1.2 -> 0.7 ms.)
