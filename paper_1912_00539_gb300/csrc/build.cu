@@ -637,6 +637,14 @@ k_build_async(PatternView P, const double *__restrict__ A, double *L, double *U,
     }
 }
 
+// The asynchronous sweeps' queue, reset by the prepare pass before them (two
+// memsets between the two kernels cost about 2 us each on the device)
+struct QueueInit {
+    unsigned long long *ticket;   // NULL: no asynchronous sweep follows
+    int *flags;                   // per ticket: completed sweeps (count 0: unordered)
+    int count, fill;
+};
+
 // Once per build, one pass over the FP64 A:
 //  * the constant blocks (U_ij, i < j, with no product pair: U_ij = A_ij in
 //    every sweep) go into U[cur] and, for synchronous builds, U[other];
@@ -650,9 +658,13 @@ __global__ void __launch_bounds__(BUILD_THREADS, sizeof(T) == 8 ? 3 : 4)
 k_build_prepare(PatternView P, const double *__restrict__ A, float *__restrict__ A32,
                 T *__restrict__ L, T *__restrict__ U, T *__restrict__ Uother, T *__restrict__ D,
                 T *__restrict__ Udiag, int init_all, const int *__restrict__ chunk_init,
-                unsigned long long *nsing) {
+                unsigned long long *nsing, QueueInit qi) {
     pdl_wait();
     pdl_trigger();
+    for (long long k = (long long)blockIdx.x * BUILD_THREADS + threadIdx.x; k < qi.count;
+         k += (long long)gridDim.x * BUILD_THREADS)
+        qi.flags[k] = qi.fill;
+    if (qi.ticket && blockIdx.x == 0 && threadIdx.x == 0) *qi.ticket = 0ull;
     // a CTA's 64 rows are one chunk of a server's arena (BUILD_ROWS = 64)
     const int init_from_a = chunk_init ? chunk_init[blockIdx.x] : init_all;
     __shared__ double sh_u[BuildShared<T>::D];
@@ -765,9 +777,56 @@ __global__ void k_export(PatternView P, const T *__restrict__ L, const T *__rest
     }
 }
 
+// Ticket size, warps and queue of an asynchronous block build
+struct AsyncPlan {
+    int wc, sub, warps;
+    QueueInit qi;
+};
+
+template <typename T>
+static abilu_status async_plan(abilu_factors f, AsyncPlan *plan) {
+    const PatternView &P = f->p->v;
+    static std::atomic<int> per_sm_cache{-1};
+    int dev = 0, sms = 0, per_sm = per_sm_cache.load(std::memory_order_relaxed);
+    cudaGetDevice(&dev);
+    if (per_sm < 0) {   // the ordered variant is held to the same occupancy
+        ABILU_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+            &per_sm, k_build_blocks_async<T, false, 64>, BUILD_THREADS, 0));
+        per_sm_cache.store(per_sm, std::memory_order_relaxed);
+    }
+    ABILU_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    int warps = per_sm * sms * (BUILD_THREADS / 32);
+    const int resident = warps > 0 ? warps : 1;
+    int wc = f->build_chunk ? f->build_chunk : WARP_CHUNK, sub = build_sub(wc);
+    if (!f->build_chunk && (long long)P.nwork <= (long long)SMALL_TICKET * resident) {
+        wc = (int)(((long long)P.nwork + 8LL * resident - 1) / (8LL * resident)) * 8;
+        sub = 8;
+    }
+    const int wchunks = (int)build_tickets(P.nwork, wc, sub);
+    if (warps > wchunks) warps = wchunks;
+    if (warps < 1) warps = 1;
+    plan->wc = wc;
+    plan->sub = sub;
+    plan->warps = warps;
+    plan->qi = QueueInit{f->ctr + 1, nullptr, 0, 0};
+    // fewer than 4 chunks per warp: keep each chunk's sweeps in order (see
+    // the kernel); with more, an overlap needs one warp stalled for the
+    // time the others take to process several chunks each
+    if ((long long)wchunks < 4LL * warps) {
+        // failure injection (tests of the bounded wait): every flag at -1,
+        // one sweep behind, which no warp ever publishes, so the first
+        // wait of every chunk runs out after the spin limit
+        plan->qi.flags = f->chunk_done;
+        plan->qi.count = wchunks;
+        plan->qi.fill = f->stall_flags ? -1 : 0;
+        f->stall_flags = 0;
+    }
+    return ABILU_OK;
+}
+
 template <typename T>
 static abilu_status block_sweeps_t(abilu_factors f, const float *A32, int nsweeps,
-                                   abilu_mode mode, cudaStream_t st) {
+                                   abilu_mode mode, const AsyncPlan &plan, cudaStream_t st) {
     const PatternView &P = f->p->v;
     const int grid = (P.nwork + WORK_PER_CTA - 1) / WORK_PER_CTA;
     T **L = reinterpret_cast<T **>(f->L), **U = reinterpret_cast<T **>(f->U);
@@ -783,40 +842,9 @@ static abilu_status block_sweeps_t(abilu_factors f, const float *A32, int nsweep
             f->cur = o;
         }
     } else {
-        static std::atomic<int> per_sm_cache{-1};
-        int dev = 0, sms = 0, per_sm = per_sm_cache.load(std::memory_order_relaxed);
-        cudaGetDevice(&dev);
-        if (per_sm < 0) {   // the ordered variant is held to the same occupancy
-            ABILU_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                &per_sm, k_build_blocks_async<T, false, 64>, BUILD_THREADS, 0));
-            per_sm_cache.store(per_sm, std::memory_order_relaxed);
-        }
-        ABILU_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        int warps = per_sm * sms * (BUILD_THREADS / 32);
-        const int resident = warps > 0 ? warps : 1;
-        int wc = f->build_chunk ? f->build_chunk : WARP_CHUNK, sub = build_sub(wc);
-        if (!f->build_chunk && (long long)P.nwork <= (long long)SMALL_TICKET * resident) {
-            wc = (int)(((long long)P.nwork + 8LL * resident - 1) / (8LL * resident)) * 8;
-            sub = 8;
-        }
-        const int wchunks = (int)build_tickets(P.nwork, wc, sub);
-        if (warps > wchunks) warps = wchunks;
-        if (warps < 1) warps = 1;
+        const int wc = plan.wc, sub = plan.sub, warps = plan.warps;
         const int ctas = (warps + BUILD_THREADS / 32 - 1) / (BUILD_THREADS / 32);
-        ABILU_CUDA(cudaMemsetAsync(f->ctr + 1, 0, sizeof(unsigned long long), st));
-        // fewer than 4 chunks per warp: keep each chunk's sweeps in order (see
-        // the kernel); with more, an overlap needs one warp stalled for the
-        // time the others take to process several chunks each
-        int *done = nullptr;
-        if ((long long)wchunks < 4LL * warps) {
-            done = f->chunk_done;
-            // failure injection (tests of the bounded wait): every flag at -1,
-            // one sweep behind, which no warp ever publishes, so the first
-            // wait of every chunk runs out after the spin limit
-            const int fill = f->stall_flags ? 0xff : 0;
-            f->stall_flags = 0;
-            ABILU_CUDA(cudaMemsetAsync(done, fill, sizeof(int) * (size_t)wchunks, st));
-        }
+        int *done = plan.qi.count > 0 ? plan.qi.flags : nullptr;
         const int c = f->cur;
         const unsigned long long lim = spin_limit_or_default(f->spin_limit);
         auto kern = sub == 8 ? k_build_blocks_async<T, true, 8>   // one ticket per warp: always ordered
@@ -862,7 +890,6 @@ static abilu_status sweeps_f64(abilu_factors f, const double *Asrc, int nsweeps,
         int ctas = per_sm * sms;
         if (ctas > grid) ctas = grid;
         if (ctas < 1) ctas = 1;
-        ABILU_CUDA(cudaMemsetAsync(f->ctr + 1, 0, sizeof(unsigned long long), st));
         const int c = f->cur;
         launch_pdl(k_build_async, ctas, BUILD_THREADS, 0, st, P, Asrc, L[c], U[c], D[c], Ud,
             nsweeps, f->ctr, f->ctr + 1);
@@ -892,16 +919,25 @@ static abilu_status build_t(abilu_factors f, const double *A, int nsweeps, abilu
     constexpr bool narrow = sizeof(T) < 8;
     float *A32 = narrow ? reinterpret_cast<float *>(f->A32) : nullptr;
     const int c = f->cur;
+    AsyncPlan plan = {};
+    if (mode == ABILU_ASYNC && nsweeps > 0) {
+        if constexpr (narrow) {
+            abilu_status s = P.nwork > 0 ? async_plan<T>(f, &plan) : ABILU_OK;
+            if (s != ABILU_OK) return s;
+        } else {
+            plan.qi.ticket = f->ctr + 1;
+        }
+    }
     // U_ii of the initial guess only when no sweep follows: the last sweep
     // stores the build's U_ii (33.5 MB fewer writes at 512x512)
     launch_pdl(k_build_prepare<T>, grid, BUILD_THREADS, 0, st,
         P, A, A32, L[c], U[c], mode == ABILU_SYNC ? U[1 - c] : nullptr, D[c], nsweeps > 0 ? nullptr : Ud,
-        init == ABILU_INIT_FROM_A ? 1 : 0, f->chunk_init, f->ctr);
+        init == ABILU_INIT_FROM_A ? 1 : 0, f->chunk_init, f->ctr, plan.qi);
     ABILU_LAUNCH_CHECK("k_build_prepare");
     if constexpr (narrow) {
         if (nsweeps > 0) {
             abilu_status s = timing_mark(f, 0, st);
-            if (s == ABILU_OK) s = block_sweeps_t<T>(f, A32, nsweeps, mode, st);
+            if (s == ABILU_OK) s = block_sweeps_t<T>(f, A32, nsweeps, mode, plan, st);
             if (s == ABILU_OK) s = timing_mark(f, 1, st);
             if (s != ABILU_OK) return s;
         }

@@ -73,6 +73,24 @@ __device__ __forceinline__ void publish(SolveState *S) {
     __threadfence_system();
 }
 
+// The singular-block and timed-out-wait counters of a solve's factors handles
+// into the host-mapped status, so the host reads them with the status after
+// its final stream synchronisation
+struct CtrList {
+    const unsigned long long *p[ABILU_MG_MAX_LEVELS];
+    int n;
+};
+__device__ __forceinline__ void publish_counters(HostStatus *hs, const CtrList &cl) {
+    unsigned long long ns = 0ull, nt = 0ull;
+    for (int k = 0; k < cl.n; k++) {
+        ns += cl.p[k][0];
+        nt += cl.p[k][4];
+    }
+    volatile HostStatus *vh = hs;
+    vh->nsing = ns;
+    vh->ntimeout = nt;
+}
+
 // In the first CTA of the kernel after a Gram-Schmidt step or a residual: that
 // kernel's status to the host-mapped mirror (see givens_column)
 __device__ __forceinline__ void publish_early(SolveState *S) {
@@ -227,9 +245,11 @@ __device__ __forceinline__ void zero_tickets(unsigned long long *tk) {
 // same into y0, the application's in-place iterate, when given)
 __global__ void __launch_bounds__(RED_THREADS)
 k_scale(const double *vin, double *vout, float *v32, long long nv2, SolveState *S, float *y0,
-        unsigned long long *tk) {
+        unsigned long long *tk, CtrList cl) {
     pdl_wait();
     pdl_trigger();
+    // at the end of a cycle (cl.n > 0) also the handles' counters
+    if (cl.n > 0 && blockIdx.x == 0 && threadIdx.x == 0) publish_counters(S->hs, cl);
     publish_early(S);      // the previous kernel's status (k_residual: a new cycle's)
     if (S->done) return;   // set by an earlier kernel: a plain load
     zero_tickets(tk);
@@ -853,7 +873,10 @@ static void launch_update(int nred, cudaStream_t st, const double *V, long long 
     }
 }
 
-// y = R^{-1} g (every CTA, redundantly, in shared memory), then x += Z y
+// y = R^{-1} g (every CTA, redundantly, in shared memory), then x += Z y, or
+// x = Z y (ASSIGN: the first cycle from a zero guess, so that x is neither
+// zeroed before the solve nor read here)
+template <bool ASSIGN>
 __global__ void __launch_bounds__(RED_THREADS)
 k_xupdate(const double *__restrict__ Z, long long nv2, double *__restrict__ x, SolveState *S) {
     pdl_wait();
@@ -861,7 +884,7 @@ k_xupdate(const double *__restrict__ Z, long long nv2, double *__restrict__ x, S
     __shared__ double y[MAXM];
     __shared__ double sR[MAXM * MAXM / 2 + MAXM], sg[MAXM], sinv[MAXM];   // R's upper triangle, g
     const int kd = S->kdim;
-    if (kd == 0) return;
+    if (!ASSIGN && kd == 0) return;
     // R and g into shared memory by the whole CTA (one round of loads), the
     // reciprocals of R's diagonal by kd threads at once, then the back
     // substitution by one thread from there: its chain of dependent FP64
@@ -889,7 +912,7 @@ k_xupdate(const double *__restrict__ Z, long long nv2, double *__restrict__ x, S
     double2 *x2 = reinterpret_cast<double2 *>(x);
     for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < nv2;
          e += (long long)gridDim.x * blockDim.x) {
-        double2 t = x2[e];
+        double2 t = ASSIGN ? make_double2(0.0, 0.0) : x2[e];
         for (int k = 0; k < kd; k++) {
             const double2 z = Z2[(size_t)k * nv2 + e];
             t.x += y[k] * z.x;
@@ -899,23 +922,25 @@ k_xupdate(const double *__restrict__ Z, long long nv2, double *__restrict__ x, S
     }
 }
 
-// the singular-block and timed-out-wait counters of one factors handle into
-// the host-mapped status (first: assign, else add), so the host reads them
-// with the status after its final stream synchronisation
-__global__ void k_counters(const unsigned long long *ctr, HostStatus *hs, int first) {
+// the counters into the status by themselves (a solve that ended early)
+__global__ void k_counters(SolveState *S, CtrList cl) {
     if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    volatile HostStatus *vh = hs;
-    vh->nsing = (first ? 0ull : vh->nsing) + ctr[0];
-    vh->ntimeout = (first ? 0ull : vh->ntimeout) + ctr[4];
+    publish_counters(S->hs, cl);
     __threadfence_system();
 }
 
+// The solve state at its start: the fields read before a kernel writes them
 __global__ void k_solve_init(SolveState *S, HostStatus *hs, double rtol, int max_iters, int m) {
+    pdl_wait();
+    pdl_trigger();
     if (threadIdx.x != 0 || blockIdx.x != 0) return;
     S->rtol = rtol;
     S->max_iters = max_iters;
     S->m = m;
     S->hs = hs;
+    S->bnorm = S->beta = S->hn_inv = S->est = 0.0;
+    S->done = S->iters = S->converged = S->kdim = S->restarts = S->breakdown = 0;
+    S->counter = 0;
 }
 
 }  // namespace abilu
@@ -986,21 +1011,25 @@ abilu_status fgmres_run(const PatternView &P, const double *A, abilu_factors ws,
     SolveState *SS = reinterpret_cast<SolveState *>(ws->scal);
     HostStatus *hs = reinterpret_cast<HostStatus *>(ws->host_status);
     const int nred = red_ctas();
-    const int nres = nred / 4 * 3;   // k_residual: 3 CTAs per SM
+    // k_residual, k_spmv_dots: 3 CTAs per SM in one wave, no CTA without rows (a
+    // small system's reductions then add few partials)
+    const int chunks = (P.n + RED_THREADS / 4 - 1) / (RED_THREADS / 4);
+    const int nres = chunks < nred / 4 * 3 ? chunks : nred / 4 * 3;
     const Skip skip{&SS->done, nullptr, nullptr};
     float *v32 = pc.v32;
     const int form = gs_form_for(opts->reorth, opts->rtol);
 
-    ABILU_CUDA(cudaMemsetAsync(SS, 0, sizeof(SolveState), st));
-    k_solve_init<<<counted(1), 1, 0, st>>>(SS, hs, opts->rtol, opts->max_iters, m);
-    if (opts->zero_guess) ABILU_CUDA(cudaMemsetAsync(x, 0, sizeof(double) * nv, st));
+    CtrList cl = {}, none = {};
+    for (int k = 0; k < ncnt; k++) cl.p[k] = cnt[k]->ctr;
+    cl.n = ncnt;
+    launch_pdl(k_solve_init, 1, 32, 0, st, SS, hs, opts->rtol, opts->max_iters, m);
     if (opts->zero_guess)
         launch_pdl(k_residual<true>, nres, RED_THREADS, 0, st, P, A, b, x, V, SS, ws->partials, 1);
     else
         launch_pdl(k_residual<false>, nres, RED_THREADS, 0, st, P, A, b, x, V, SS, ws->partials, 1);
     // v_0 = r / beta; with x = 0, r = b is read from b itself
     launch_pdl(k_scale, nred, RED_THREADS, 0, st, opts->zero_guess ? b : V, V, v32, nv2, SS,
-               pc.y0, pc.tickets);
+               pc.y0, pc.tickets, none);
     ABILU_LAUNCH_CHECK("fgmres init");
     // the look-ahead events live in the workspace handle (made on first use)
     for (int k = 0; k < 2; k++)
@@ -1032,13 +1061,13 @@ abilu_status fgmres_run(const PatternView &P, const double *A, abilu_factors ws,
             } else if (form == GS_CLASSICAL) {  // one pass, the norm of the updated w
                 launch_update(nred, st, V, nv2, j, w, SS, ws->partials, 0, 1);
                 launch_pdl(k_scale, nred, RED_THREADS, 0, st, w, V + (size_t)(j + 1) * nv, v32, nv2, SS,
-                           pc.y0, pc.tickets);
+                           pc.y0, pc.tickets, none);
             } else {               // CGS2: two passes, the norm of the updated w
                 launch_update(nred, st, V, nv2, j, w, SS, ws->partials, 0, 0);
                 launch_dots(nred, st, V, nv2, j + 1, w, SS, ws->partials, 1);
                 launch_update(nred, st, V, nv2, j, w, SS, ws->partials, 1, 1);
                 launch_pdl(k_scale, nred, RED_THREADS, 0, st, w, V + (size_t)(j + 1) * nv, v32, nv2, SS,
-                           pc.y0, pc.tickets);
+                           pc.y0, pc.tickets, none);
             }
             cudaError_t e = cudaGetLastError();
             if (e != cudaSuccess) { ret = cuda_fail(e, "fgmres step"); break; }
@@ -1065,13 +1094,12 @@ abilu_status fgmres_run(const PatternView &P, const double *A, abilu_factors ws,
             }
         }
         if (ret != ABILU_OK) break;
-        launch_pdl(k_xupdate, nred, RED_THREADS, 0, st, Z, nv2, x, SS);
+        if (first && opts->zero_guess) launch_pdl(k_xupdate<true>, nred, RED_THREADS, 0, st, Z, nv2, x, SS);
+        else launch_pdl(k_xupdate<false>, nred, RED_THREADS, 0, st, Z, nv2, x, SS);
         launch_pdl(k_residual<false>, nres, RED_THREADS, 0, st, P, A, b, x, V, SS, ws->partials, 0);
-        launch_pdl(k_scale, nred, RED_THREADS, 0, st, V, V, v32, nv2, SS, pc.y0, pc.tickets);
-        // the handles' counters into the status with every cycle's result, so
+        // the handles' counters go into the status with every cycle's result, so
         // the synchronisation that ends the last cycle also ends the solve
-        for (int k = 0; k < ncnt; k++)
-            k_counters<<<counted(1), 32, 0, st>>>(cnt[k]->ctr, hs, k == 0);
+        launch_pdl(k_scale, nred, RED_THREADS, 0, st, V, V, v32, nv2, SS, pc.y0, pc.tickets, cl);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) { ret = cuda_fail(e, "fgmres restart"); break; }
         e = cudaStreamSynchronize(st);
@@ -1082,8 +1110,7 @@ abilu_status fgmres_run(const PatternView &P, const double *A, abilu_factors ws,
     if (zero_b)  // b = 0: the solution is x = 0
         ABILU_CUDA(cudaMemsetAsync(x, 0, sizeof(double) * nv, st));
     if (ret != ABILU_OK || zero_b) {   // a cycle that did not finish, or the memset
-        for (int k = 0; k < ncnt; k++)
-            k_counters<<<counted(1), 32, 0, st>>>(cnt[k]->ctr, hs, k == 0);
+        k_counters<<<counted(1), 32, 0, st>>>(SS, cl);
         cudaStreamSynchronize(st);
         h = read_status(hs);
     }
