@@ -60,10 +60,10 @@ __device__ __forceinline__ VT dot4(const VT a[4], const VT b[4]) {
 // VOL: the vector is being updated in place by other threads.  (Prefetching
 // the row's blocks before the arithmetic was measured slower here: the extra
 // registers cost more occupancy than the shorter dependency chain gained.)
-template <bool VOL, typename T, typename VT>
+template <bool VOL, typename T, typename VT, typename R>
 __device__ __forceinline__ VT row_sweep_sum(VT s, const T *__restrict__ F,
                                             const int32_t *__restrict__ col, int l0, int l1,
-                                            const VT *v) {
+                                            const R *v) {
     const int q = threadIdx.x & 3;
     for (int l = l0; l < l1; l++) {
         VT a[4], b[4];
@@ -130,12 +130,22 @@ __device__ __forceinline__ void st_result(double *z, size_t o, double v, int zad
     z[o] = zadd ? z[o] + v : v;
 }
 
+// The right-hand side of an application called with FP64 vectors (R = double) on
+// FP32/BF16 factors is rounded where its first kernel reads it, and that kernel
+// leaves the FP32 copy the later sweeps read in r32 (a conversion pass of its
+// own cost 2.7 us of a 31 us application on 130k cells).
+template <typename VT> __device__ __forceinline__ VT ld_rhs(const VT *r, size_t o) { return r[o]; }
+template <typename VT>
+__device__ __forceinline__ VT ld_rhs(const std::conditional_t<sizeof(VT) == 4, double, float> *r, size_t o) {
+    return (VT)to_f32_int((double)r[o]);
+}
+
 // one Jacobi lower sweep; optionally x^1 = Dinv y fused (into x1 or, when
 // it is the last upper result, into z as FP64)
-template <typename T, typename VT>
+template <typename T, typename VT, typename R = VT>
 __global__ void __launch_bounds__(APPLY_THREADS)
-k_lower_sync(PatternView P, const T *__restrict__ L, const VT *__restrict__ r,
-             const VT *__restrict__ yin, VT *__restrict__ yout, const T *__restrict__ D,
+k_lower_sync(PatternView P, const T *__restrict__ L, const R *__restrict__ r, VT *__restrict__ r32,
+             const R *__restrict__ yin, VT *__restrict__ yout, const T *__restrict__ D,
              VT *__restrict__ x1, double *__restrict__ z, int zadd, Skip skip) {
     pdl_wait();
     pdl_trigger();
@@ -144,7 +154,9 @@ k_lower_sync(PatternView P, const T *__restrict__ L, const VT *__restrict__ r,
     int l0, l1;
     const int i = sweep_row<VT>(P.lrow, blockIdx.x * APPLY_ROWS, P.n, l0, l1);
     if (i >= P.n) return;
-    const VT s = row_sweep_sum<false>(r[(size_t)i * BS + q], L, P.lcol, l0, l1, yin);
+    const VT b = ld_rhs<VT>(r, (size_t)i * BS + q);
+    if (r32) r32[(size_t)i * BS + q] = b;
+    const VT s = row_sweep_sum<false>(b, L, P.lcol, l0, l1, yin);
     if (yout) yout[(size_t)i * BS + q] = s;
     if (x1 || z) {
         VT x = dinv_times<T, VT>(D, i, s);
@@ -154,16 +166,17 @@ k_lower_sync(PatternView P, const T *__restrict__ L, const VT *__restrict__ r,
 }
 
 // x^1 = Dinv y (used when fewer than two lower sweeps run)
-template <typename T, typename VT>
+template <typename T, typename VT, typename R = VT>
 __global__ void __launch_bounds__(APPLY_THREADS)
-k_diag_apply(PatternView P, const T *__restrict__ D, const VT *__restrict__ y,
+k_diag_apply(PatternView P, const T *__restrict__ D, const R *__restrict__ y, VT *__restrict__ r32,
              VT *__restrict__ x1, double *__restrict__ z, int zadd, Skip skip) {
     pdl_wait();
     pdl_trigger();
     if (skip_all(skip) || skip_chunk(skip, blockIdx.x)) return;
     const int i = blockIdx.x * APPLY_ROWS + (threadIdx.x >> 2), q = threadIdx.x & 3;
     if (i >= P.n) return;
-    VT t = y[(size_t)i * BS + q];
+    VT t = ld_rhs<VT>(y, (size_t)i * BS + q);
+    if (r32) r32[(size_t)i * BS + q] = t;
     VT x = dinv_times<T, VT>(D, i, t);
     if (x1) x1[(size_t)i * BS + q] = x;
     if (z) st_result(z, (size_t)i * BS + q, to_f64v(x), zadd);
@@ -241,9 +254,9 @@ k_lower_async(PatternView P, const T *__restrict__ L, const VT *__restrict__ r, 
 // First update of the asynchronous application: y = b, and when no further
 // lower sweep runs also x^1 = Dinv b (into x1 or z); resets the two ticket
 // counters of the in-place kernels that follow.
-template <typename T, typename VT>
+template <typename T, typename VT, typename R = VT>
 __global__ void __launch_bounds__(APPLY_THREADS)
-k_async_start(PatternView P, const T *__restrict__ D, const VT *__restrict__ r,
+k_async_start(PatternView P, const T *__restrict__ D, const R *__restrict__ r, VT *__restrict__ r32,
               VT *__restrict__ y, VT *__restrict__ x1, VT *__restrict__ yh, double *__restrict__ z,
               int zadd, unsigned long long *tickets, Skip skip) {
     pdl_wait();
@@ -253,7 +266,8 @@ k_async_start(PatternView P, const T *__restrict__ D, const VT *__restrict__ r,
     if (skip_chunk(skip, blockIdx.x)) return;
     const int i = blockIdx.x * APPLY_ROWS + (threadIdx.x >> 2), q = threadIdx.x & 3;
     if (i >= P.n) return;
-    const VT b = r[(size_t)i * BS + q];
+    const VT b = ld_rhs<VT>(r, (size_t)i * BS + q);
+    if (r32) r32[(size_t)i * BS + q] = b;
     y[(size_t)i * BS + q] = b;
     if (x1 || z) {
         const VT x = dinv_times<T, VT>(D, i, b);
@@ -485,17 +499,6 @@ k_tri_staged(PatternView P, const T *__restrict__ F, const T *__restrict__ D,
     }
 }
 
-// r32 = (float) r, once per application (the sweeps then read 16-byte FP32
-// rows and do no FP64 conversions on the slow FP64 pipe)
-__global__ void __launch_bounds__(APPLY_THREADS)
-k_to_f32(const double *__restrict__ r, float *__restrict__ r32, long long n4) {
-    const long long e = ((long long)blockIdx.x * blockDim.x + threadIdx.x) * 4;
-    if (e >= n4) return;
-    double v[4];
-    ld_row(r + e, v);
-    st_row(r32 + e, v);
-}
-
 // v = 0 (n values) unless the launch is skipped: the zero initial guess of the
 // in-place sweeps, as a kernel so that a skipped FGMRES step costs no memset
 template <typename VT>
@@ -549,20 +552,16 @@ static abilu_status apply_t(abilu_factors f, const double *r, const float *r32_i
     VT *x[2] = {reinterpret_cast<VT *>(f->x[0]), reinterpret_cast<VT *>(f->x[1])};
     const int grid = (P.n + APPLY_ROWS - 1) / APPLY_ROWS;
 
-    // right-hand side in the compute type
+    // right-hand side in the compute type: `conv` while it is still to be
+    // rounded into r32 by the first kernel
+    const bool conv = sizeof(VT) == 4 && !r32_in;
     const VT *rv;
+    VT *r32 = nullptr;
     if constexpr (sizeof(VT) == 8) {
         rv = r;
     } else {
-        if (r32_in) {
-            rv = r32_in;
-        } else {
-            const long long n4 = (long long)P.n * BS;
-            k_to_f32<<<counted((int)((n4 / 4 + APPLY_THREADS - 1) / APPLY_THREADS)), APPLY_THREADS,
-                       0, st>>>(r, reinterpret_cast<float *>(f->r32), n4);
-            ABILU_LAUNCH_CHECK("k_to_f32");
-            rv = reinterpret_cast<const float *>(f->r32);
-        }
+        r32 = reinterpret_cast<float *>(f->r32);
+        rv = conv ? r32 : r32_in;
     }
 
     // FP32 factors: upper sweeps on Us = Dinv U with right-hand side yh = Dinv y
@@ -584,9 +583,14 @@ static abilu_status apply_t(abilu_factors f, const double *r, const float *r32_i
         VT *yh = SC && nu >= 2 ? y[1] : nullptr;
         double *z1 = nu == 1 ? z : nullptr;
         if (!(y_ready && sizeof(VT) == 4 && nl >= 2)) {
-            launch_pdl(k_async_start<T, VT>, grid, APPLY_THREADS, 0, st,
-                P, D, rv, y[0], nl == 1 ? x1 : nullptr, nl == 1 ? yh : nullptr, nl == 1 ? z1 : nullptr,
-                zadd, tk, skip);
+            if (conv)
+                launch_pdl(k_async_start<T, VT, double>, grid, APPLY_THREADS, 0, st,
+                    P, D, r, r32, y[0], nl == 1 ? x1 : nullptr, nl == 1 ? yh : nullptr,
+                    nl == 1 ? z1 : nullptr, zadd, tk, skip);
+            else
+                launch_pdl(k_async_start<T, VT>, grid, APPLY_THREADS, 0, st,
+                    P, D, rv, nullptr, y[0], nl == 1 ? x1 : nullptr, nl == 1 ? yh : nullptr,
+                    nl == 1 ? z1 : nullptr, zadd, tk, skip);
             ABILU_LAUNCH_CHECK("k_async_start");
         }
         unsigned long long *err = f->ctr + 4;
@@ -631,8 +635,12 @@ static abilu_status apply_t(abilu_factors f, const double *r, const float *r32_i
     const VT *xfirst;   // x^1
     if (nl == 1) {      // no lower sweep runs: x^1 = Dinv r
         VT *x1 = nu >= 2 ? (SC ? y[0] : x[1]) : nullptr;
-        launch_pdl(k_diag_apply<T, VT>, grid, APPLY_THREADS, 0, st, P, D, rv, x1,
-            nu == 1 ? z : nullptr, zadd, skip);
+        if (conv)
+            launch_pdl(k_diag_apply<T, VT, double>, grid, APPLY_THREADS, 0, st, P, D, r, r32, x1,
+                nu == 1 ? z : nullptr, zadd, skip);
+        else
+            launch_pdl(k_diag_apply<T, VT>, grid, APPLY_THREADS, 0, st, P, D, rv, nullptr, x1,
+                nu == 1 ? z : nullptr, zadd, skip);
         ABILU_LAUNCH_CHECK("k_diag_apply");
         yfin = SC ? y[0] : rv;
         xfirst = x1;
@@ -644,8 +652,13 @@ static abilu_status apply_t(abilu_factors f, const double *r, const float *r32_i
             VT *yout = y[s & 1];
             if (last) x1 = nu >= 2 ? (SC ? yout : x[1]) : nullptr;
             // (the staged form was measured slower for this sweep: 19.3 vs 17.1 us)
-            launch_pdl(k_lower_sync<T, VT>, grid, APPLY_THREADS, 0, st,
-                P, L, rv, yprev, (last && SC) ? nullptr : yout, D, last ? x1 : nullptr,
+            if (conv && s == 2)
+                launch_pdl(k_lower_sync<T, VT, double>, grid, APPLY_THREADS, 0, st,
+                    P, L, r, r32, r, (last && SC) ? nullptr : yout, D, last ? x1 : nullptr,
+                    (last && nu == 1) ? z : nullptr, zadd, skip);
+            else
+                launch_pdl(k_lower_sync<T, VT>, grid, APPLY_THREADS, 0, st,
+                P, L, rv, nullptr, yprev, (last && SC) ? nullptr : yout, D, last ? x1 : nullptr,
                 (last && nu == 1) ? z : nullptr, zadd, skip);
             ABILU_LAUNCH_CHECK("lower sync");
             yprev = yout;
