@@ -82,8 +82,8 @@ k_block_norm2(const double *__restrict__ A, long long nnzb, double *__restrict__
 // Up to four fine blocks are loaded before they are added (in list order), so
 // the gathers of a coarse block overlap instead of forming a chain.
 //
-// The records are sorted by list length (stable, so neighbours in memory stay
-// close): an FP64 add holds this GPU's FP64 pipe for 16 cycles whatever lanes
+// The records are sorted by list length, longest first (a long list started last
+// ran alone at the end; stable, so neighbours in memory stay close): an FP64 add holds this GPU's FP64 pipe for 16 cycles whatever lanes
 // are active, and with the coarse blocks in storage order the eight quads of a
 // warp waited for its one diagonal block's ten or so entries.  The first entry
 // starts the sum (one add per entry fewer).  512x512 cells x 2, finest level
@@ -99,11 +99,17 @@ k_galerkin(long long nnzb_c, const int4 *__restrict__ grec, const int *__restric
     const int4 rec = __ldg(grec + k);
     double s[4] = {0.0, 0.0, 0.0, 0.0};
     const int t1 = rec.y + rec.z;
+    int g[4];   // the next four entries, read one round ahead
+#pragma unroll
+    for (int u = 0; u < 4; u++) g[u] = rec.y + u < t1 ? __ldg(gidx + rec.y + u) : 0;
     for (int t = rec.y; t < t1; t += 4) {
         double v[4][4];
 #pragma unroll
         for (int u = 0; u < 4; u++)
-            if (t + u < t1) ld_row(A + (size_t)__ldg(gidx + t + u) * BB + q * BS, v[u]);
+            if (t + u < t1) ld_row(A + (size_t)g[u] * BB + q * BS, v[u]);
+#pragma unroll
+        for (int u = 0; u < 4; u++)
+            if (t + 4 + u < t1) g[u] = __ldg(gidx + t + 4 + u);
 #pragma unroll
         for (int u = 0; u < 4; u++)
             if (t + u < t1) {
@@ -332,14 +338,14 @@ static void coarse_host(int n, const std::vector<int> &rowptr, const std::vector
         std::vector<int> pos(gptr.begin(), gptr.end() - 1);
         for (long long p = 0; p < nnzb; p++) c.gidx[pos[cpos[p]]++] = (int)p;
     }
-    // the records of k_galerkin: a stable counting sort by list length
+    // the records of k_galerkin: a stable counting sort, longest lists first
     std::vector<int> at(longest + 2, 0);
-    for (int k = 0; k < nnzc; k++) at[gptr[k + 1] - gptr[k] + 1]++;
+    for (int k = 0; k < nnzc; k++) at[longest - (gptr[k + 1] - gptr[k]) + 1]++;
     for (int l = 0; l <= longest; l++) at[l + 1] += at[l];
     c.grec.resize(nnzc);
     for (int k = 0; k < nnzc; k++) {
         const int len = gptr[k + 1] - gptr[k];
-        c.grec[at[len]++] = make_int4(k, gptr[k], len, 0);
+        c.grec[at[longest - len]++] = make_int4(k, gptr[k], len, 0);
     }
 }
 
