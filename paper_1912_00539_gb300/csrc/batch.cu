@@ -77,13 +77,7 @@ struct BTab {
 };
 
 __device__ __forceinline__ bool last_cta_of(BState *St, int nck) {
-    __shared__ bool am_last;
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) am_last = atomicAdd(&St->counter, 1u) == (unsigned)(nck - 1);
-    __syncthreads();
-    if (am_last) __threadfence();
-    return am_last;
+    return last_arrival(&St->counter, (unsigned)nck);
 }
 
 // sum over the system's chunks c0..c1-1 (in this order per thread, then a
@@ -309,6 +303,14 @@ k_b_update(const double *__restrict__ V, size_t nv, int j, double *__restrict__ 
     b_givens(St, s, j, pass == 1, sqrt(sh_o[0]), cf, hs_done, sys_done, bflag);
 }
 
+// system s is out of the current cycle
+__device__ __forceinline__ void b_leave_cycle(int s, int *hs_done, int *sys_done, int *bflag) {
+    sys_done[s] = 1;
+    if (atomicSub(bflag + 1, 1) == 1) bflag[0] = 1;  // the last active system left
+    reinterpret_cast<volatile int *>(hs_done)[s] = 1;
+    __threadfence_system();
+}
+
 // The Givens update of system s's column j with h_{j+1,j} = hn, its estimate
 // and cycle-end test (one thread of the system's last CTA)
 __device__ __forceinline__ void b_givens(BState *St, int s, int j, int two_pass, double hn,
@@ -342,36 +344,32 @@ __device__ __forceinline__ void b_givens(BState *St, int s, int j, int two_pass,
                 St->iters >= cf.max_iters || j + 1 >= cf.m) ? 1 : 0;
     St->hn_inv = hn != 0.0 ? 1.0 / hn : 0.0;
     St->counter = 0;
-    if (St->done) {
-        sys_done[s] = 1;
-        if (atomicSub(bflag + 1, 1) == 1) bflag[0] = 1;  // the last active system left
-        reinterpret_cast<volatile int *>(hs_done)[s] = 1;
-        __threadfence_system();
-    }
+    if (St->done) b_leave_cycle(s, hs_done, sys_done, bflag);
 }
 
 // The system's last CTA of a single-reduction step: h[k], k <= j, and ||w||^2
-// (slot BMAXM + 1) from the partials of super-chunks c0..c1-1, then
-// h_{j+1,j} = sqrt(||w||^2 - sum h_k^2) (a difference below 1e-12 ||w||^2 is a
-// breakdown) and the Givens update
+// (slot j + 1) from the partials of super-chunks c0..c1-1, then h_{j+1,j} and
+// the Givens update (givens_update).  sh_w holds RED_THREADS * BTILE doubles.
+static_assert(GIVENS_MAX == BMAXM, "one leading dimension");
 __device__ __forceinline__ void b_dots_norm_last(BState *St, int s, int j, const double *partials,
                                                  int c0, int c1, double *sh_w, double *sh_o,
                                                  const BConf &cf, int *hs_done, int *sys_done,
                                                  int *bflag) {
-    const int jp1 = j + 1;
-    for (int k0 = 0; k0 < jp1; k0 += BTILE) {
-        const int kn = jp1 - k0 < BTILE ? jp1 - k0 : BTILE;
+    __shared__ GivensIn G;
+    givens_stage(St, j, &G);
+    const int vals = j + 2;
+    for (int k0 = 0; k0 < vals; k0 += BTILE) {
+        const int kn = vals - k0 < BTILE ? vals - k0 : BTILE;
         reduce_sys<BTILE, PSTRIDE>(partials, c0, c1, k0, kn, sh_w, sh_o);
-        if (threadIdx.x < kn) St->h[k0 + threadIdx.x] = sh_o[threadIdx.x];
+        const int k = k0 + threadIdx.x;
+        if (threadIdx.x < kn) {
+            if (k <= j) St->h[k] = G.h[k] = sh_o[threadIdx.x];
+            else G.ww = sh_o[threadIdx.x];
+        }
         __syncthreads();
     }
-    reduce_sys<1, PSTRIDE>(partials, c0, c1, BMAXM + 1, 1, sh_w, sh_o);
-    if (threadIdx.x != 0) return;
-    const double ww = sh_o[0];
-    double hh = 0.0;
-    for (int k = 0; k < jp1; k++) hh = fma(St->h[k], St->h[k], hh);
-    const double d = ww - hh;
-    b_givens(St, s, j, 0, d > 1e-12 * ww ? sqrt(d) : 0.0, cf, hs_done, sys_done, bflag);
+    if (givens_update(St, j, &G, cf.rtol, cf.max_iters, cf.m))
+        b_leave_cycle(s, hs_done, sys_done, bflag);
 }
 
 // w = A z for the super-chunk's rows (a quad of threads per block row, one
@@ -384,7 +382,8 @@ template <int KF, bool NORM>
 __device__ __forceinline__ void b_spmv_tile(const PatternView &P, const double *__restrict__ A,
                                             const double *__restrict__ z, double *w,
                                             const double *__restrict__ V, size_t nv, int c0, int c1,
-                                            double *sh_w, double *sh_o, double *partials, int sc) {
+                                            double *sh_w, double *sh_o, double *partials, int sc,
+                                            int nslot) {
     constexpr int KA = KF + (NORM ? 1 : 0);
     double acc[KA];
 #pragma unroll
@@ -404,7 +403,7 @@ __device__ __forceinline__ void b_spmv_tile(const PatternView &P, const double *
     }
     block_sum<KA>(acc, sh_w, sh_o, KA);
     if (threadIdx.x < KF) partials[(size_t)sc * PSTRIDE + threadIdx.x] = sh_o[threadIdx.x];
-    if (NORM && threadIdx.x == 0) partials[(size_t)sc * PSTRIDE + BMAXM + 1] = sh_o[KF];
+    if (NORM && threadIdx.x == 0) partials[(size_t)sc * PSTRIDE + nslot] = sh_o[KF];   // ||w||^2
 }
 
 // The Arnoldi product of the batch fused with the first Gram-Schmidt pass (the
@@ -434,9 +433,9 @@ k_b_spmv_dots(PatternView P, const double *__restrict__ A, const double *__restr
     const int jp1 = j + 1;
     const int f0 = T.sc_first[sc], f1 = T.sc_first[sc + 1];
     switch (jp1 < B_FUSED ? jp1 : B_FUSED) {
-    case 1: b_spmv_tile<1, NORM>(P, A, z, w, V, nv, f0, f1, sh_w, sh_o, partials, sc); break;
-    case 2: b_spmv_tile<2, NORM>(P, A, z, w, V, nv, f0, f1, sh_w, sh_o, partials, sc); break;
-    default: b_spmv_tile<3, NORM>(P, A, z, w, V, nv, f0, f1, sh_w, sh_o, partials, sc); break;
+    case 1: b_spmv_tile<1, NORM>(P, A, z, w, V, nv, f0, f1, sh_w, sh_o, partials, sc, jp1); break;
+    case 2: b_spmv_tile<2, NORM>(P, A, z, w, V, nv, f0, f1, sh_w, sh_o, partials, sc, jp1); break;
+    default: b_spmv_tile<3, NORM>(P, A, z, w, V, nv, f0, f1, sh_w, sh_o, partials, sc, jp1); break;
     }
     if (jp1 > B_FUSED) b_dots_tiles<true>(V, nv, jp1, w, f0, f1, sh_w, sh_o, partials, sc, B_FUSED);
     const int c0 = T.sys_sc0[s], c1 = T.sys_sc0[s + 1];

@@ -97,16 +97,7 @@ __device__ __forceinline__ void publish_early(SolveState *S) {
     if (blockIdx.x == 0 && threadIdx.x == 0) publish(S);
 }
 
-// last-CTA election after this CTA stored its partials
-__device__ __forceinline__ bool last_cta(SolveState *S) {
-    __shared__ bool am_last;
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) am_last = atomicAdd(&S->counter, 1u) == gridDim.x - 1;
-    __syncthreads();
-    if (am_last) __threadfence();
-    return am_last;
-}
+__device__ __forceinline__ bool last_cta(SolveState *S) { return last_arrival(&S->counter, gridDim.x); }
 
 // In the last CTA: out[k] = sum over CTAs c of partials[c*stride + k0 + k],
 // k < kn <= TILE.  Thread t adds the partials of CTAs t, t+256, ... in that
@@ -390,66 +381,6 @@ __device__ __forceinline__ void givens_column(SolveState *S, int j, int two_pass
     if (pub) publish(S);
 }
 
-// What givens_column reads of the solve state besides the new column, staged
-// in shared memory by the last CTA of a reduction while it reduces the
-// partials, so that the serial FP64 chain of one thread reads no global
-// memory (an FP64 operation takes 64 cycles on this GPU and an L2 load
-// several hundred; with the loads in the chain the update took 4-9 us)
-struct GivensIn {
-    double cs[MAXM], sn[MAXM], gj, bnorm, rtol;
-    int iters, max_iters, m;
-};
-__device__ __forceinline__ void givens_stage(const SolveState *S, int j, GivensIn *G) {
-    for (int i = threadIdx.x; i < j; i += blockDim.x) {
-        G->cs[i] = S->cs[i];
-        G->sn[i] = S->sn[i];
-    }
-    switch (threadIdx.x) {
-    case 0: G->gj = S->g[j]; break;
-    case 1: G->bnorm = S->bnorm; break;
-    case 2: G->rtol = S->rtol; break;
-    case 3: G->iters = S->iters; break;
-    case 4: G->max_iters = S->max_iters; break;
-    case 5: G->m = S->m; break;
-    default: break;
-    }
-}
-
-// givens_column (one pass, the status published by the next kernel) from the
-// staged inputs and the coefficients h[0..j] in shared memory: the same
-// operations in the same order, so the same results bit for bit
-__device__ __forceinline__ void givens_column_staged(SolveState *S, int j, const double *h,
-                                                     const GivensIn *G, double hn) {
-    // independent of the rotations: overlaps their chain
-    S->hn_inv = hn != 0.0 ? 1.0 / hn : 0.0;
-    double a = h[0];
-    for (int i = 0; i < j; i++) {
-        const double c = h[i + 1];
-        S->H[i * MAXM + j] = G->cs[i] * a + G->sn[i] * c;
-        a = -G->sn[i] * a + G->cs[i] * c;
-    }
-    const double c = hn;
-    const double d = sqrt(a * a + c * c);
-    double cs = 1.0, sn = 0.0;
-    if (d != 0.0) { cs = a / d; sn = c / d; }
-    S->cs[j] = cs;
-    S->sn[j] = sn;
-    S->H[j * MAXM + j] = cs * a + sn * c;
-    const double gj = G->gj;
-    const double g1 = -sn * gj;
-    S->g[j + 1] = g1;
-    S->g[j] = cs * gj;
-    const int iters = G->iters + 1;
-    S->iters = iters;
-    S->kdim = j + 1;
-    S->est = fabs(g1) / G->bnorm;
-    S->breakdown = hn == 0.0 ? 1 : 0;
-    S->done = (fabs(g1) <= G->rtol * G->bnorm || hn == 0.0 || iters >= G->max_iters ||
-               j + 1 >= G->m) ? 1 : 0;
-    S->counter = 0;
-}
-
-
 // The last CTA of a dot-product pass: h[k] = sum over CTAs of the partials of
 // slot k, k < jp1, in tiles of T (pass 0 -> S->h, pass 1 -> S->h2).  sh_w
 // holds RED_THREADS * T doubles.
@@ -471,19 +402,16 @@ __device__ __forceinline__ void dots_last(SolveState *S, const double *partials,
 // of slots k < jp1 and ||w||^2 (slot jp1) reduced in tiles of T, the last tile
 // with the norm; the Givens inputs staged while the partials are reduced;
 // every thread's partials loaded before any add (R CTAs per thread in one
-// round); then h_{j+1,j} = sqrt(||w||^2 - sum_k h_k^2) (Pythagoras: w - V h is
-// orthogonal to V_0..V_j when they are orthonormal, so the norm needs neither
-// a pass over the updated w nor a second reduction) and the Givens update of
-// column j by one thread.  sh_w holds RED_THREADS * (T + 1) doubles.  A
-// difference below 1e-12 ||w||^2 (more than twelve digits cancelled, or
-// negative) is taken as a breakdown: the cycle ends at this column and the
-// explicit FP64 residual at its end decides whether it restarts.
+// round); then the Givens update of column j (givens_update).  sh_w holds
+// RED_THREADS * (T + 1) doubles.  The next kernel publishes the status.
+static_assert(GIVENS_MAX == MAXM, "one leading dimension");
 template <int T>
 __device__ __forceinline__ void dots_norm_last(SolveState *S, const double *partials, int jp1,
                                                double *sh_w, double *sh_o) {
     __shared__ GivensIn G;
-    __shared__ double sh_h[MAXM + 1], sh_ww;
     givens_stage(S, jp1 - 1, &G);
+    const double rtol = S->rtol;
+    const int max_iters = S->max_iters, m = S->m;
     for (int k0 = 0; k0 < jp1; k0 += T) {
         const int kn = jp1 - k0 < T ? jp1 - k0 : T;
         const bool lastt = k0 + T >= jp1;
@@ -491,17 +419,12 @@ __device__ __forceinline__ void dots_norm_last(SolveState *S, const double *part
                                                      lastt ? kn + 1 : kn, sh_w, sh_o);
         if (threadIdx.x < kn) {
             S->h[k0 + threadIdx.x] = sh_o[threadIdx.x];
-            sh_h[k0 + threadIdx.x] = sh_o[threadIdx.x];
+            G.h[k0 + threadIdx.x] = sh_o[threadIdx.x];
         }
-        if (lastt && threadIdx.x == 0) sh_ww = sh_o[kn];
+        if (lastt && threadIdx.x == 0) G.ww = sh_o[kn];
         __syncthreads();
     }
-    if (threadIdx.x != 0) return;
-    const double ww = sh_ww;
-    double hh = 0.0;
-    for (int k = 0; k < jp1; k++) hh = fma(sh_h[k], sh_h[k], hh);
-    const double d = ww - hh;
-    givens_column_staged(S, jp1 - 1, sh_h, &G, d > 1e-12 * ww ? sqrt(d) : 0.0);   // the next kernel publishes
+    givens_update(S, jp1 - 1, &G, rtol, max_iters, m);
 }
 
 // h[k] = <V_k, w>, k < jp1 (pass 0 -> S->h, pass 1 -> S->h2).  The grid is
