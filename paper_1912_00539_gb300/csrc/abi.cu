@@ -14,7 +14,7 @@ abilu_status apply_dispatch(abilu_factors f, const double *r, const float *r32, 
                             int nl, int nu, abilu_mode mode, cudaStream_t st, Skip skip);
 abilu_status export_dispatch(abilu_factors f, double *X, double *Dinv, cudaStream_t st);
 abilu_status spmv_launch(const PatternView &P, const double *A, double alpha, const double *x,
-                         double beta, double *y, cudaStream_t st, Skip skip);
+                         double beta, double *y, cudaStream_t st);
 size_t solve_state_bytes();
 size_t host_status_bytes();
 int max_restart();
@@ -35,6 +35,8 @@ int red_ctas() {
     }
     return v;
 }
+
+int sm_count() { return red_ctas() / 4; }
 
 static inline bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
@@ -190,7 +192,7 @@ extern "C" abilu_status bsr_spmv(abilu_pattern p, const double *A, double alpha,
     if (x == y) return fail(ABILU_EINVAL, "spmv: x and y must be distinct");
     if (!aligned16(A) || !aligned16(x) || !aligned16(y))
         return fail(ABILU_EINVAL, "spmv: pointers must be 16-byte aligned");
-    return spmv_launch(p->v, A, alpha, x, beta, y, S(stream), Skip{});
+    return spmv_launch(p->v, A, alpha, x, beta, y, S(stream));
 }
 
 extern "C" abilu_status abilu_factors_export(abilu_factors f, double *X, double *Dinv,

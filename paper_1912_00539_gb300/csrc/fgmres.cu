@@ -22,6 +22,8 @@
 #include <math.h>
 #include <string.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 #include "reduce.cuh"
 #include "spmv.cuh"
@@ -105,7 +107,7 @@ __device__ __forceinline__ bool last_cta(SolveState *S) { return last_arrival(&S
 // block reduction: deterministic for a fixed grid.  Every thread of the CTA
 // calls it.
 // R: CTAs whose partials are loaded before any add
-template <int K, int R = (K <= 2 ? 4 : 1)>
+template <int K, int R = (K <= 2 ? 4 : 1), int TH = RED_THREADS>
 __device__ __forceinline__ void reduce_partials(const double *partials, int stride, int k0,
                                                 int kn, double *sh_w, double *out) {
     double v[K];
@@ -125,7 +127,7 @@ __device__ __forceinline__ void reduce_partials(const double *partials, int stri
 #pragma unroll
             for (int k = 0; k < K; k++) v[k] += t[r][k];
     }
-    block_sum<K>(v, sh_w, out, kn);
+    block_sum<K, TH>(v, sh_w, out, kn);
 }
 
 // ---------------------------------------------------------------- residual
@@ -136,8 +138,8 @@ __device__ __forceinline__ void reduce_partials(const double *partials, int stri
 // (ZERO) r = b and ||r||^2 = ||b||^2 is accumulated once, and r_out is not
 // written (the caller scales b itself); after a cycle (init = 0) ||b||^2 is
 // not formed.
-template <bool ZERO>
-__global__ void __launch_bounds__(RED_THREADS, 3)
+template <bool ZERO, int TH = RED_THREADS>
+__global__ void __launch_bounds__(TH, TH == RED_THREADS ? 3 : 1)
 k_residual(PatternView P, const double *__restrict__ A, const double *__restrict__ b,
            const double *__restrict__ x, double *__restrict__ r_out, SolveState *S,
            double *partials, int init) {
@@ -146,12 +148,13 @@ k_residual(PatternView P, const double *__restrict__ A, const double *__restrict
     // a restart after a cycle in which no step ran (the initial guess had
     // already converged) would recompute the same residual: keep the state
     if (!init && S->kdim == 0) return;
-    __shared__ double sh_w[RED_THREADS * 2], sh_o[2];
+    extern __shared__ __align__(128) char smem[];   // the row stages, if any
+    __shared__ double sh_w[TH * 2], sh_o[2];
     const int q = threadIdx.x & 3;
     double v[2] = {0.0, 0.0};
-    const int rows_per_grid = gridDim.x * (RED_THREADS / 4);
-    int i = blockIdx.x * (RED_THREADS / 4) + (threadIdx.x >> 2);
     if constexpr (ZERO) {
+        const int rows_per_grid = gridDim.x * (TH / 4);
+        int i = blockIdx.x * (TH / 4) + (threadIdx.x >> 2);
         // r = b, not stored (the scale kernel that forms v_0 = r / beta reads
         // b itself); ||b||^2 with four rows' loads in flight per thread (one
         // per iteration left each thread waiting on a load 18 times in a
@@ -173,20 +176,17 @@ k_residual(PatternView P, const double *__restrict__ A, const double *__restrict
         }
         v[1] = v[0];
     } else {
-        for (; i < P.n; i += rows_per_grid) {
-            const size_t o = (size_t)i * BS + q;
-            // b issued with the row's matrix loads (after the product: 81.7
-            // against 78.6 us per launch at 512x512, ncu)
-            const double bi = __ldg(b + o);
-            // the SpMV kernel's arithmetic
-            const double s = row_dot_blocks(P, A, x, i, q);
-            const double ri = bi - s;
-            r_out[o] = ri;
-            v[0] += ri * ri;
-            if (init) v[1] += bi * bi;
-        }
+        // b issued with the row's matrix loads (after the product: 81.7
+        // against 78.6 us per launch at 512x512, ncu)
+        for_rows<TH>(P, A, x, smem, [&](int i) { return __ldg(b + (size_t)i * BS + q); },
+            [&](int i, double s, double bi) {
+                const double ri = bi - s;
+                r_out[(size_t)i * BS + q] = ri;
+                v[0] += ri * ri;
+                if (init) v[1] += bi * bi;
+            });
     }
-    block_sum<2>(v, sh_w, sh_o, 2);
+    block_sum<2, TH>(v, sh_w, sh_o, 2);
     if (threadIdx.x == 0) {
         partials[blockIdx.x * 2 + 0] = sh_o[0];
         partials[blockIdx.x * 2 + 1] = sh_o[1];
@@ -205,7 +205,7 @@ k_residual(PatternView P, const double *__restrict__ A, const double *__restrict
     case 3: sh_i[1] = S->max_iters; break;
     default: break;
     }
-    reduce_partials<2>(partials, 2, 0, 2, sh_w, sh_o);
+    reduce_partials<2, 4, TH>(partials, 2, 0, 2, sh_w, sh_o);
     if (threadIdx.x == 0) {
         const double rr = sh_o[0];
         const double bnorm = init ? sqrt(sh_o[1]) : sh_b[0];
@@ -223,6 +223,12 @@ k_residual(PatternView P, const double *__restrict__ A, const double *__restrict
         if (init) S->est = bnorm > 0.0 ? beta / bnorm : 0.0;
         S->counter = 0;
     }
+}
+
+static void launch_residual(int grid, cudaStream_t st, const PatternView &P, const double *A, const double *b,
+                            const double *x, double *r, SolveState *S, double *partials, int init) {
+    if (streamed(P.n)) launch_stream<k_residual<false, STREAM_THREADS>>(st, P, A, b, x, r, S, partials, init);
+    else launch_pdl(k_residual<false>, grid, RED_THREADS, 0, st, P, A, b, x, r, S, partials, init);
 }
 
 // the preconditioner's ticket counters zeroed for its next application
@@ -383,14 +389,14 @@ __device__ __forceinline__ void givens_column(SolveState *S, int j, int two_pass
 
 // The last CTA of a dot-product pass: h[k] = sum over CTAs of the partials of
 // slot k, k < jp1, in tiles of T (pass 0 -> S->h, pass 1 -> S->h2).  sh_w
-// holds RED_THREADS * T doubles.
-template <int T>
+// holds TH * T doubles.
+template <int T, int TH = RED_THREADS>
 __device__ __forceinline__ void dots_last(SolveState *S, const double *partials, int jp1, int pass,
                                           double *sh_w, double *sh_o) {
     double *h = pass == 0 ? S->h : S->h2;
     for (int k0 = 0; k0 < jp1; k0 += T) {
         const int kn = jp1 - k0 < T ? jp1 - k0 : T;
-        reduce_partials<T>(partials, MAXM + 2, k0, kn, sh_w, sh_o);
+        reduce_partials<T, (T <= 2 ? 4 : 1), TH>(partials, MAXM + 2, k0, kn, sh_w, sh_o);
         if (threadIdx.x < kn) h[k0 + threadIdx.x] = sh_o[threadIdx.x];
         __syncthreads();
     }
@@ -403,9 +409,9 @@ __device__ __forceinline__ void dots_last(SolveState *S, const double *partials,
 // with the norm; the Givens inputs staged while the partials are reduced;
 // every thread's partials loaded before any add (R CTAs per thread in one
 // round); then the Givens update of column j (givens_update).  sh_w holds
-// RED_THREADS * (T + 1) doubles.  The next kernel publishes the status.
+// TH * (T + 1) doubles.  The next kernel publishes the status.
 static_assert(GIVENS_MAX == MAXM, "one leading dimension");
-template <int T>
+template <int T, int TH>
 __device__ __forceinline__ void dots_norm_last(SolveState *S, const double *partials, int jp1,
                                                double *sh_w, double *sh_o) {
     __shared__ GivensIn G;
@@ -415,8 +421,8 @@ __device__ __forceinline__ void dots_norm_last(SolveState *S, const double *part
     for (int k0 = 0; k0 < jp1; k0 += T) {
         const int kn = jp1 - k0 < T ? jp1 - k0 : T;
         const bool lastt = k0 + T >= jp1;
-        reduce_partials<T + 1, (T + 1 <= 5 ? 3 : 2)>(partials, MAXM + 2, k0,
-                                                     lastt ? kn + 1 : kn, sh_w, sh_o);
+        reduce_partials<T + 1, (TH > RED_THREADS ? 1 : T + 1 <= 5 ? 3 : 2), TH>(
+            partials, MAXM + 2, k0, lastt ? kn + 1 : kn, sh_w, sh_o);
         if (threadIdx.x < kn) {
             S->h[k0 + threadIdx.x] = sh_o[threadIdx.x];
             G.h[k0 + threadIdx.x] = sh_o[threadIdx.x];
@@ -481,7 +487,7 @@ static void launch_dots(int nred, cudaStream_t st, const double *V, long long nv
 // kernel's grid stride (the same value-to-thread map as its product pass), for
 // the tiles past the first: w was written earlier in the same kernel by this
 // thread, so it is read back through L2 (never the read-only path).
-template <int K>
+template <int K, int TH>
 __device__ __forceinline__ void rows_dots_tile(int n, const double *__restrict__ V, long long nv,
                                                int k0, const double *w, double *sh_w, double *sh_o,
                                                double *partials) {
@@ -489,14 +495,14 @@ __device__ __forceinline__ void rows_dots_tile(int n, const double *__restrict__
 #pragma unroll
     for (int k = 0; k < K; k++) acc[k] = 0.0;
     const int q = threadIdx.x & 3;
-    const int rows_per_grid = gridDim.x * (RED_THREADS / 4);
-    for (int i = blockIdx.x * (RED_THREADS / 4) + (threadIdx.x >> 2); i < n; i += rows_per_grid) {
+    const int rows_per_grid = gridDim.x * (TH / 4);
+    for (int i = blockIdx.x * (TH / 4) + (threadIdx.x >> 2); i < n; i += rows_per_grid) {
         const size_t o = (size_t)i * BS + q;
         const double wv = __ldcg(w + o);
 #pragma unroll
         for (int k = 0; k < K; k++) acc[k] = fma(__ldg(V + (size_t)(k0 + k) * nv + o), wv, acc[k]);
     }
-    block_sum<K>(acc, sh_w, sh_o, K);
+    block_sum<K, TH>(acc, sh_w, sh_o, K);
     if (threadIdx.x < K) partials[(size_t)blockIdx.x * (MAXM + 2) + k0 + threadIdx.x] = sh_o[threadIdx.x];
 }
 
@@ -513,16 +519,17 @@ __device__ __forceinline__ void rows_dots_tile(int n, const double *__restrict__
 // Per thread the sums run over its rows in order, then the block sum; the
 // last CTA reduces the partials (slots 0..j, the norm in slot j + 1) and with
 // NORM forms h_{j+1,j} and the Givens update, so the result is deterministic
-// for a fixed grid.  Launched like the residual kernel, 3 CTAs per SM in one
-// wave: 80 registers hold a row's four blocks, its x gathers and the basis
-// entries in flight (at 64 registers and 4 CTAs per SM every width spilled,
-// and the solve was 0.5% slower).  SPMV_DOTS_MAX = 3: with four and five
-// basis vectors in the product's pass the accumulators spilled and the FP64
-// pipe's busy share fell from 89-92% to 84%; three there and the rest in a
-// tile that re-reads w measured 1.661 against 1.666 ms per solve.
+// for a fixed grid.  TH = RED_THREADS: 3 CTAs per SM in one wave; 80 registers
+// hold a row's four blocks, its x gathers and the basis entries in flight, with
+// up to three vectors in the product's pass (four and five spilled, the rest in a
+// tile that re-reads w measured 1.661 against 1.666 ms per solve).  TH =
+// STREAM_THREADS (large systems, spmv.cuh): the blocks in flight need no
+// registers, and six vectors fit the pass (fourth and fifth in a tile of their
+// own: 82 us each, in the pass 75 and 80).
 constexpr int SPMV_DOTS_MAX = 3;
-template <int KF, bool NORM, bool WIDE>
-__global__ void __launch_bounds__(RED_THREADS, 3)
+constexpr int SPMV_DOTS_STREAM = 6;
+template <int KF, bool NORM, bool WIDE, int TH = RED_THREADS>
+__global__ void __launch_bounds__(TH, TH == RED_THREADS ? 3 : 1)
 k_spmv_dots(PatternView P, const double *__restrict__ A, const double *__restrict__ z,
             double *w, const double *__restrict__ V, long long nv, int jp1, SolveState *S,
             double *partials) {
@@ -532,42 +539,49 @@ k_spmv_dots(PatternView P, const double *__restrict__ A, const double *__restric
     constexpr int KA = KF + (NORM ? 1 : 0);
     constexpr int T = WIDE ? TILE : KF;   // the tail's reduction tiles
     static_assert(KA <= TILE + 1, "the product pass's values fit the tail's staging");
-    __shared__ double sh_w[RED_THREADS * (T + 1)], sh_o[T + 1];
+    extern __shared__ __align__(128) char smem[];   // the row stages; then the reductions
+    constexpr bool STREAM = TH == STREAM_THREADS;
+    __shared__ double sh_own[STREAM ? 1 : TH * (T + 1)], sh_o[T + 1];
+    double *sh_w = STREAM ? reinterpret_cast<double *>(smem) : sh_own;
+    static_assert(!STREAM || (int)sizeof(double) * TH * (T + 1) <= STREAM_SMEM, "the reductions fit the stages");
     const int q = threadIdx.x & 3;
     double acc[KA];
 #pragma unroll
     for (int k = 0; k < KA; k++) acc[k] = 0.0;
-    const int rows_per_grid = gridDim.x * (RED_THREADS / 4);
-    for (int i = blockIdx.x * (RED_THREADS / 4) + (threadIdx.x >> 2); i < P.n; i += rows_per_grid) {
-        const size_t o = (size_t)i * BS + q;
-        double v[KF];   // issued with the row's matrix loads
+    struct Basis { double v[KF]; };
+    for_rows<TH>(P, A, z, smem,
+        [&](int i) {   // issued with the row's matrix loads
+            Basis t;
 #pragma unroll
-        for (int k = 0; k < KF; k++) v[k] = __ldg(V + (size_t)k * nv + o);
-        const double s = row_dot_blocks(P, A, z, i, q);
-        w[o] = s;
+            for (int k = 0; k < KF; k++) t.v[k] = __ldg(V + (size_t)k * nv + (size_t)i * BS + q);
+            return t;
+        },
+        [&](int i, double s, const Basis &t) {
+            w[(size_t)i * BS + q] = s;
 #pragma unroll
-        for (int k = 0; k < KF; k++) acc[k] = fma(v[k], s, acc[k]);
-        if constexpr (NORM) acc[KF] = fma(s, s, acc[KF]);
-    }
-    block_sum<KA>(acc, sh_w, sh_o, KA);
+            for (int k = 0; k < KF; k++) acc[k] = fma(t.v[k], s, acc[k]);
+            if constexpr (NORM) acc[KF] = fma(s, s, acc[KF]);
+        });
+    if constexpr (STREAM) __syncthreads();   // every warp done with its stages
+    block_sum<KA, TH>(acc, sh_w, sh_o, KA);
     double *pc = partials + (size_t)blockIdx.x * (MAXM + 2);
     if (threadIdx.x < KF) pc[threadIdx.x] = sh_o[threadIdx.x];
     if (NORM && threadIdx.x == 0) pc[WIDE ? jp1 : KF] = sh_o[KF];   // the norm's slot: j + 1
     if constexpr (WIDE) {
         for (int k0 = KF; k0 < jp1; k0 += TILE) {
             switch (jp1 - k0 < TILE ? jp1 - k0 : TILE) {
-            case 1: rows_dots_tile<1>(P.n, V, nv, k0, w, sh_w, sh_o, partials); break;
-            case 2: rows_dots_tile<2>(P.n, V, nv, k0, w, sh_w, sh_o, partials); break;
-            case 3: rows_dots_tile<3>(P.n, V, nv, k0, w, sh_w, sh_o, partials); break;
-            case 4: rows_dots_tile<4>(P.n, V, nv, k0, w, sh_w, sh_o, partials); break;
-            case 5: rows_dots_tile<5>(P.n, V, nv, k0, w, sh_w, sh_o, partials); break;
-            default: rows_dots_tile<6>(P.n, V, nv, k0, w, sh_w, sh_o, partials); break;
+            case 1: rows_dots_tile<1, TH>(P.n, V, nv, k0, w, sh_w, sh_o, partials); break;
+            case 2: rows_dots_tile<2, TH>(P.n, V, nv, k0, w, sh_w, sh_o, partials); break;
+            case 3: rows_dots_tile<3, TH>(P.n, V, nv, k0, w, sh_w, sh_o, partials); break;
+            case 4: rows_dots_tile<4, TH>(P.n, V, nv, k0, w, sh_w, sh_o, partials); break;
+            case 5: rows_dots_tile<5, TH>(P.n, V, nv, k0, w, sh_w, sh_o, partials); break;
+            default: rows_dots_tile<6, TH>(P.n, V, nv, k0, w, sh_w, sh_o, partials); break;
             }
         }
     }
     if (!last_cta(S)) return;
-    if constexpr (NORM) dots_norm_last<T>(S, partials, jp1, sh_w, sh_o);   // k_update_scale publishes
-    else dots_last<T>(S, partials, jp1, 0, sh_w, sh_o);
+    if constexpr (NORM) dots_norm_last<T, TH>(S, partials, jp1, sh_w, sh_o);   // k_update_scale publishes
+    else dots_last<T, TH>(S, partials, jp1, 0, sh_w, sh_o);
 }
 
 // k_spmv_dots for step j (jp1 = j + 1 basis vectors)
@@ -575,14 +589,32 @@ template <bool NORM>
 static void launch_spmv_dots_n(int grid, cudaStream_t st, const PatternView &P, const double *A,
                                const double *z, double *w, const double *V, long long nv, int jp1,
                                SolveState *S, double *partials) {
+    auto go = [&](auto kf, auto wide) {
+        constexpr int KF = decltype(kf)::value;
+        constexpr bool WIDE = decltype(wide)::value;
+        if constexpr (KF <= SPMV_DOTS_MAX) {
+            if (!streamed(P.n)) {
+                launch_pdl(k_spmv_dots<KF, NORM, WIDE>, grid, RED_THREADS, 0, st, P, A, z, w, V, nv, jp1, S, partials);
+                return;
+            }
+        }
+        if constexpr (!WIDE || KF == SPMV_DOTS_STREAM)
+            launch_stream<k_spmv_dots<KF, NORM, WIDE, STREAM_THREADS>>(st, P, A, z, w, V, nv, jp1, S, partials);
+    };
+    using F = std::false_type;
+    using W = std::true_type;
+    if (!streamed(P.n) && jp1 > SPMV_DOTS_MAX) return go(std::integral_constant<int, SPMV_DOTS_MAX>{}, W{});
     switch (jp1) {
-    case 1: launch_pdl(k_spmv_dots<1, NORM, false>, grid, RED_THREADS, 0, st, P, A, z, w, V, nv, jp1, S, partials); break;
-    case 2: launch_pdl(k_spmv_dots<2, NORM, false>, grid, RED_THREADS, 0, st, P, A, z, w, V, nv, jp1, S, partials); break;
-    case 3: launch_pdl(k_spmv_dots<3, NORM, false>, grid, RED_THREADS, 0, st, P, A, z, w, V, nv, jp1, S, partials); break;
-    default: launch_pdl(k_spmv_dots<3, NORM, true>, grid, RED_THREADS, 0, st, P, A, z, w, V, nv, jp1, S, partials); break;
+    case 1: go(std::integral_constant<int, 1>{}, F{}); break;
+    case 2: go(std::integral_constant<int, 2>{}, F{}); break;
+    case 3: go(std::integral_constant<int, 3>{}, F{}); break;
+    case 4: go(std::integral_constant<int, 4>{}, F{}); break;
+    case 5: go(std::integral_constant<int, 5>{}, F{}); break;
+    case 6: go(std::integral_constant<int, 6>{}, F{}); break;
+    default: go(std::integral_constant<int, SPMV_DOTS_STREAM>{}, W{}); break;
     }
 }
-static_assert(SPMV_DOTS_MAX == 3, "one instance per width up to SPMV_DOTS_MAX");
+static_assert(SPMV_DOTS_MAX <= 6 && SPMV_DOTS_STREAM == 6, "an instance per width");
 
 // v_{j+1} = (w - sum_k h[k] V_k) * hn_inv and its FP32 copy (the next
 // preconditioner's input) in one pass; w itself is not written back.  J =
@@ -949,7 +981,7 @@ abilu_status fgmres_run(const PatternView &P, const double *A, abilu_factors ws,
     if (opts->zero_guess)
         launch_pdl(k_residual<true>, nres, RED_THREADS, 0, st, P, A, b, x, V, SS, ws->partials, 1);
     else
-        launch_pdl(k_residual<false>, nres, RED_THREADS, 0, st, P, A, b, x, V, SS, ws->partials, 1);
+        launch_residual(nres, st, P, A, b, x, V, SS, ws->partials, 1);
     // v_0 = r / beta; with x = 0, r = b is read from b itself
     launch_pdl(k_scale, nred, RED_THREADS, 0, st, opts->zero_guess ? b : V, V, v32, nv2, SS,
                pc.y0, pc.tickets, none);
@@ -1019,7 +1051,7 @@ abilu_status fgmres_run(const PatternView &P, const double *A, abilu_factors ws,
         if (ret != ABILU_OK) break;
         if (first && opts->zero_guess) launch_pdl(k_xupdate<true>, nred, RED_THREADS, 0, st, Z, nv2, x, SS);
         else launch_pdl(k_xupdate<false>, nred, RED_THREADS, 0, st, Z, nv2, x, SS);
-        launch_pdl(k_residual<false>, nres, RED_THREADS, 0, st, P, A, b, x, V, SS, ws->partials, 0);
+        launch_residual(nres, st, P, A, b, x, V, SS, ws->partials, 0);
         // the handles' counters go into the status with every cycle's result, so
         // the synchronisation that ends the last cycle also ends the solve
         launch_pdl(k_scale, nred, RED_THREADS, 0, st, V, V, v32, nv2, SS, pc.y0, pc.tickets, cl);

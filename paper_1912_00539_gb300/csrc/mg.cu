@@ -127,19 +127,30 @@ k_galerkin(long long nnzb_c, const int4 *__restrict__ grec, const int *__restric
 
 // r = b - A x, a quad per block row; into r, or rounded into r32 when only the
 // FP32 right-hand side of a smoothing step is wanted (r NULL)
-__global__ void __launch_bounds__(MG_THREADS)
+template <int TH>
+__global__ void __launch_bounds__(TH, TH == STREAM_THREADS ? 1 : 3)
 k_mg_residual(PatternView P, const double *__restrict__ A, const double *__restrict__ b,
               const double *__restrict__ x, double *__restrict__ r, float *__restrict__ r32,
               Skip skip) {
+    extern __shared__ __align__(128) char smem[];
     pdl_wait();
     pdl_trigger();
     if (skip_all(skip)) return;
-    const int i = blockIdx.x * MG_ROWS + (threadIdx.x >> 2), q = threadIdx.x & 3;
-    if (i >= P.n) return;
-    const size_t o = (size_t)i * BS + q;
-    const double v = b[o] - row_dot_blocks(P, A, x, i, q);
-    if (r) r[o] = v;
-    else r32[o] = to_f32_int(v);
+    const int q = threadIdx.x & 3;
+    for_rows<TH>(P, A, x, smem, [&](int i) { return __ldg(b + (size_t)i * BS + q); },
+        [&](int i, double s, double bi) {
+            const size_t o = (size_t)i * BS + q;
+            const double v = bi - s;
+            if (r) r[o] = v;
+            else r32[o] = to_f32_int(v);
+        });
+}
+
+static void launch_residual(const PatternView &P, const double *A, const double *b, const double *x,
+                            double *r, float *r32, cudaStream_t st, Skip skip) {
+    if (streamed(P.n)) launch_stream<k_mg_residual<STREAM_THREADS>>(st, P, A, b, x, r, r32, skip);
+    else launch_pdl(k_mg_residual<MG_THREADS>, (P.n + MG_ROWS - 1) / MG_ROWS, MG_THREADS, 0, st, P, A, b, x,
+                    r, r32, skip);
 }
 
 // Restriction bc = P^T r: bc[I] = sum over the cells i of aggregate I, in
@@ -398,8 +409,7 @@ static abilu_status smooth(abilu_mg mg, int l, int steps, const double *b, const
             *xzero = false;
             continue;
         }
-        launch_pdl(k_mg_residual, grid_of(4LL * L.n), MG_THREADS, 0, st, L.p->v, L.A, b, x,
-                   r32 ? nullptr : L.r, r32, skip);
+        launch_residual(L.p->v, L.A, b, x, r32 ? nullptr : L.r, r32, st, skip);
         ABILU_LAUNCH_CHECK("k_mg_residual");
         s = apply_add_dispatch(L.f, L.r, r32, x, o.apply_sweeps_lower, o.apply_sweeps_upper, mode,
                                st, skip);
@@ -425,8 +435,7 @@ static abilu_status vcycle(abilu_mg mg, int l, const double *b, const float *b32
     if ((s = smooth(mg, l, o.pre_smooth, b, b32, x, &xzero, st, skip)) != ABILU_OK) return s;
     const double *rf = b;   // the fine residual: b itself while x = 0
     if (!xzero) {
-        launch_pdl(k_mg_residual, grid_of(4LL * L.n), MG_THREADS, 0, st, L.p->v, L.A, b, x, L.r,
-                   nullptr, skip);
+        launch_residual(L.p->v, L.A, b, x, L.r, nullptr, st, skip);
         ABILU_LAUNCH_CHECK("k_mg_residual");
         rf = L.r;
     }

@@ -13,7 +13,9 @@
 // x_j, and writes y_i[q].  The first four blocks of a row are loaded before
 // any arithmetic so each thread keeps up to 8 independent 16-byte loads in
 // flight.  Half of a row's products are FP64 FMAs, half integer sums
-// (spmv.cuh): 60.8 us at 512x512 (5.1 TB/s), 65.7 with FMAs alone.
+// (spmv.cuh).  Large systems stream the rows through shared memory, one CTA
+// per SM: 512x512 51.0 us, 6.1 TB/s (65.7 with FMAs alone, 60.8 before the
+// streamed form).
 #include "common.cuh"
 #include "spmv.cuh"
 
@@ -27,29 +29,35 @@ constexpr int SPMV_ROWS = SPMV_THREADS / 4;
 // per output cost 12% when the FP64 pipe bounded this kernel).
 // Otherwise y = alpha A x + beta y, and beta == 0 never reads y (which may
 // hold NaN).
-template <bool PLAIN>
-__global__ void __launch_bounds__(SPMV_THREADS)
+template <bool PLAIN, int TH>
+__global__ void __launch_bounds__(TH, TH == STREAM_THREADS ? 1 : 3)
 k_spmv(PatternView P, const double *__restrict__ A, double alpha, const double *__restrict__ x,
-       double beta, double *__restrict__ y, Skip skip) {
+       double beta, double *__restrict__ y) {
+    extern __shared__ __align__(128) char smem[];
     pdl_wait();
     pdl_trigger();
-    if (skip_all(skip) || skip_chunk(skip, blockIdx.x)) return;
-    const int i = blockIdx.x * SPMV_ROWS + (threadIdx.x >> 2), q = threadIdx.x & 3;
-    if (i >= P.n) return;
-    const double s = row_dot_blocks(P, A, x, i, q);
-    const size_t o = (size_t)i * BS + q;
-    if constexpr (PLAIN) y[o] = s;
-    else y[o] = beta == 0.0 ? alpha * s : alpha * s + beta * y[o];
+    const int q = threadIdx.x & 3;
+    for_rows<TH>(P, A, x, smem,
+        [&](int i) { return PLAIN || beta == 0.0 ? 0.0 : y[(size_t)i * BS + q]; },
+        [&](int i, double s, double y0) {
+            const size_t o = (size_t)i * BS + q;
+            if constexpr (PLAIN) y[o] = s;
+            else y[o] = beta == 0.0 ? alpha * s : alpha * s + beta * y0;
+        });
 }
 
 abilu_status spmv_launch(const PatternView &P, const double *A, double alpha, const double *x,
-                         double beta, double *y, cudaStream_t st, Skip skip) {
-    static_assert(SPMV_ROWS == SKIP_CHUNK_ROWS, "one CTA per 64-row chunk");
+                         double beta, double *y, cudaStream_t st) {
     const int grid = (P.n + SPMV_ROWS - 1) / SPMV_ROWS;
-    if (alpha == 1.0 && beta == 0.0)
-        launch_pdl(k_spmv<true>, grid, SPMV_THREADS, 0, st, P, A, alpha, x, beta, y, skip);
-    else
-        launch_pdl(k_spmv<false>, grid, SPMV_THREADS, 0, st, P, A, alpha, x, beta, y, skip);
+    const bool plain = alpha == 1.0 && beta == 0.0;
+    if (streamed(P.n)) {
+        if (plain) launch_stream<k_spmv<true, STREAM_THREADS>>(st, P, A, alpha, x, beta, y);
+        else launch_stream<k_spmv<false, STREAM_THREADS>>(st, P, A, alpha, x, beta, y);
+    } else if (plain) {
+        launch_pdl(k_spmv<true, SPMV_THREADS>, grid, SPMV_THREADS, 0, st, P, A, alpha, x, beta, y);
+    } else {
+        launch_pdl(k_spmv<false, SPMV_THREADS>, grid, SPMV_THREADS, 0, st, P, A, alpha, x, beta, y);
+    }
     ABILU_LAUNCH_CHECK("k_spmv");
     return ABILU_OK;
 }

@@ -5,6 +5,8 @@
 // flight.  Blocks in order, within a block x_j[0..3]; the third and fourth
 // blocks' eight products are summed with integer instructions (fx_dot8).
 #pragma once
+#include <atomic>
+
 #include "common.cuh"
 
 namespace abilu {
@@ -136,6 +138,189 @@ __device__ __forceinline__ double row_dot_blocks(const PatternView &P, const dou
         s = fma(b1.y, x1.y, s);
     }
     return s;
+}
+
+// ---- large systems: the rows' blocks and their x through shared memory
+//
+// One CTA per SM takes 160 rows at a time and has the next 160 rows' first four
+// blocks and the x they meet in flight into a second shared-memory stage while
+// it works on the current ones: 16-byte cp.async copies, waited for by the
+// copying warp alone (a wait instruction, no polling), so no block-wide barrier,
+// no registers for blocks in flight (32 in row_dot_blocks, which spilled in the
+// fused kernels) and no gather on a row's critical path: pointers are read three
+// rows ahead, columns two.  512x512 (us, direct -> streamed; 47 are the bytes at
+// the copy rate): product 60.8 -> 51.0, residual 71 -> 61, fused product and 1 .. 5
+// dots 72, 79, 82, 91, 91 -> 64, 67, 71, 75, 80.  Gathers of x left to the row's own
+// loads: product 58.
+// One CTA per SM and not three: behind the staged sweeps, whose CTAs leave an SM
+// one by one, three CTAs of 64 KB did not always fit side by side, and the grid
+// took two waves (fused kernels of 73 .. 91 us took 96 .. 150).
+//
+// A quad's copies of blocks are 64 contiguous bytes per instruction; odd rows
+// swap the 16-byte halves of each 32 bytes, so the lanes of a shared-memory phase
+// (two rows) use distinct banks.
+constexpr int STREAM_THREADS = 640;
+constexpr int STREAM_ROWS = STREAM_THREADS / 4;
+constexpr int STREAM_SLOT = 4 * BB * (int)sizeof(double) + 4 * BS * (int)sizeof(double);   // 640 bytes a row
+constexpr int STREAM_STAGE = STREAM_ROWS * STREAM_SLOT;
+constexpr int STREAM_SMEM = 2 * STREAM_STAGE;                                              // 200 KB
+
+__device__ __forceinline__ void cp_async16_cg(unsigned dst, const void *src, int bytes) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void cp_async16_ca(unsigned dst, const void *src, int bytes) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+
+// the positions of a row's blocks; thread q of the quad: the column of block p0 + q
+struct StreamRow {
+    int p0, p1, jq;
+    __device__ __forceinline__ void ptrs(const PatternView &P, int i, int end) {
+        p0 = p1 = 0;
+        if (i < end) {
+            p0 = __ldg(P.rowptr + i);
+            p1 = __ldg(P.rowptr + i + 1);
+        }
+    }
+    __device__ __forceinline__ void col(const PatternView &P) {
+        const int p = p0 + (int)(threadIdx.x & 3);
+        jq = p < p1 ? __ldg(P.colind + p) : -1;
+    }
+};
+
+// copies of the row's first four blocks and their x into the quad's slot (zeros
+// where the row has fewer)
+__device__ __forceinline__ void stream_issue(const double *__restrict__ A, const double *__restrict__ x,
+                                             unsigned slot, const StreamRow &r) {
+    const int q = threadIdx.x & 3, sw = (threadIdx.x >> 2) & 1;
+    const unsigned dst = slot + (unsigned)((q ^ sw) * 16);
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+        const bool in = r.p0 + k < r.p1;
+        const double *src = A + (in ? (size_t)(r.p0 + k) * BB + q * 2 : 0);
+        cp_async16_cg(dst + k * 128, src, in ? 16 : 0);
+        cp_async16_cg(dst + k * 128 + 64, in ? src + 8 : src, in ? 16 : 0);
+    }
+    const bool in = r.jq >= 0;
+    const double *src = x + (in ? (size_t)r.jq * BS : 0);
+    const unsigned xd = slot + 512u + (unsigned)(q * 32);
+    cp_async16_ca(xd + (unsigned)(sw * 16), src, in ? 16 : 0);
+    cp_async16_ca(xd + (unsigned)((sw ^ 1) * 16), in ? src + 2 : src, in ? 16 : 0);
+}
+
+// entry q of the row in the quad's slot: row_dot_blocks's operations
+__device__ __forceinline__ double stream_dot(const PatternView &P, const double *__restrict__ A,
+                                             const double *__restrict__ x, const char *slot, int p0, int p1) {
+    const int q = threadIdx.x & 3, sw = (threadIdx.x >> 2) & 1;
+    const char *alo = slot + ((2 * q) ^ sw) * 16, *ahi = slot + ((2 * q + 1) ^ sw) * 16;
+    const char *xlo = slot + 512 + sw * 16, *xhi = slot + 512 + (sw ^ 1) * 16;
+    auto ld = [](const char *p) { return *reinterpret_cast<const double2 *>(p); };
+    double s = 0.0;
+#pragma unroll
+    for (int k = 0; k < 2; k++) {
+        const double2 a0 = ld(alo + k * 128), a1 = ld(ahi + k * 128), x0 = ld(xlo + k * 32), x1 = ld(xhi + k * 32);
+        s = fma(a0.x, x0.x, s);
+        s = fma(a0.y, x0.y, s);
+        s = fma(a1.x, x1.x, s);
+        s = fma(a1.y, x1.y, s);
+    }
+    if (p1 - p0 > 2) {
+        double av[8], xv[8];
+#pragma unroll
+        for (int k = 0; k < 2; k++) {
+            const double2 a0 = ld(alo + 256 + k * 128), a1 = ld(ahi + 256 + k * 128);
+            const double2 x0 = ld(xlo + 64 + k * 32), x1 = ld(xhi + 64 + k * 32);
+            av[4 * k] = a0.x; av[4 * k + 1] = a0.y; av[4 * k + 2] = a1.x; av[4 * k + 3] = a1.y;
+            xv[4 * k] = x0.x; xv[4 * k + 1] = x0.y; xv[4 * k + 2] = x1.x; xv[4 * k + 3] = x1.y;
+        }
+        s += fx_dot8(av, xv);
+    }
+    for (int p = p0 + 4; p < p1; p++) {  // rows longer than four blocks
+        const int j = __ldg(P.colind + p);
+        const double2 *ap = reinterpret_cast<const double2 *>(A + (size_t)p * BB + q * BS);
+        const double2 *xp = reinterpret_cast<const double2 *>(x + (size_t)j * BS);
+        double2 b0 = __ldg(ap), b1 = __ldg(ap + 1), x0 = __ldg(xp), x1 = __ldg(xp + 1);
+        s = fma(b0.x, x0.x, s);
+        s = fma(b0.y, x0.y, s);
+        s = fma(b1.x, x1.x, s);
+        s = fma(b1.y, x1.y, s);
+    }
+    return s;
+}
+
+// The CTA's rows blockIdx.x * TH / 4 .., a grid stride of TH / 4 rows per CTA,
+// below n: post(i, (A x)_i[q], pre(i)) in the quad of row i, pre's loads issued
+// before the row's product.  TH = STREAM_THREADS: through `smem`, the CTA's
+// STREAM_SMEM bytes, free again after a block-wide barrier; else directly.
+// Every thread of the CTA calls it.
+template <int TH, typename Pre, typename Post>
+__device__ __forceinline__ void for_rows(const PatternView &P, const double *__restrict__ A,
+                                         const double *__restrict__ x, char *smem, Pre pre, Post post) {
+    const int q = threadIdx.x & 3, n = P.n, step = gridDim.x * (TH / 4);
+    int i = blockIdx.x * (TH / 4) + (threadIdx.x >> 2);
+    if constexpr (TH != STREAM_THREADS) {
+        for (; i < n; i += step) {
+            auto v = pre(i);
+            post(i, row_dot_blocks(P, A, x, i, q), v);
+        }
+    } else {
+        int wi = i - (int)((threadIdx.x & 31) >> 2);   // the warp's first row: its loop is uniform
+        if (wi >= n) return;
+        char *slot = smem + (threadIdx.x >> 2) * STREAM_SLOT;
+        const unsigned uslot = (unsigned)__cvta_generic_to_shared(slot);
+        StreamRow r, r1, r2;
+        r.ptrs(P, i, n);
+        r1.ptrs(P, i + step, n);
+        r2.ptrs(P, i + 2 * step, n);
+        r.col(P);
+        r1.col(P);
+        stream_issue(A, x, uslot, r);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        for (int off = 0;; off = STREAM_STAGE - off) {
+            const bool more = wi + step < n;
+            if (more) stream_issue(A, x, uslot + (unsigned)(STREAM_STAGE - off), r1);
+            asm volatile("cp.async.commit_group;" ::: "memory");
+            r2.col(P);
+            StreamRow r3;
+            r3.ptrs(P, i + 3 * step, n);
+            auto v = pre(i < n ? i : n - 1);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+            __syncwarp();   // the quad's other copies
+            if (i < n) post(i, stream_dot(P, A, x, slot + off, r.p0, r.p1), v);
+            if (!more) break;
+            __syncwarp();   // every lane has read this stage
+            r = r1;
+            r1 = r2;
+            r2 = r3;
+            i += step;
+            wi += step;
+        }
+    }
+}
+
+// Whether the streamed form takes a system of n rows.  Both forms measured (us,
+// product / FGMRES solve, direct -> streamed): 16k rows 9.3 / 226 -> 9.9 / 236, 51k
+// 9.9 / 305 -> 11.2 / 309, 99k 12.4 / 432 -> 13.3 / 430, 131k 16.4 / 502 -> 15.9 /
+// 499, 262k 37.4 / 802 -> 29.0 / 781: with five passes of 160 rows per SM the
+// pipeline's ramp is paid for.
+constexpr int STREAM_MIN_ROWS = 120000;
+int sm_count();
+inline bool streamed(int n) { return n >= STREAM_MIN_ROWS; }
+
+// launch_pdl of a kernel of STREAM_THREADS threads with the stages (its dynamic
+// shared memory allowed once per kernel and device)
+template <auto K, typename... Args>
+inline cudaError_t launch_stream(cudaStream_t st, Args &&...args) {
+    static std::atomic<unsigned long long> allowed{0ull};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const unsigned long long bit = 1ull << (dev & 63);
+    if (!(allowed.load(std::memory_order_relaxed) & bit)) {
+        const cudaError_t e = cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, STREAM_SMEM);
+        if (e != cudaSuccess) return e;
+        allowed.fetch_or(bit, std::memory_order_relaxed);
+    }
+    return launch_pdl(K, sm_count(), STREAM_THREADS, STREAM_SMEM, st, std::forward<Args>(args)...);
 }
 
 }  // namespace abilu

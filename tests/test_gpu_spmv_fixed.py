@@ -101,3 +101,42 @@ def test_integers_are_exact():
         for q in range(4):
             s = sum(int(A[p, q, c]) * int(x[colind[p], c]) for p in range(rowptr[i], rowptr[i + 1]) for c in range(4))
             assert y[i, q] == float(s)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n,blocks", [(119999, 4), (120000, 4), (120001, 7), (121599, 3), (121601, 5)])
+def test_streamed_rows_match_the_direct_form(n, blocks):
+    """Both sides of the size where the rows go through shared memory, row counts
+    that leave the last 160-row pass of some CTAs ragged, rows of 1 .. `blocks`
+    blocks (none to three beyond the staged four).  Both forms run the same
+    operations in the same order, so a system's rows give the same bits alone
+    (direct) and as the tail of a larger one (streamed)."""
+    import torch
+    import paper_1912_00539_gb300.abilu as ab
+    rng = np.random.default_rng(n + blocks)
+    cnt = 1 + np.arange(n) % blocks
+    rowptr = np.concatenate([[0], np.cumsum(cnt)]).astype(np.int32)
+    row = np.repeat(np.arange(n), cnt)
+    k = np.arange(len(row)) - rowptr[row]
+    # columns within the last or the first 60,000 rows of each half, sorted and
+    # distinct: row - a few .. row, kept inside the row's half
+    half = np.where(row >= n - 60000, n - 60000, 0)
+    colind = np.where(row - cnt[row] + 1 >= half, row - (cnt[row] - 1 - k), np.maximum(half, row) + k)
+    colind = np.minimum(colind, n - 1).astype(np.int32)
+    A = torch.from_numpy(rng.standard_normal((len(row), 4, 4))).cuda()
+    x = torch.from_numpy(rng.standard_normal((n, 4))).cuda()
+    y0 = torch.from_numpy(rng.standard_normal((n, 4))).cuda()
+    pat = ab.Pattern(torch.from_numpy(rowptr).cuda(), torch.from_numpy(colind).cuda())
+    y, y2 = torch.empty_like(x), y0.clone()
+    ab.bsr_spmv(pat, A, x, y)
+    ab.bsr_spmv(pat, A, x, y2, alpha=-0.5, beta=2.0)
+    # the last 60,000 rows as a system of their own
+    o, p = n - 60000, int(rowptr[n - 60000])
+    sub = ab.Pattern(torch.from_numpy(rowptr[o:] - p).cuda(), torch.from_numpy(colind[p:] - o).cuda())
+    z, z2 = torch.empty_like(x[o:]), y0[o:].clone()
+    ab.bsr_spmv(sub, A[p:], x[o:], z)
+    ab.bsr_spmv(sub, A[p:], x[o:], z2, alpha=-0.5, beta=2.0)
+    assert torch.equal(y[o:], z) and torch.equal(y2[o:], z2)
+    want = np.zeros((n, 4))
+    np.add.at(want, row, np.einsum("prc,pc->pr", A.cpu().numpy(), x.cpu().numpy()[colind]))
+    assert np.abs(y.cpu().numpy() - want).max() < 1e-13 * np.abs(want).max()
