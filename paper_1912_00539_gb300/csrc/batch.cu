@@ -155,15 +155,6 @@ k_b_residual(PatternView P, const double *__restrict__ A, const double *__restri
     }
 }
 
-// bflag = {all systems done with the cycle, systems still active}; reset
-// before the residual kernel that starts a cycle
-__global__ void k_b_flags_reset(int *bflag) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        bflag[0] = 1;
-        bflag[1] = 0;
-    }
-}
-
 // The apply's two ticket counters zeroed for its next application (first
 // CTA, whatever its system's state), when the kernels that write its FP32
 // right-hand side also prepare its start (see apply_dispatch_ready)
@@ -472,17 +463,41 @@ k_b_update_scale(const double *__restrict__ V, size_t nv, int j, const double *_
     }
 }
 
-// y = R^{-1} g per system (one thread per system)
-__global__ void k_b_ysolve(BState *S, int nsys) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= nsys) return;
-    BState *St = S + s;
-    const int kd = St->kdim;
-    for (int i = kd - 1; i >= 0; i--) {
-        double v = St->g[i];
-        for (int k = i + 1; k < kd; k++) v -= St->H[i * BMAXM + k] * St->y[k];
-        St->y[i] = v / St->H[i * BMAXM + i];
+// y = R^{-1} g, a CTA per system: R's upper triangle, g and the reciprocals of
+// R's diagonal in shared memory by the whole CTA, the back substitution by one
+// thread from there (a thread per system reading them as it went took 12 us for
+// four systems).  Also resets the cycle flags {all done, active count} for the
+// residual kernel that starts the next cycle.
+__global__ void __launch_bounds__(128)
+k_b_ysolve(BState *S, int *bflag) {
+    pdl_wait();
+    pdl_trigger();
+    __shared__ double sR[BMAXM * (BMAXM + 1) / 2], sg[BMAXM], sinv[BMAXM];
+    BState *St = S + blockIdx.x;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        bflag[0] = 1;
+        bflag[1] = 0;
     }
+    const int kd = St->kdim;
+    for (int t = threadIdx.x; t < kd * kd; t += blockDim.x) {
+        const int i = t / kd, k = t % kd;
+        if (k >= i) sR[i * kd - i * (i - 1) / 2 + (k - i)] = St->H[i * BMAXM + k];
+    }
+    for (int t = threadIdx.x; t < kd; t += blockDim.x) {
+        sg[t] = St->g[t];
+        sinv[t] = 1.0 / St->H[t * BMAXM + t];
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int i = kd - 1; i >= 0; i--) {
+            const double *Ri = sR + i * kd - i * (i - 1) / 2 - i;   // Ri[k] = R[i][k], k >= i
+            double v = sg[i];
+            for (int k = i + 1; k < kd; k++) v -= Ri[k] * sg[k];
+            sg[i] = v * sinv[i];
+        }
+    }
+    __syncthreads();
+    for (int t = threadIdx.x; t < kd; t += blockDim.x) St->y[t] = sg[t];
 }
 
 // x += Z y for the chunk's system
@@ -501,14 +516,24 @@ k_b_xupdate(const double *__restrict__ Z, size_t nv, double *__restrict__ x, con
     x[e] = t;
 }
 
-__global__ void k_b_init(BState *S, int nsys) {
+// The systems' states at a solve's start (the fields read before a kernel writes
+// them) and bflag = {all systems done with the cycle, systems still active},
+// for the residual kernel that starts the first cycle
+__global__ void k_b_init(BState *S, int nsys, int *bflag) {
+    pdl_wait();
+    pdl_trigger();
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    if (s == 0) {
+        bflag[0] = 1;
+        bflag[1] = 0;
+    }
     if (s >= nsys) return;
     S[s].iters = 0;
     S[s].restarts = 0;
     S[s].counter = 0;
     S[s].finished = 0;
     S[s].done = 0;
+    S[s].kdim = 0;
 }
 
 // ---- concatenation
@@ -928,9 +953,8 @@ static abilu_status enqueue_restart(abilu_batch b, const fgmres_opts *opts, cons
     const size_t nv = (size_t)b->rows * BS;
     double *V = b->krylov, *Z = V + (size_t)(m + 1) * nv;
     float *v32 = reinterpret_cast<float *>(b->fac->r32);
-    k_b_ysolve<<<counted((nsys + 127) / 128), 128, 0, st>>>(b->S, nsys);
+    k_b_ysolve<<<counted(nsys), 128, 0, st>>>(b->S, b->bflag);   // (may follow a conditional node)
     launch_pdl(k_b_xupdate, nck, RED_THREADS, 0, st, Z, nv, b->x, b->S, b->chunk_sys);
-    k_b_flags_reset<<<counted(1), 32, 0, st>>>(b->bflag);
     launch_pdl(k_b_residual, b->nsc, RED_THREADS, 0, st, P, b->A, b->b, b->x, V, b->S, batch_tab(b),
         b->partials, cf, 0, b->hs_done, b->hs_fin, b->sys_done, b->bflag);
     launch_pdl(k_b_scale, nck, RED_THREADS, 0, st, V, V, v32, b->S, b->chunk_sys, ys.y0, ys.tk);
@@ -1054,9 +1078,7 @@ static abilu_status batch_solve_core(abilu_batch b, const fgmres_opts *opts, fgm
         if (s != ABILU_OK) return s;
     }
     ABILU_CUDA(cudaMemsetAsync(b->x, 0, sizeof(double) * nv, st));
-    ABILU_CUDA(cudaMemsetAsync(b->S, 0, sizeof(BState) * nsys, st));
-    k_b_init<<<counted((nsys + 127) / 128), 128, 0, st>>>(b->S, nsys);
-    k_b_flags_reset<<<counted(1), 32, 0, st>>>(b->bflag);
+    launch_pdl(k_b_init, (nsys + 127) / 128, 128, 0, st, b->S, nsys, b->bflag);
     launch_pdl(k_b_residual, b->nsc, RED_THREADS, 0, st, P, b->A, b->b, b->x, V, b->S, batch_tab(b),
         b->partials, cf, 1, b->hs_done, b->hs_fin, b->sys_done, b->bflag);
     launch_pdl(k_b_scale, nck, RED_THREADS, 0, st, V, V, v32, b->S, b->chunk_sys, ys.y0, ys.tk);
