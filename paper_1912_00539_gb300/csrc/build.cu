@@ -281,6 +281,68 @@ constexpr int WORK_PER_CTA = BUILD_THREADS / 4;
 static_assert(WORK_PER_CTA == WORK_CHUNK, "work list chunks are sorted per CTA");
 static_assert(sizeof(WorkItem) == 32, "work records are two 16-byte loads");
 
+// The synchronous sweeps: rows exchanged by shuffles (through shared memory, as
+// below, they took the same 66 us each, and rounded their sums in another order).
+//
+// s -= L_ik U_kj for the quad's block (thread q: row q); u's row k lives in thread k
+__device__ __forceinline__ void sub_product_shfl(float s[4], const float l[4], const float u[4]) {
+    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int k = 0; k < 4; k++)
+#pragma unroll
+        for (int c = 0; c < 4; c++) acc[c] += l[k] * qshfl(u[c], k);
+#pragma unroll
+    for (int c = 0; c < 4; c++) s[c] -= acc[c];
+}
+
+template <typename T>
+__device__ __forceinline__ void build_block_sync(const PatternView &P, int w,
+                                            const float *__restrict__ A32, const T *Lin,
+                                            const T *Uin, const T *Din, T *Lout, T *Uout, T *Dout,
+                                            T *Udiag, float *sh_q, unsigned long long *nsing) {
+    const int q = threadIdx.x & 3;
+    const WorkItem it = P.work[w];
+    float s[4], d[4];
+    ld_row(A32 + (size_t)w * BB + q * BS, s);
+    const int kind = it.kind_np & 3, np = it.kind_np >> 2, dst = it.dst;
+    if (kind == WORK_L) ld_row(Din + (size_t)it.j * BB + q * BS, d);
+    if (np > 0) {  // products in pair order (ascending k)
+        float l0[4], u0[4], l1[4], u1[4];
+        ld_row(Lin + (size_t)it.pr[0].x * BB + q * BS, l0);  // row q of L_ik
+        ld_row(Uin + (size_t)it.pr[0].y * BB + q * BS, u0);  // row q of U_kj
+        if (np > 1) {
+            ld_row(Lin + (size_t)it.pr[1].x * BB + q * BS, l1);
+            ld_row(Uin + (size_t)it.pr[1].y * BB + q * BS, u1);
+        }
+        sub_product_shfl(s, l0, u0);
+        if (np > 1) sub_product_shfl(s, l1, u1);
+        for (int t = 2; t < np; t++) {
+            const int2 pr = P.pairs[it.t0 + t];
+            ld_row(Lin + (size_t)pr.x * BB + q * BS, l0);
+            ld_row(Uin + (size_t)pr.y * BB + q * BS, u0);
+            sub_product_shfl(s, l0, u0);
+        }
+    }
+    if (kind == WORK_L) {  // L_ij = S Dinv_j; row k of Dinv_j lives in thread k
+        float o[4];
+#pragma unroll
+        for (int c = 0; c < 4; c++) {
+            float d0 = qshfl(d[c], 0), d1 = qshfl(d[c], 1), d2 = qshfl(d[c], 2), d3 = qshfl(d[c], 3);
+            o[c] = s[0] * d0 + s[1] * d1 + s[2] * d2 + s[3] * d3;
+        }
+        st_row(Lout + (size_t)dst * BB + q * BS, o);
+    } else if (kind == WORK_U) {
+        st_row(Uout + (size_t)dst * BB + q * BS, s);
+    } else {  // U_ii = S, Dinv_i = inv(U_ii), refined only in a build's last sweep, in
+              // either mode (Udiag passed): earlier inverses only feed the next updates
+        float x[4];
+        if (quad_inv4_refined(s, x, sh_q, Udiag != nullptr) && q == 0) atomicAdd(nsing, 1ull);
+        st_row(Dout + (size_t)dst * BB + q * BS, x);
+        if (Udiag) st_row(Udiag + (size_t)dst * BB + q * BS, s);
+    }
+}
+
+// ---- in place
 // The quad's rows of one block through shared memory: thread q stores row q,
 // after the barrier every thread reads the four rows (one 16-byte store and four
 // broadcast loads; 16 shuffles before, which had the load/store unit 41% and
@@ -312,8 +374,8 @@ __device__ __forceinline__ void sub_product(float s[4], const float l[4], const 
     for (int c = 0; c < 4; c++) s[c] -= acc[c];
 }
 
-template <typename T, bool VOL>
-__device__ __forceinline__ void build_block(const PatternView &P, int w,
+template <typename T>
+__device__ __forceinline__ void build_block_async(const PatternView &P, int w,
                                             const float *__restrict__ A32, const T *Lin,
                                             const T *Uin, const T *Din, T *Lout, T *Uout, T *Dout,
                                             T *Udiag, float *sh_q, unsigned long long *nsing) {
@@ -323,15 +385,15 @@ __device__ __forceinline__ void build_block(const PatternView &P, int w,
     float s[4], d[4];
     ld_row(A32 + (size_t)w * BB + q * BS, s);
     const int kind = it.kind_np & 3, np = it.kind_np >> 2, dst = it.dst;
-    if (kind == WORK_L) ld_row_sel<VOL>(Din + (size_t)it.j * BB + q * BS, d);
+    if (kind == WORK_L) ld_row_sel<true>(Din + (size_t)it.j * BB + q * BS, d);
     if (np > 0) {  // products in pair order (ascending k)
         float l0[4], u[4], l1[4];
-        ld_row_sel<VOL>(Lin + (size_t)it.pr[0].x * BB + q * BS, l0);  // row q of L_ik
-        ld_row_sel<VOL>(Uin + (size_t)it.pr[0].y * BB + q * BS, u);   // row q of U_kj
+        ld_row_sel<true>(Lin + (size_t)it.pr[0].x * BB + q * BS, l0);  // row q of L_ik
+        ld_row_sel<true>(Uin + (size_t)it.pr[0].y * BB + q * BS, u);   // row q of U_kj
         if (np > 1) {
             float u1[4];
-            ld_row_sel<VOL>(Lin + (size_t)it.pr[1].x * BB + q * BS, l1);
-            ld_row_sel<VOL>(Uin + (size_t)it.pr[1].y * BB + q * BS, u1);
+            ld_row_sel<true>(Lin + (size_t)it.pr[1].x * BB + q * BS, l1);
+            ld_row_sel<true>(Uin + (size_t)it.pr[1].y * BB + q * BS, u1);
             put_row(sh_q + 16, u1);
         }
         put_row(sh_q, u);
@@ -340,8 +402,8 @@ __device__ __forceinline__ void build_block(const PatternView &P, int w,
         if (np > 1) sub_product(s, l1, sh_q + 16);
         for (int t = 2; t < np; t++) {
             const int2 pr = P.pairs[it.t0 + t];
-            ld_row_sel<VOL>(Lin + (size_t)pr.x * BB + q * BS, l0);
-            ld_row_sel<VOL>(Uin + (size_t)pr.y * BB + q * BS, u);
+            ld_row_sel<true>(Lin + (size_t)pr.x * BB + q * BS, l0);
+            ld_row_sel<true>(Uin + (size_t)pr.y * BB + q * BS, u);
             __syncwarp(m);   // every thread has read the previous rows
             put_row(sh_q, u);
             __syncwarp(m);
@@ -353,15 +415,15 @@ __device__ __forceinline__ void build_block(const PatternView &P, int w,
         put_row(sh_q + 32, d);
         __syncwarp(m);
         row_times(o, s, sh_q + 32);
-        st_row_sel<VOL>(Lout + (size_t)dst * BB + q * BS, o);
+        st_row_sel<true>(Lout + (size_t)dst * BB + q * BS, o);
     } else if (kind == WORK_U) {
-        st_row_sel<VOL>(Uout + (size_t)dst * BB + q * BS, s);
+        st_row_sel<true>(Uout + (size_t)dst * BB + q * BS, s);
     } else {  // U_ii = S, Dinv_i = inv(U_ii), refined only in a build's last sweep, in
               // either mode (Udiag passed): earlier inverses only feed the next updates
         float x[4];
         __syncwarp(m);   // the products' rows are read
         if (quad_inv4_refined(s, x, sh_q, Udiag != nullptr) && q == 0) atomicAdd(nsing, 1ull);
-        st_row_sel<VOL>(Dout + (size_t)dst * BB + q * BS, x);
+        st_row_sel<true>(Dout + (size_t)dst * BB + q * BS, x);
         if (Udiag) st_row_sel<false>(Udiag + (size_t)dst * BB + q * BS, s);
     }
     __syncwarp(m);   // the scratch is free for the quad's next block
@@ -378,7 +440,7 @@ k_build_blocks_sync(PatternView P, const float *__restrict__ A32, const T *__res
     __shared__ __align__(16) float sh_q[WORK_PER_CTA * QUAD_SCRATCH];
     const int w = blockIdx.x * WORK_PER_CTA + (threadIdx.x >> 2);
     if (w >= P.nwork) return;  // whole quads leave together
-    build_block<T, false>(P, w, A32, Lin, Uin, Din, Lout, Uout, Dout, Udiag,
+    build_block_sync<T>(P, w, A32, Lin, Uin, Din, Lout, Uout, Dout, Udiag,
                           sh_q + (threadIdx.x >> 2) * QUAD_SCRATCH, nsing);
 }
 
@@ -390,7 +452,7 @@ k_build_blocks_sync(PatternView P, const float *__restrict__ A32, const T *__res
 // of nchunks sub-chunks: sub-chunks c, c + nchunks, c + 2 nchunks, ...  Each
 // sub-chunk is done in steps of 8 blocks (one block per quad, consecutive
 // blocks, so a step stays within one kind).  Small lists take tickets of
-// 8-block sub-chunks (SMALL_TICKET).
+// consecutive blocks (SMALL_TICKET).
 //
 // Why the stride: the ILU fixed-point residual after a given number of sweeps
 // falls as the blocks in flight (resident warps x blocks per ticket) span
@@ -425,18 +487,23 @@ __host__ __device__ __forceinline__ long long build_tickets(int nwork, int wchun
 }
 
 // Lists of at most SMALL_TICKET blocks per resident warp (7,296 warps at 48 per
-// SM: 467k blocks, 187k grid cells) take the smallest ticket of 8-block
-// sub-chunks that gives no more tickets than warps, so a sweep is at most one
-// ticket per warp.  Such lists are bound by the serial steps of a ticket: with
-// 128-block tickets a 20k-block list kept 160 warps busy for 16 dependent
-// steps per sweep.  Measured, 4 sweeps with the prepare pass, 40 warps per SM (us, 128-block
-// tickets -> this rule): 2.4k blocks 80 -> 30, 20k 91 -> 34, 82k 96 -> 53, 144k
-// 105 -> 68, 327k 149 -> 124; 8 sweeps of 326k (wall-normal coupling 100x) 231 ->
-// 178.  Above the line the 64-block groups win: 737k blocks 253 against 286.
-// FGMRES iterations over those lists: the same or within one at the settings
-// used with them.  Fixing each warp's blocks for all sweeps (no tickets, no
-// flags) was faster still (20k: 22) but lets warps drift apart by sweeps:
-// FGMRES took 24 iterations where the ordered tickets take 7.
+// SM: 467k blocks, 187k grid cells) take the smallest ticket, a multiple of 8
+// consecutive blocks (SUB = 8), that gives no more tickets than warps, so a sweep
+// is at most one ticket per warp.  Such lists are bound by the serial steps of a
+// ticket: with 128-block tickets a 20k-block list kept 160 warps busy for 16
+// dependent steps per sweep.  Measured, 4 sweeps with the prepare pass, 40 warps
+// per SM (us, 128-block tickets -> this rule): 2.4k blocks 80 -> 30, 20k 91 -> 34,
+// 82k 96 -> 53, 144k 105 -> 68, 327k 149 -> 124.  Above the line the 64-block groups
+// win: 737k blocks 253 against 286.  Consecutive blocks, not the strided ones
+// of the large lists: on wall-normal lines (coupling 100x along the line) a
+// warp that updates a piece of a line in order carries it as Gauss-Seidel does;
+// FGMRES on 182k cells in line order took 3 iterations (587 us per solve), 5.3
+// with 8-block pieces half the list apart (848), 3 with 128-block tickets (682).
+// Whole solves over 26 drawn grids of 3k to 435k cells, both orderings: all
+// faster than with 128-block tickets, iterations the same in RCM order, up to
+// one more (3 -> 4) on the smallest lines.  Fixing each warp's blocks for all
+// sweeps (no tickets, no flags) was faster still (20k: 22) but lets warps drift
+// apart by sweeps: FGMRES took 24 iterations where the ordered tickets take 7.
 constexpr int SMALL_TICKET = 64;
 
 template <typename T, bool ORDERED, int SUB>
@@ -478,12 +545,12 @@ k_build_blocks_async(PatternView P, const float *__restrict__ A32, T *L, T *U, T
         // steps (32-bit: block indices stay below (nsub + wchunk / SUB) * SUB,
         // and nwork <= nnzb < 2^31 - 2^16)
         constexpr int SSH = SUB == 64 ? 3 : SUB == 32 ? 2 : 0;   // log2(steps per sub-chunk)
-        const int base = chunk * SUB + (lane >> 2);
+        const int base = chunk * (SUB == 8 ? wchunk : SUB) + (lane >> 2);
 #pragma unroll 1
         for (int k = 0; k < wchunk / 8; k++) {
-            const int w = base + (k >> SSH) * stride + ((k & ((1 << SSH) - 1)) << 3);
+            const int w = SUB == 8 ? base + 8 * k : base + (k >> SSH) * stride + ((k & ((1 << SSH) - 1)) << 3);
             if (w < P.nwork)
-                build_block<T, true>(P, w, A32, L, U, D, L, U, D, last ? Udiag : nullptr, myq, nsing);
+                build_block_async<T>(P, w, A32, L, U, D, L, U, D, last ? Udiag : nullptr, myq, nsing);
         }
         if constexpr (ORDERED) __threadfence();   // this lane's factor writes, before the flag
         __syncwarp();
