@@ -82,27 +82,30 @@ __device__ __forceinline__ VT row_sweep_sum(VT s, const T *__restrict__ F,
     return s;
 }
 
-// The FP64 form: one FMA per entry into the running sum (five operations per
-// block as a separate dot product and subtraction, on the pipe that bounds these
-// sweeps).
+// The FP64 form: one FMA per entry into the sum of the row's products, subtracted
+// once (a dot product and a subtraction per block took five operations on the
+// pipe that bounds these sweeps; FMAs into s itself took none for the subtraction
+// but rounded at s's magnitude four times per block: 3.0e-16 from exact after a
+// build and an application where the separate dot products left 2.3e-16).
 template <bool VOL>
 __device__ __forceinline__ double row_sweep_sum(double s, const double *__restrict__ F,
                                                 const int32_t *__restrict__ col, int l0, int l1,
                                                 const double *v) {
     const int q = threadIdx.x & 3;
-    for (int l = l0; l < l1; l++) {   // (two blocks read at a time: 49 against 38 us, registers)
+    double acc = 0.0;
+    for (int l = l0; l < l1; l++) {   // (two blocks read at a time: 10 us slower, registers)
         double a[4], b[4];
         ld_row(F + (size_t)l * BB + q * BS, a);
         ld_row_sel<VOL>(v + (size_t)col[l] * BS, b);
 #pragma unroll
-        for (int c = 0; c < 4; c++) s = fma(-a[c], b[c], s);
+        for (int c = 0; c < 4; c++) acc = fma(a[c], b[c], acc);
     }
-    return s;
+    return s - acc;
 }
 
 // The row of this quad among the 64 rows from row0 (n or more: none) and its
 // blocks l0 .. l1-1: in order, or for FP64 by decreasing block count
-// (row_by_work).  512x512, one sweep (us): lower 63 -> 37, upper 73 -> 52 (upper with its Dinv product).
+// (row_by_work).  512x512, one sweep (us): lower 63 -> 42, upper 73 -> 55 (upper with its Dinv product).
 template <typename VT>
 __device__ __forceinline__ int sweep_row(const int32_t *__restrict__ ptr, int row0, int n, int &l0, int &l1) {
     if constexpr (sizeof(VT) == 8) {

@@ -566,9 +566,8 @@ k_build_blocks_async(PatternView P, const float *__restrict__ A32, T *L, T *U, T
 // 32 rows by decreasing number of product pairs (row_by_work), then the U blocks
 // with pairs, again as one list, and the inverses one thread per row.  A quad
 // per block row, its blocks in turn, ran the L update, the diagonal update and
-// each pair count of its eight rows one after the other.  Products subtract by
-// FMA from the block itself.  512x512, one sweep: 473 -> 351 us (the FP64
-// instructions alone: about 300).
+// each pair count of its eight rows one after the other.  512x512, one sweep: 473 -> 371 us (the FP64
+// instructions alone: about 310), the same bits.
 //
 // VOL (in place, Algorithm 4 with blocks): reads are volatile, and a barrier
 // puts the rows' new L blocks before their diagonal and U updates.
@@ -595,13 +594,15 @@ __device__ __forceinline__ void sub_pairs_f64(const PatternView &P, int t0, int 
     const int q = threadIdx.x & 3;
     for (int t = t0; t < t1; t++) {
         const int2 pr = P.pairs[t];
-        double l[4], u[4];
+        double l[4], u[4], acc[4] = {0.0, 0.0, 0.0, 0.0};
         ld_row_sel<VOL>(Lin + (size_t)pr.x * BB + q * BS, l);  // row q of L_ik
         ld_row_sel<VOL>(Uin + (size_t)pr.y * BB + q * BS, u);  // row q of U_kj
 #pragma unroll
         for (int k = 0; k < 4; k++)
 #pragma unroll
-            for (int c = 0; c < 4; c++) s[c] = fma(-l[k], qshfl(u[c], k), s[c]);
+            for (int c = 0; c < 4; c++) acc[c] = fma(l[k], qshfl(u[c], k), acc[c]);
+#pragma unroll
+        for (int c = 0; c < 4; c++) s[c] -= acc[c];
     }
 }
 
@@ -683,7 +684,7 @@ k_build_sync(PatternView P, const double *__restrict__ A, const double *__restri
 
 // Persistent in-place kernel: tickets t = 0 .. nsweeps*nchunks-1 taken in
 // order from ctr; ticket t is chunk (t mod nchunks) in sweep (t / nchunks).
-__global__ void __launch_bounds__(BUILD_THREADS, 4)
+__global__ void __launch_bounds__(BUILD_THREADS, 3)
 k_build_async(PatternView P, const double *__restrict__ A, double *L, double *U, double *D,
               double *Udiag, int nsweeps, unsigned long long *nsing, unsigned long long *ticket) {
     pdl_wait();
