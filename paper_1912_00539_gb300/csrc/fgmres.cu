@@ -996,6 +996,7 @@ abilu_status fgmres_run(const PatternView &P, const double *A, abilu_factors ws,
     // (the device flag is set).  The host reads the status one step behind.
     HostStatus h = {};
     abilu_status ret = ABILU_OK;
+    bool x_written = false;
     for (bool first = true; first || (!h.converged && h.iters < opts->max_iters); first = false) {
         int j = 0;
         double e_prev = -1.0;   // the estimate after step j-2, as the host last read it
@@ -1049,6 +1050,7 @@ abilu_status fgmres_run(const PatternView &P, const double *A, abilu_factors ws,
             }
         }
         if (ret != ABILU_OK) break;
+        x_written = true;
         if (first && opts->zero_guess) launch_pdl(k_xupdate<true>, nred, RED_THREADS, 0, st, Z, nv2, x, SS);
         else launch_pdl(k_xupdate<false>, nred, RED_THREADS, 0, st, Z, nv2, x, SS);
         launch_residual(nres, st, P, A, b, x, V, SS, ws->partials, 0);
@@ -1062,7 +1064,9 @@ abilu_status fgmres_run(const PatternView &P, const double *A, abilu_factors ws,
         h = read_status(hs);
     }
     const bool zero_b = ret == ABILU_OK && h.bnorm == 0.0;
-    if (zero_b)  // b = 0: the solution is x = 0
+    // b = 0: the solution is x = 0; a solve from a zero guess that failed before
+    // it wrote x leaves the guess
+    if (zero_b || (opts->zero_guess && !x_written))
         ABILU_CUDA(cudaMemsetAsync(x, 0, sizeof(double) * nv, st));
     if (ret != ABILU_OK || zero_b) {   // a cycle that did not finish, or the memset
         k_counters<<<counted(1), 32, 0, st>>>(SS, cl);
