@@ -3,9 +3,10 @@
 // One sweep evaluates, for every block (i,j) of S_B,
 //   S_ij = A_ij - sum_{k<min(i,j)} L_ik U_kj            (Eq. bilu)
 //   U_ij = S_ij (i <= j),  L_ij = S_ij U_jj^{-1} (i > j),
-// and refreshes Dinv_i = U_ii^{-1}.  Work item = one block row (the paper's
-// work item, Sec. 3.3), blocks of the row in ascending column order with a
-// local accumulator and one write per block.
+// and refreshes Dinv_i = U_ii^{-1}.  Work item = one block (FP32/BF16 factors) or
+// the blocks of 64 rows (FP64), a local accumulator and one write per block.  In
+// place, FP64 keeps the order of the paper's work item, a block row (Sec. 3.3): a
+// block sees its own row's blocks of smaller column as this sweep made them.
 //
 // Thread mapping: 4 threads ("a quad") per block; thread q of the quad
 // owns row q of every 4x4 block, so a block is read with four 16/32-byte row
@@ -566,11 +567,17 @@ k_build_blocks_async(PatternView P, const float *__restrict__ A32, T *L, T *U, T
 // 32 rows by decreasing number of product pairs (row_by_work), then the U blocks
 // with pairs, again as one list, and the inverses one thread per row.  A quad
 // per block row, its blocks in turn, ran the L update, the diagonal update and
-// each pair count of its eight rows one after the other.  512x512, one sweep: 473 -> 371 us (the FP64
-// instructions alone: about 310), the same bits.
+// each pair count of its eight rows one after the other.  512x512, one synchronous sweep: 473 -> 371 us
+// (the FP64 instructions alone: about 310), the same bits.
 //
-// VOL (in place, Algorithm 4 with blocks): reads are volatile, and a barrier
-// puts the rows' new L blocks before their diagonal and U updates.
+// VOL (in place, Algorithm 4 with blocks): reads are volatile, and a block reads
+// the blocks of its own row with smaller column from this sweep.  So the list
+// holds the L blocks without product pairs only; the ones with pairs (patterns
+// with triangles: S_ij needs L_ik, k < j) follow behind a barrier, a quad per
+// row in ascending order (a thread reads back the rows it wrote itself), and a
+// barrier puts the rows' L blocks before their diagonal and U updates.  All L
+// blocks as one list in place left the factors of a nine-point grid ten times
+// further from the sequential ones after four sweeps (7.3e-4, in order 6.3e-5).
 struct F64Rows {
     double u[BUILD_ROWS * INV_LD];      // U_ii, then Dinv_i
     int lr[BUILD_ROWS + 1], ur[BUILD_ROWS + 1];
@@ -619,21 +626,39 @@ __device__ __forceinline__ void build_rows_f64(const PatternView &P, int row0,
         sh.ur[threadIdx.x] = P.urow[row0 + threadIdx.x];
     }
     __syncthreads();
-    for (int t = sh.lr[0] + quad; t < sh.lr[rows]; t += BUILD_ROWS) {   // L_ij = S Dinv_j
-        const int r = list_row(sh.lr, rows, t);
-        const int p = P.rowptr[row0 + r] + (t - sh.lr[r]);
+    auto l_block = [&](int t, int p, int t0, int t1) {   // L_ij = S Dinv_j
         double s[4], d[4], o[4];
         ld_row_sel<VOL>(Din + (size_t)P.lcol[t] * BB + q * BS, d);
         ld_row(A + (size_t)p * BB + q * BS, s);
-        sub_pairs_f64<VOL>(P, P.pair_ptr[p], P.pair_ptr[p + 1], Lin, Uin, s);
+        sub_pairs_f64<VOL>(P, t0, t1, Lin, Uin, s);
 #pragma unroll
         for (int c = 0; c < 4; c++) {   // row k of Dinv_j lives in thread k
             const double d0 = qshfl(d[c], 0), d1 = qshfl(d[c], 1), d2 = qshfl(d[c], 2), d3 = qshfl(d[c], 3);
             o[c] = s[0] * d0 + s[1] * d1 + s[2] * d2 + s[3] * d3;
         }
         st_row_sel<VOL>(Lout + (size_t)t * BB + q * BS, o);
+    };
+    bool paired = false;
+    for (int t = sh.lr[0] + quad; t < sh.lr[rows]; t += BUILD_ROWS) {
+        const int r = list_row(sh.lr, rows, t);
+        const int p = P.rowptr[row0 + r] + (t - sh.lr[r]);
+        const int t0 = P.pair_ptr[p], t1 = P.pair_ptr[p + 1];
+        if (VOL && t0 != t1) paired = true;
+        else l_block(t, p, t0, t1);
     }
-    if constexpr (VOL) __syncthreads();
+    if constexpr (VOL) {
+        if (__syncthreads_or(paired)) {
+            if (quad < rows) {
+                const int p0 = P.rowptr[row0 + quad];
+                for (int t = sh.lr[quad]; t < sh.lr[quad + 1]; t++) {
+                    const int p = p0 + (t - sh.lr[quad]);
+                    const int t0 = P.pair_ptr[p], t1 = P.pair_ptr[p + 1];
+                    if (t0 != t1) l_block(t, p, t0, t1);
+                }
+            }
+            __syncthreads();
+        }
+    }
     {   // U_ii = S
         const int lane = threadIdx.x & 31, base = row0 + (threadIdx.x >> 7) * 32, mine = base + lane;
         int dp = 0, t0 = 0, t1 = 0;

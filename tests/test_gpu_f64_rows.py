@@ -56,3 +56,34 @@ def test_f64_build_and_sweeps_match_the_oracle(n, longest):
     ys = oracle.lower_solve(rowptr, colind, Xs, r)
     zs = oracle.upper_solve(rowptr, colind, Xs, Ds, ys)
     assert np.abs(z.cpu().numpy() - zs).max() / np.abs(zs).max() < 1e-12
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n,longest", [(2, 3), (20, 9), (33, 14), (64, 7), (64, 65)])
+def test_f64_in_place_keeps_the_order_of_a_row(n, longest):
+    """One in-place sweep over at most 64 rows, which one CTA does: U and Dinv are
+    still A's when the L blocks are formed, so L_ij = (A_ij - sum_{k<j} L_ik A_kj)
+    A_jj^-1 with the L_ik of the same sweep, whatever the timing (up to a full
+    lower triangle, 63 blocks in a row, 62 product pairs).  The bound is that of
+    the comparison with the oracle above."""
+    import torch
+    import paper_1912_00539_gb300.abilu as ab
+    rowptr, colind, A, _ = _system(n, longest, 7 * n + longest)
+    pos = {(i, int(colind[p])): p for i in range(n) for p in range(rowptr[i], rowptr[i + 1])}
+    want, pairs = A.copy(), 0
+    for (i, j), p in sorted(pos.items()):
+        if j >= i:
+            continue
+        s = A[p].copy()
+        for k in range(j):
+            if (i, k) in pos and (k, j) in pos:
+                s -= want[pos[i, k]] @ A[pos[k, j]]
+                pairs += 1
+        want[p] = s @ np.linalg.inv(A[pos[j, j]])
+    assert pairs > 0 or longest < 9
+    pat = ab.Pattern(torch.from_numpy(rowptr).cuda(), torch.from_numpy(colind).cuda())
+    fac = ab.Factors(pat, "f64")
+    fac.build(torch.from_numpy(A).cuda(), 1, mode="async")
+    X = fac.export()[0].cpu().numpy()
+    low = np.array([p for (i, j), p in pos.items() if j < i], np.int64)
+    assert np.abs(X[low] - want[low]).max(initial=0.0) < 1e-13 * np.abs(want).max()
