@@ -561,26 +561,35 @@ k_build_blocks_async(PatternView P, const float *__restrict__ A32, T *L, T *U, T
 
 // ---- FP64 factors: 64 rows per CTA
 // The FP64 pipe bounds these sweeps (16 cycles per warp-wide instruction
-// whatever lanes are active), so every quad of a warp gets the same work: the
-// rows' L blocks as one list (they are contiguous in the compact array; the
-// row of each by a search in shared memory), then the diagonal blocks of each
-// 32 rows by decreasing number of product pairs (row_by_work), then the U blocks
-// with pairs, again as one list, and the inverses one thread per row.  A quad
-// per block row, its blocks in turn, ran the L update, the diagonal update and
-// each pair count of its eight rows one after the other.  512x512, one synchronous sweep: 473 -> 371 us
-// (the FP64 instructions alone: about 310), the same bits.
+// whatever lanes are active), so the quads of a warp get the same work.  Without
+// product pairs among the L blocks (no triangles in the pattern): the rows' L
+// blocks as one list (contiguous in the compact array; the row of each by a
+// search in shared memory), then the diagonal blocks of each 32 rows by
+// decreasing number of pairs (row_by_work), the inverses one thread per row.  A
+// quad per block row, its blocks in turn, ran the L update, the diagonal update
+// and each pair count of its eight rows one after the other.  512x512
+// triangulated cells, one synchronous sweep: 473 -> 371 us (the FP64
+// instructions alone: about 310), the same bits.
+//
+// L and U blocks with pairs (patterns with triangles: S_ij needs L_ik and U_kj)
+// are done a quad per row, rows by decreasing work.  Neighbours in a row have
+// different pair counts, so a warp that took them from a list ran the largest of
+// its eight for each.  The L blocks without pairs join their row when most rows
+// of the CTA have pairs, else they stay a list.  4 synchronous sweeps (us: a quad
+// per row in storage order, everything as lists, this): nine-point grid of 262k cells
+// 2,677, 5,076, 2,724; random rows of about 30 blocks, 200k, 22,030, 18,010, 17,380;
+// of about 14, 60k, 2,684, 1,760, 1,917; of about 4, 200k, 1,511, 831, 872.
 //
 // VOL (in place, Algorithm 4 with blocks): reads are volatile, and a block reads
-// the blocks of its own row with smaller column from this sweep.  So the list
-// holds the L blocks without product pairs only; the ones with pairs (patterns
-// with triangles: S_ij needs L_ik, k < j) follow behind a barrier, a quad per
-// row in ascending order (a thread reads back the rows it wrote itself), and a
-// barrier puts the rows' L blocks before their diagonal and U updates.  All L
-// blocks as one list in place left the factors of a nine-point grid ten times
-// further from the sequential ones after four sweeps (7.3e-4, in order 6.3e-5).
+// the blocks of its own row with smaller column from this sweep: the L blocks
+// with pairs wait for the list behind a barrier and are done in ascending order (a
+// thread reads back the rows it wrote itself), and a barrier puts the rows' L
+// blocks before their diagonal and U updates.  All L blocks as one list in place
+// left the factors of a nine-point grid ten times further from the sequential
+// ones after four sweeps (7.3e-4, in order 6.3e-5).
 struct F64Rows {
     double u[BUILD_ROWS * INV_LD];      // U_ii, then Dinv_i
-    int lr[BUILD_ROWS + 1], ur[BUILD_ROWS + 1];
+    int lr[BUILD_ROWS + 1];             // first L block of each row
     unsigned char ord[BUILD_THREADS];
 };
 
@@ -621,11 +630,18 @@ __device__ __forceinline__ void build_rows_f64(const PatternView &P, int row0,
                                                F64Rows &sh, unsigned long long *nsing) {
     const int q = threadIdx.x & 3, quad = threadIdx.x >> 2;
     const int rows = min(BUILD_ROWS, P.n - row0);
-    if (threadIdx.x <= rows) {
-        sh.lr[threadIdx.x] = P.lrow[row0 + threadIdx.x];
-        sh.ur[threadIdx.x] = P.urow[row0 + threadIdx.x];
+    if (threadIdx.x <= rows) sh.lr[threadIdx.x] = P.lrow[row0 + threadIdx.x];
+    // the pairs of this lane's row: L blocks' m0 .. m1-1, diagonal's .. m2-1, U blocks' .. m3-1
+    const int lane = threadIdx.x & 31, base = row0 + (threadIdx.x >> 7) * 32, mine = base + lane;
+    int m0 = 0, m1 = 0, m2 = 0, m3 = 0;
+    if (mine < P.n) {
+        const int dp = P.diagpos[mine];
+        m0 = P.pair_ptr[P.rowptr[mine]];
+        m1 = P.pair_ptr[dp];
+        m2 = P.pair_ptr[dp + 1];
+        m3 = P.pair_ptr[P.rowptr[mine + 1]];
     }
-    __syncthreads();
+    unsigned char *ord = sh.ord + (threadIdx.x & ~31);
     auto l_block = [&](int t, int p, int t0, int t1) {   // L_ij = S Dinv_j
         double s[4], d[4], o[4];
         ld_row_sel<VOL>(Din + (size_t)P.lcol[t] * BB + q * BS, d);
@@ -638,43 +654,37 @@ __device__ __forceinline__ void build_rows_f64(const PatternView &P, int row0,
         }
         st_row_sel<VOL>(Lout + (size_t)t * BB + q * BS, o);
     };
-    bool paired = false;
-    for (int t = sh.lr[0] + quad; t < sh.lr[rows]; t += BUILD_ROWS) {
-        const int r = list_row(sh.lr, rows, t);
-        const int p = P.rowptr[row0 + r] + (t - sh.lr[r]);
-        const int t0 = P.pair_ptr[p], t1 = P.pair_ptr[p + 1];
-        if (VOL && t0 != t1) paired = true;
-        else l_block(t, p, t0, t1);
-    }
-    if constexpr (VOL) {
-        if (__syncthreads_or(paired)) {
-            if (quad < rows) {
-                const int p0 = P.rowptr[row0 + quad];
-                for (int t = sh.lr[quad]; t < sh.lr[quad + 1]; t++) {
-                    const int p = p0 + (t - sh.lr[quad]);
-                    const int t0 = P.pair_ptr[p], t1 = P.pair_ptr[p + 1];
-                    if (t0 != t1) l_block(t, p, t0, t1);
-                }
+    // (also the barrier behind sh.lr; a row is counted by four threads, and more
+    // than half of the rows must have pairs)
+    const int with_pairs = __syncthreads_count(m1 > m0);
+    const bool by_row = with_pairs > 2 * rows;
+    if (!by_row)
+        for (int t = sh.lr[0] + quad; t < sh.lr[rows]; t += BUILD_ROWS) {
+            const int r = list_row(sh.lr, rows, t);
+            const int p = P.rowptr[row0 + r] + (t - sh.lr[r]);
+            const int t0 = with_pairs ? P.pair_ptr[p] : 0;
+            if (!with_pairs || t0 == P.pair_ptr[p + 1]) l_block(t, p, t0, t0);
+        }
+    if (with_pairs) {
+        if (VOL && !by_row) __syncthreads();
+        const int off = row_by_work<true>(by_row && mine < P.n ? m1 - m0 + P.lrow[mine + 1] - P.lrow[mine] : m1 - m0, ord);
+        const int i = base + off;
+        if (i < P.n) {
+            const int p0 = P.rowptr[i], dp = P.diagpos[i], l0 = sh.lr[i - row0];
+            for (int p = p0; p < dp; p++) {
+                const int t0 = P.pair_ptr[p], t1 = P.pair_ptr[p + 1];
+                if (by_row || t0 != t1) l_block(l0 + (p - p0), p, t0, t1);
             }
-            __syncthreads();
         }
     }
+    if constexpr (VOL) __syncthreads();
     {   // U_ii = S
-        const int lane = threadIdx.x & 31, base = row0 + (threadIdx.x >> 7) * 32, mine = base + lane;
-        int dp = 0, t0 = 0, t1 = 0;
-        if (mine < P.n) {
-            dp = P.diagpos[mine];
-            t0 = P.pair_ptr[dp];
-            t1 = P.pair_ptr[dp + 1];
-        }
-        const int off = row_by_work(t1 - t0, sh.ord + (threadIdx.x & ~31));
-        dp = __shfl_sync(0xffffffffu, dp, off);
-        t0 = __shfl_sync(0xffffffffu, t0, off);
-        t1 = __shfl_sync(0xffffffffu, t1, off);
+        const int off = row_by_work(m2 - m1, ord);
+        const int t0 = __shfl_sync(0xffffffffu, m1, off), t1 = __shfl_sync(0xffffffffu, m2, off);
         const int i = base + off;
         if (i < P.n) {
             double s[4];
-            ld_row(A + (size_t)dp * BB + q * BS, s);
+            ld_row(A + (size_t)P.diagpos[i] * BB + q * BS, s);
             sub_pairs_f64<VOL>(P, t0, t1, Lin, Uin, s);
             double *su = sh.u + (i - row0) * INV_LD + q * BS;
             su[0] = s[0]; su[1] = s[1]; su[2] = s[2]; su[3] = s[3];
@@ -683,15 +693,20 @@ __device__ __forceinline__ void build_rows_f64(const PatternView &P, int row0,
     }
     // U_ij with no product pair equals A_ij in every sweep: written once per
     // build by k_build_prepare into every buffer, not touched here
-    for (int t = sh.ur[0] + quad; t < sh.ur[rows]; t += BUILD_ROWS) {
-        const int r = list_row(sh.ur, rows, t);
-        const int p = P.diagpos[row0 + r] + 1 + (t - sh.ur[r]);
-        const int t0 = P.pair_ptr[p], t1 = P.pair_ptr[p + 1];
-        if (t0 == t1) continue;
-        double s[4];
-        ld_row(A + (size_t)p * BB + q * BS, s);
-        sub_pairs_f64<VOL>(P, t0, t1, Lin, Uin, s);
-        st_row_sel<VOL>(Uout + (size_t)t * BB + q * BS, s);
+    if (__any_sync(0xffffffffu, m3 > m2)) {
+        const int off = row_by_work<true>(m3 - m2, ord);
+        const int i = base + off, cnt = __shfl_sync(0xffffffffu, m3 - m2, off);
+        if (cnt > 0) {
+            const int dp = P.diagpos[i], p1 = P.rowptr[i + 1], u0 = P.urow[i];
+            for (int p = dp + 1; p < p1; p++) {
+                const int t0 = P.pair_ptr[p], t1 = P.pair_ptr[p + 1];
+                if (t0 == t1) continue;
+                double s[4];
+                ld_row(A + (size_t)p * BB + q * BS, s);
+                sub_pairs_f64<VOL>(P, t0, t1, Lin, Uin, s);
+                st_row_sel<VOL>(Uout + (size_t)(u0 + p - dp - 1) * BB + q * BS, s);
+            }
+        }
     }
     build_cta_invert<double, VOL>(row0, P.n, Dout, sh.u, nsing);
 }

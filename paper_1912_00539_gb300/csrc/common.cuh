@@ -453,16 +453,26 @@ __device__ __forceinline__ C qshfl(C v, int src_q) {
 // pays for 3 in every row.  Groups of four warps (32 rows) therefore hand their
 // rows to quads by decreasing block count.  `key` is the work of row base + lane
 // of the group; returns the offset in the group of this quad's row.  `sh` is the
-// warp's 32 bytes of shared memory; every lane calls it.
+// warp's 32 bytes of shared memory; every lane calls it.  FULL: counts above 4
+// told apart too (32 shuffles; for work of tens of blocks and pairs a row).
+template <bool FULL = false>
 __device__ __forceinline__ int row_by_work(int key, unsigned char *sh) {
     const int lane = threadIdx.x & 31;
-    const int c = min(key, 4);
-    int above = 0, rank = 0;
+    int rank = 0;
+    if constexpr (FULL) {
+        for (int o = 0; o < 32; o++) {
+            const int k = __shfl_sync(0xffffffffu, key, o);
+            rank += k > key || (k == key && o < lane);
+        }
+    } else {
+        const int c = min(key, 4);
+        int above = 0;
 #pragma unroll
-    for (int v = 4; v >= 0; v--) {
-        const unsigned m = __ballot_sync(0xffffffffu, c == v);
-        if (c == v) rank = above + __popc(m & ((1u << lane) - 1u));
-        above += __popc(m);
+        for (int v = 4; v >= 0; v--) {
+            const unsigned m = __ballot_sync(0xffffffffu, c == v);
+            if (c == v) rank = above + __popc(m & ((1u << lane) - 1u));
+            above += __popc(m);
+        }
     }
     sh[rank] = (unsigned char)lane;
     __syncwarp();

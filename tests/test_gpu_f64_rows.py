@@ -24,11 +24,11 @@ def _system(n, longest, seed):
 
 @pytest.mark.gpu
 @pytest.mark.parametrize("n,longest", [(1, 1), (7, 3), (32, 5), (33, 2), (64, 9), (65, 4), (200, 1),
-                                       (333, 14)])
+                                       (333, 14), (130, 3), (96, 40)])
 def test_f64_build_and_sweeps_match_the_oracle(n, longest):
     """Ragged groups of 32 and 64 rows, rows of one block, rows with more blocks
     than the counts that are told apart (4), L and U blocks with and without
-    product pairs.  The oracle runs the same sweeps in FP64 in another order
+    product pairs: in no row, few rows and most rows of a CTA.  The oracle runs the same sweeps in FP64 in another order
     of operations: a few hundred roundings of diagonally dominant blocks."""
     import torch
     import oracle
