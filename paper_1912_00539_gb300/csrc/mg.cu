@@ -128,7 +128,7 @@ k_galerkin(long long nnzb_c, const int4 *__restrict__ grec, const int *__restric
 // r = b - A x, a quad per block row; into r, or rounded into r32 when only the
 // FP32 right-hand side of a smoothing step is wanted (r NULL)
 template <int TH>
-__global__ void __launch_bounds__(TH, TH == STREAM_THREADS ? 1 : 3)
+__global__ void __launch_bounds__(TH, TH == STREAM_THREADS ? 1 : 4)
 k_mg_residual(PatternView P, const double *__restrict__ A, const double *__restrict__ b,
               const double *__restrict__ x, double *__restrict__ r, float *__restrict__ r32,
               Skip skip) {
@@ -137,7 +137,7 @@ k_mg_residual(PatternView P, const double *__restrict__ A, const double *__restr
     pdl_trigger();
     if (skip_all(skip)) return;
     const int q = threadIdx.x & 3;
-    for_rows<TH>(P, A, x, smem, [&](int i) { return __ldg(b + (size_t)i * BS + q); },
+    for_rows<TH, true>(P, A, x, smem, [&](int i) { return __ldg(b + (size_t)i * BS + q); },
         [&](int i, double s, double bi) {
             const size_t o = (size_t)i * BS + q;
             const double v = bi - s;

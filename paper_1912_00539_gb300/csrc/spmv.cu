@@ -30,14 +30,14 @@ constexpr int SPMV_ROWS = SPMV_THREADS / 4;
 // Otherwise y = alpha A x + beta y, and beta == 0 never reads y (which may
 // hold NaN).
 template <bool PLAIN, int TH>
-__global__ void __launch_bounds__(TH, TH == STREAM_THREADS ? 1 : 3)
+__global__ void __launch_bounds__(TH, TH == STREAM_THREADS ? 1 : 4)
 k_spmv(PatternView P, const double *__restrict__ A, double alpha, const double *__restrict__ x,
        double beta, double *__restrict__ y) {
     extern __shared__ __align__(128) char smem[];
     pdl_wait();
     pdl_trigger();
     const int q = threadIdx.x & 3;
-    for_rows<TH>(P, A, x, smem,
+    for_rows<TH, true>(P, A, x, smem,
         [&](int i) { return PLAIN || beta == 0.0 ? 0.0 : y[(size_t)i * BS + q]; },
         [&](int i, double s, double y0) {
             const size_t o = (size_t)i * BS + q;

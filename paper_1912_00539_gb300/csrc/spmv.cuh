@@ -251,9 +251,11 @@ __device__ __forceinline__ double stream_dot(const PatternView &P, const double 
 // The CTA's rows blockIdx.x * TH / 4 .., a grid stride of TH / 4 rows per CTA,
 // below n: post(i, (A x)_i[q], pre(i)) in the quad of row i, pre's loads issued
 // before the row's product.  TH = STREAM_THREADS: through `smem`, the CTA's
-// STREAM_SMEM bytes, free again after a block-wide barrier; else directly.
-// Every thread of the CTA calls it.
-template <int TH, typename Pre, typename Post>
+// STREAM_SMEM bytes, free again after a block-wide barrier; else directly.  ONE:
+// the grid covers the rows, no loop (the direct form then fits 64 registers and
+// four CTAs per SM; product of 262k rows of 9 blocks 75.4 -> 65.1 us, 524k of 4
+// 68.4 -> 62.9).  Every thread of the CTA calls it.
+template <int TH, bool ONE = false, typename Pre, typename Post>
 __device__ __forceinline__ void for_rows(const PatternView &P, const double *__restrict__ A,
                                          const double *__restrict__ x, char *smem, Pre pre, Post post) {
     const int q = threadIdx.x & 3, n = P.n, step = gridDim.x * (TH / 4);
@@ -262,6 +264,7 @@ __device__ __forceinline__ void for_rows(const PatternView &P, const double *__r
         for (; i < n; i += step) {
             auto v = pre(i);
             post(i, row_dot_blocks(P, A, x, i, q), v);
+            if constexpr (ONE) return;
         }
     } else {
         int wi = i - (int)((threadIdx.x & 31) >> 2);   // the warp's first row: its loop is uniform
