@@ -227,7 +227,7 @@ k_residual(PatternView P, const double *__restrict__ A, const double *__restrict
 
 static void launch_residual(int grid, cudaStream_t st, const PatternView &P, const double *A, const double *b,
                             const double *x, double *r, SolveState *S, double *partials, int init) {
-    if (streamed(P.n)) launch_stream<k_residual<false, STREAM_THREADS>>(st, P, A, b, x, r, S, partials, init);
+    if (streamed(P)) launch_stream<k_residual<false, STREAM_THREADS>>(st, P, A, b, x, r, S, partials, init);
     else launch_pdl(k_residual<false>, grid, RED_THREADS, 0, st, P, A, b, x, r, S, partials, init);
 }
 
@@ -593,7 +593,7 @@ static void launch_spmv_dots_n(int grid, cudaStream_t st, const PatternView &P, 
         constexpr int KF = decltype(kf)::value;
         constexpr bool WIDE = decltype(wide)::value;
         if constexpr (KF <= SPMV_DOTS_MAX) {
-            if (!streamed(P.n)) {
+            if (!streamed(P)) {
                 launch_pdl(k_spmv_dots<KF, NORM, WIDE>, grid, RED_THREADS, 0, st, P, A, z, w, V, nv, jp1, S, partials);
                 return;
             }
@@ -603,7 +603,7 @@ static void launch_spmv_dots_n(int grid, cudaStream_t st, const PatternView &P, 
     };
     using F = std::false_type;
     using W = std::true_type;
-    if (!streamed(P.n) && jp1 > SPMV_DOTS_MAX) return go(std::integral_constant<int, SPMV_DOTS_MAX>{}, W{});
+    if (!streamed(P) && jp1 > SPMV_DOTS_MAX) return go(std::integral_constant<int, SPMV_DOTS_MAX>{}, W{});
     switch (jp1) {
     case 1: go(std::integral_constant<int, 1>{}, F{}); break;
     case 2: go(std::integral_constant<int, 2>{}, F{}); break;

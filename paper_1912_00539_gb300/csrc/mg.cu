@@ -148,7 +148,7 @@ k_mg_residual(PatternView P, const double *__restrict__ A, const double *__restr
 
 static void launch_residual(const PatternView &P, const double *A, const double *b, const double *x,
                             double *r, float *r32, cudaStream_t st, Skip skip) {
-    if (streamed(P.n)) launch_stream<k_mg_residual<STREAM_THREADS>>(st, P, A, b, x, r, r32, skip);
+    if (streamed(P)) launch_stream<k_mg_residual<STREAM_THREADS>>(st, P, A, b, x, r, r32, skip);
     else launch_pdl(k_mg_residual<MG_THREADS>, (P.n + MG_ROWS - 1) / MG_ROWS, MG_THREADS, 0, st, P, A, b, x,
                     r, r32, skip);
 }

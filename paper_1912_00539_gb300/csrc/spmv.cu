@@ -50,7 +50,7 @@ abilu_status spmv_launch(const PatternView &P, const double *A, double alpha, co
                          double beta, double *y, cudaStream_t st) {
     const int grid = (P.n + SPMV_ROWS - 1) / SPMV_ROWS;
     const bool plain = alpha == 1.0 && beta == 0.0;
-    if (streamed(P.n)) {
+    if (streamed(P)) {
         if (plain) launch_stream<k_spmv<true, STREAM_THREADS>>(st, P, A, alpha, x, beta, y);
         else launch_stream<k_spmv<false, STREAM_THREADS>>(st, P, A, alpha, x, beta, y);
     } else if (plain) {

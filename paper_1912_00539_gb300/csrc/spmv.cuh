@@ -301,14 +301,21 @@ __device__ __forceinline__ void for_rows(const PatternView &P, const double *__r
     }
 }
 
-// Whether the streamed form takes a system of n rows.  Both forms measured (us,
-// product / FGMRES solve, direct -> streamed): 16k rows 9.3 / 226 -> 9.9 / 236, 51k
-// 9.9 / 305 -> 11.2 / 309, 99k 12.4 / 432 -> 13.3 / 430, 131k 16.4 / 502 -> 15.9 /
-// 499, 262k 37.4 / 802 -> 29.0 / 781: with five passes of 160 rows per SM the
-// pipeline's ramp is paid for.
-constexpr int STREAM_MIN_ROWS = 120000;
+// Whether the streamed form takes a system, by rows and blocks per row (blocks
+// five and on of a row are loaded from global memory as they are used, by 20 warps
+// per SM; the direct form has 24 to 32).  Both forms measured (us, product / FGMRES
+// solve of six steps, direct -> streamed): four blocks a row: 80k rows 10.6 / 314 ->
+// 12.8 / 330, 120k 14.4 / 385 -> 13.9 / 385, 140k 17.1 / 417 -> 16.2 / 410, 262k 35.3 /
+// 596 -> 29.6 / 588, 524k 63.2 / 960 -> 52.8 / 917 (120k: about five passes of 160 rows
+// per SM pay for the pipeline's ramp).  Five: 200k 32.1 / 539 -> 30.9 / 548, 262k
+// 39.7 / 646 -> 37.0 / 643, 700k 93.6 / 1,309 -> 85.5 / 1,267.  Six: 262k 47.1 / 723 ->
+// 50.3 / 738, 700k 112.8 / 1,509 -> 118.8 / 1,505.  Nine, 262k: 65.1 -> 76.4; 26, 125k:
+// 95.2 -> 127.5.
+inline bool streamed(const PatternView &P) {
+    const long long blocks = P.nnzb, n = P.n;
+    return blocks <= 5 * n && n >= (2 * blocks <= 9 * n ? 120000 : 250000);
+}
 int sm_count();
-inline bool streamed(int n) { return n >= STREAM_MIN_ROWS; }
 
 // launch_pdl of a kernel of STREAM_THREADS threads with the stages (its dynamic
 // shared memory allowed once per kernel and device)

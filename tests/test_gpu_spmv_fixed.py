@@ -104,11 +104,13 @@ def test_integers_are_exact():
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("n,blocks", [(119999, 4), (120000, 4), (120001, 7), (121599, 3), (121601, 5)])
+@pytest.mark.parametrize("n,blocks", [(119999, 4), (120000, 4), (120001, 7), (121599, 3), (121601, 5),
+                                      (120001, 9), (250000, 9)])
 def test_streamed_rows_match_the_direct_form(n, blocks):
     """Both sides of the size where the rows go through shared memory, row counts
     that leave the last 160-row pass of some CTAs ragged, rows of 1 .. `blocks`
-    blocks (none to three beyond the staged four).  Both forms run the same
+    blocks (none to five beyond the staged four; five a row and more on average:
+    direct below 250,000 rows).  Both forms run the same
     operations in the same order, so a system's rows give the same bits alone
     (direct) and as the tail of a larger one (streamed)."""
     import torch
