@@ -143,8 +143,13 @@ __device__ __forceinline__ void st_result(double *z, size_t o, double v, int zad
 
 // The right-hand side of an application called with FP64 vectors (R = double) on
 // FP32/BF16 factors is rounded where its first kernel reads it, and that kernel
-// leaves the FP32 copy the later sweeps read in r32 (a conversion pass of its
-// own cost 2.7 us of a 31 us application on 130k cells).
+// leaves the FP32 copy the later sweeps read in r32.  A first kernel that gathers
+// the neighbours' right-hand sides (k_lower_sync) reads each in FP64 and rounds it
+// once per L block; from CONV_PASS_BLOCKS of those a pass that rounds every row once
+// comes first (us, two sweeps each way, in the sweep -> a pass: FP32, 49k L blocks
+// 10.9 -> 14.5, 81k 11.5 -> 13.1, 104k 14.9 -> 14.3, 196k 13.7 -> 13.6, 524k 30.3 -> 26.3,
+// 786k 53.1 -> 44.6; BF16, 786k 54.9 -> 44.7, 1.6M, 12 a row, 57.2 -> 45.2).
+constexpr int CONV_PASS_BLOCKS = 150000;
 template <typename VT> __device__ __forceinline__ VT ld_rhs(const VT *r, size_t o) { return r[o]; }
 template <typename VT>
 __device__ __forceinline__ VT ld_rhs(const std::conditional_t<sizeof(VT) == 4, double, float> *r, size_t o) {
@@ -510,6 +515,19 @@ k_tri_staged(PatternView P, const T *__restrict__ F, const T *__restrict__ D,
     }
 }
 
+// r32 = (float) r
+__global__ void __launch_bounds__(APPLY_THREADS)
+k_to_f32(const double *__restrict__ r, float *__restrict__ r32, long long n4, Skip skip) {
+    pdl_wait();
+    pdl_trigger();
+    if (skip_all(skip)) return;
+    const long long e = ((long long)blockIdx.x * blockDim.x + threadIdx.x) * 4;
+    if (e >= n4) return;
+    float v[4];
+    ld_row(r + e, v);
+    st_row(r32 + e, v);
+}
+
 // v = 0 (n values) unless the launch is skipped: the zero initial guess of the
 // in-place sweeps, as a kernel so that a skipped FGMRES step costs no memset
 template <typename VT>
@@ -565,7 +583,7 @@ static abilu_status apply_t(abilu_factors f, const double *r, const float *r32_i
 
     // right-hand side in the compute type: `conv` while it is still to be
     // rounded into r32 by the first kernel
-    const bool conv = sizeof(VT) == 4 && !r32_in;
+    bool conv = sizeof(VT) == 4 && !r32_in;
     const VT *rv;
     VT *r32 = nullptr;
     if constexpr (sizeof(VT) == 8) {
@@ -573,6 +591,12 @@ static abilu_status apply_t(abilu_factors f, const double *r, const float *r32_i
     } else {
         r32 = reinterpret_cast<float *>(f->r32);
         rv = conv ? r32 : r32_in;
+        if (conv && mode == ABILU_SYNC && nl >= 2 && nu >= 1 && P.nl >= CONV_PASS_BLOCKS) {
+            launch_pdl(k_to_f32, (P.n + APPLY_THREADS - 1) / APPLY_THREADS, APPLY_THREADS, 0, st, r, r32,
+                (long long)P.n * BS, skip);
+            ABILU_LAUNCH_CHECK("k_to_f32");
+            conv = false;
+        }
     }
 
     // FP32 factors: upper sweeps on Us = Dinv U with right-hand side yh = Dinv y
