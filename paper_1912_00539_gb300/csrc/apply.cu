@@ -563,6 +563,21 @@ template <bool UPPER, bool SCALED, bool SYNC, typename T> static int staged_ctas
 }
 
 
+// Whether the FP32/BF16 sweeps of a triangle with `blocks` factor blocks run
+// staged.  A chunk of more than PIPE_CAP blocks reads them from global memory one
+// pair after another; for rows that long the kernels without stages, which read
+// a pair's blocks and its neighbours' values side by side on up to 64 warps per
+// SM, are faster.  Staged -> plain (us, four sweeps each way, FP32 in place; BF16
+// in place; FP32 synchronous): 262k rows of 9 blocks 93.1 -> 81.4; 84.0 -> 74.8; 94.6
+// -> 82.0, 216k of 15 146 -> 121; 106 -> 85; 161 -> 123, 262k of 26 329 -> 258; 267 -> 184;
+// 319 -> 263.  Rows of 7 blocks (192 a chunk): 262k 74.9 -> 67.5; 68.3 -> 63.8; 80.2 ->
+// 72.7, 1 M rows 320 -> 315; 280 -> 304; 310 -> 296 (so a large system's are staged in
+// place).  Rows of 4 (96 a chunk, staged), 524k: 93.4 -> 106.9; 98.1 -> 106.2; 97.2 -> 100.
+static bool staged_rows(int blocks, int n, abilu_mode mode) {
+    const long long per = (long long)PIPE_CAP * n, all = (long long)APPLY_ROWS * blocks;
+    return all <= per || (mode == ABILU_ASYNC && 5 * all <= 7 * per && n >= 500000);
+}
+
 // y_ready (asynchronous mode, FP32/BF16 factors, nl >= 2): the caller already
 // wrote y[0] = the FP32 right-hand side and zeroed the two ticket counters in
 // an earlier kernel on `st` (FGMRES does it where it writes that right-hand
@@ -604,6 +619,8 @@ static abilu_status apply_t(abilu_factors f, const double *r, const float *r32_i
     constexpr bool SC = std::is_same<T, float>::value;
     const T *UU = SC ? reinterpret_cast<const T *>(f->Us) : U;
     const long long n4 = (long long)P.n * BS;
+    const bool staged_l = sizeof(VT) == 4 && staged_rows(P.nl, P.n, mode);
+    const bool staged_u = sizeof(VT) == 4 && staged_rows(P.nu, P.n, mode);
     if (nl == 0 || nu == 0) {  // y = 0, or no upper update: z = x^0 = 0
         if (zadd) return ABILU_OK;
         k_zero<double><<<counted((int)((n4 + 255) / 256)), 256, 0, st>>>(z, n4, skip);
@@ -631,11 +648,13 @@ static abilu_status apply_t(abilu_factors f, const double *r, const float *r32_i
         unsigned long long *err = f->ctr + 4;
         const unsigned long long lim = spin_limit_or_default(f->spin_limit);
         if (nl >= 2) {
-            if constexpr (sizeof(VT) == 4) {  // staged pipeline (FP32/BF16 factors)
-                const int c = staged_ctas<false, false, false, T>();
-                const int g = (int)(c < nchunks ? c : nchunks);
-                launch_pdl(k_tri_staged<false, false, false, T>, g, PIPE_THREADS, 0, st,
-                    P, L, D, rv, nullptr, y[0], nl - 1, 0, x1, yh, z1, zadd, tk, err, skip, lim);
+            if (staged_l) {  // pipeline (FP32/BF16 factors)
+                if constexpr (sizeof(VT) == 4) {
+                    const int c = staged_ctas<false, false, false, T>();
+                    const int g = (int)(c < nchunks ? c : nchunks);
+                    launch_pdl(k_tri_staged<false, false, false, T>, g, PIPE_THREADS, 0, st,
+                        P, L, D, rv, nullptr, y[0], nl - 1, 0, x1, yh, z1, zadd, tk, err, skip, lim);
+                }
             } else {
                 const int ctas_l = lower_async_ctas<T, VT>();
                 const int g = (int)(ctas_l < nchunks ? ctas_l : nchunks);
@@ -645,12 +664,14 @@ static abilu_status apply_t(abilu_factors f, const double *r, const float *r32_i
             ABILU_LAUNCH_CHECK("lower async");
         }
         if (nu >= 2) {
-            if constexpr (sizeof(VT) == 4) {
-                const int c = staged_ctas<true, SC, false, T>();
-                const int g = (int)(c < nchunks ? c : nchunks);
-                launch_pdl(k_tri_staged<true, SC, false, T>, g, PIPE_THREADS, 0, st,
-                    P, UU, D, SC ? y[1] : y[0], nullptr, x[0], nu - 1, 0, nullptr, nullptr, z, zadd, tk + 1,
-                    err, skip, lim);
+            if (staged_u) {
+                if constexpr (sizeof(VT) == 4) {
+                    const int c = staged_ctas<true, SC, false, T>();
+                    const int g = (int)(c < nchunks ? c : nchunks);
+                    launch_pdl(k_tri_staged<true, SC, false, T>, g, PIPE_THREADS, 0, st,
+                        P, UU, D, SC ? y[1] : y[0], nullptr, x[0], nu - 1, 0, nullptr, nullptr, z, zadd, tk + 1,
+                        err, skip, lim);
+                }
             } else {
                 const int ctas_u = upper_async_ctas<T, VT>();
                 const int g = (int)(ctas_u < nchunks ? ctas_u : nchunks);
@@ -704,12 +725,14 @@ static abilu_status apply_t(abilu_factors f, const double *r, const float *r32_i
     for (int s = 2; s <= nu; s++) {  // x^s in x[s & 1], the last one to z
         const bool last = s == nu;
         const VT *xin = s == 2 ? xfirst : x[(s - 1) & 1];
-        if constexpr (sizeof(VT) == 4) {
-            const int c = staged_ctas<true, SC, true, T>();
-            const int g = c < grid ? c : grid;
-            launch_pdl(k_tri_staged<true, SC, true, T>, g, PIPE_THREADS, 0, st,
-                P, UU, D, yfin, xin, last ? nullptr : x[s & 1], 1, last ? 1 : 0, nullptr, nullptr,
-                last ? z : nullptr, zadd, nullptr, f->ctr + 4, skip, spin_limit_or_default(f->spin_limit));
+        if (staged_u) {
+            if constexpr (sizeof(VT) == 4) {
+                const int c = staged_ctas<true, SC, true, T>();
+                const int g = c < grid ? c : grid;
+                launch_pdl(k_tri_staged<true, SC, true, T>, g, PIPE_THREADS, 0, st,
+                    P, UU, D, yfin, xin, last ? nullptr : x[s & 1], 1, last ? 1 : 0, nullptr, nullptr,
+                    last ? z : nullptr, zadd, nullptr, f->ctr + 4, skip, spin_limit_or_default(f->spin_limit));
+            }
         } else {
             launch_pdl(k_upper_sync<T, VT, SC>, grid, APPLY_THREADS, 0, st,
                 P, UU, D, yfin, xin, last ? nullptr : x[s & 1], last ? z : nullptr, zadd, skip);
@@ -728,11 +751,15 @@ void apply_warm(abilu_dtype dt) {
         staged_ctas<false, false, false, float>();
         staged_ctas<true, true, false, float>();
         staged_ctas<true, true, true, float>();
+        lower_async_ctas<float, float>();
+        upper_async_ctas<float, float>();
         break;
     case ABILU_BF16:
         staged_ctas<false, false, false, __nv_bfloat16>();
         staged_ctas<true, false, false, __nv_bfloat16>();
         staged_ctas<true, false, true, __nv_bfloat16>();
+        lower_async_ctas<__nv_bfloat16, float>();
+        upper_async_ctas<__nv_bfloat16, float>();
         break;
     }
 }
