@@ -860,22 +860,16 @@ __global__ void k_export(PatternView P, const T *__restrict__ L, const T *__rest
     if (X) {
         const int p0 = P.rowptr[i], p1 = P.rowptr[i + 1], dp = P.diagpos[i];
         const int lb = P.lrow[i], ub = P.urow[i];
-        // four blocks of the row at a time, every load issued before any store
-        for (int pb = p0; pb < p1; pb += 4) {
-            typename BuildArith<T>::C v[4][4];
-#pragma unroll
-            for (int k = 0; k < 4; k++) {
-                const int p = pb + k;
-                if (p >= p1) break;
-                const T *src = p < dp ? L + (size_t)(lb + p - p0) * BB
-                               : p > dp ? U + (size_t)(ub + p - dp - 1) * BB : Udiag + (size_t)i * BB;
-                ld_row(src + q * BS, v[k]);
-            }
-#pragma unroll
-            for (int k = 0; k < 4; k++) {
-                if (pb + k >= p1) break;
-                st_row(X + (size_t)(pb + k) * BB + q * BS, v[k]);
-            }
+        // One block at a time, its source chosen by address (no divergent loads).
+        // Four at a time, every load issued before any store, was slower on any
+        // pattern but the smallest (us, FP32, four -> one): 524k rows of 4 blocks 95.1 -> 89.3
+        // (BF16 105 -> 82), 262k of 5 64.4 -> 57.3, of 7 78.7 -> 72.9, of 9 97.8 -> 89.5.
+        for (int p = p0; p < p1; p++) {
+            typename BuildArith<T>::C v[4];
+            const T *src = p < dp ? L + (size_t)(lb + p - p0) * BB
+                           : p > dp ? U + (size_t)(ub + p - dp - 1) * BB : Udiag + (size_t)i * BB;
+            ld_row(src + q * BS, v);
+            st_row(X + (size_t)p * BB + q * BS, v);
         }
     }
     if (Dinv) {
