@@ -31,6 +31,9 @@
 
 namespace abilu {
 
+int sm_count();
+
+
 template <typename T> struct BuildArith { using C = float; };
 template <> struct BuildArith<double> { using C = double; };
 
@@ -711,7 +714,13 @@ __device__ __forceinline__ void build_rows_f64(const PatternView &P, int row0,
     build_cta_invert<double, VOL>(row0, P.n, Dout, sh.u, nsing);
 }
 
-__global__ void __launch_bounds__(BUILD_THREADS, 4)
+// CTAS per SM: four, or three for grids that three per SM hold.  A sweep's CTAs are
+// scheduled while the one before drains and fill the SMs that have room first: with
+// room for four, some SMs of a small grid held four and ran last.  6 sweeps (us,
+// four -> three): 125 CTAs 119 -> 105, 250 191 -> 162, 422 284 -> 211, 422 with rows of 26
+// blocks 4,063 -> 3,093; 512 205 -> 236 (more than three per SM: four).
+template <int CTAS>
+__global__ void __launch_bounds__(BUILD_THREADS, CTAS)
 k_build_sync(PatternView P, const double *__restrict__ A, const double *__restrict__ Lin,
              const double *__restrict__ Uin, const double *__restrict__ Din,
              double *__restrict__ Lout, double *__restrict__ Uout, double *__restrict__ Dout,
@@ -972,7 +981,7 @@ static abilu_status sweeps_f64(abilu_factors f, const double *Asrc, int nsweeps,
     if (mode == ABILU_SYNC) {
         for (int s = 0; s < nsweeps; s++) {
             const int c = f->cur, o = 1 - f->cur;
-            launch_pdl(k_build_sync, grid, BUILD_THREADS, 0, st,
+            launch_pdl(grid <= 3 * sm_count() ? k_build_sync<3> : k_build_sync<4>, grid, BUILD_THREADS, 0, st,
                 P, Asrc, L[c], U[c], D[c], L[o], U[o], D[o], s == nsweeps - 1 ? Ud : nullptr,
                 f->ctr);
             ABILU_LAUNCH_CHECK("k_build_sync");
@@ -993,8 +1002,14 @@ static abilu_status sweeps_f64(abilu_factors f, const double *Asrc, int nsweeps,
         if (ctas > grid) ctas = grid;
         if (ctas < 1) ctas = 1;
         const int c = f->cur;
-        launch_pdl(k_build_async, ctas, BUILD_THREADS, 0, st, P, Asrc, L[c], U[c], D[c], Ud,
-            nsweeps, f->ctr, f->ctr + 1);
+        // a grid that leaves room starts when the prepare pass has left every SM, so
+        // that its CTAs spread evenly (250 CTAs, 6 sweeps: 145 -> 116 us)
+        if (ctas < per_sm * sms)
+            k_build_async<<<counted(ctas), BUILD_THREADS, 0, st>>>(P, Asrc, L[c], U[c], D[c], Ud, nsweeps, f->ctr,
+                                                                   f->ctr + 1);
+        else
+            launch_pdl(k_build_async, ctas, BUILD_THREADS, 0, st, P, Asrc, L[c], U[c], D[c], Ud, nsweeps, f->ctr,
+                f->ctr + 1);
         ABILU_LAUNCH_CHECK("k_build_async");
     }
     return ABILU_OK;
