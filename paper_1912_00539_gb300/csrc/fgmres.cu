@@ -1066,11 +1066,14 @@ abilu_status fgmres_run(const PatternView &P, const double *A, abilu_factors ws,
     const bool zero_b = ret == ABILU_OK && h.bnorm == 0.0;
     // b = 0: the solution is x = 0; a solve from a zero guess that failed before
     // it wrote x leaves the guess
-    if (zero_b || (opts->zero_guess && !x_written))
-        ABILU_CUDA(cudaMemsetAsync(x, 0, sizeof(double) * nv, st));
+    if (zero_b || (opts->zero_guess && !x_written)) {
+        const cudaError_t e = cudaMemsetAsync(x, 0, sizeof(double) * nv, st);
+        if (e != cudaSuccess && ret == ABILU_OK) ret = cuda_fail(e, "fgmres zero solution");
+    }
     if (ret != ABILU_OK || zero_b) {   // a cycle that did not finish, or the memset
         k_counters<<<counted(1), 32, 0, st>>>(SS, cl);
         cudaStreamSynchronize(st);
+        if (ret != ABILU_OK) cudaGetLastError();   // ret holds the first error; no later call finds this one
         h = read_status(hs);
     }
     res->iters = h.iters;
