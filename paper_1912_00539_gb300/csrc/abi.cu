@@ -40,13 +40,9 @@ int sm_count() { return red_ctas() / 4; }
 
 static inline bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
-// the solve's workspace: made by the first solve (a handle that only builds,
+// the Krylov vectors: made by the first solve (a handle that only builds,
 // exports or applies needs none), grown by a longer restart
 abilu_status ensure_krylov(abilu_factors f, int m) {
-    if (!f->host_status) {
-        ABILU_CUDA(cudaHostAlloc(&f->host_status, host_status_bytes(), cudaHostAllocMapped));
-        memset(f->host_status, 0, host_status_bytes());
-    }
     if (f->krylov && f->krylov_m >= m) return ABILU_OK;
     if (f->krylov) cudaFree(f->krylov);
     f->krylov = nullptr;
@@ -86,7 +82,11 @@ extern "C" abilu_status abilu_factors_create_scalar(abilu_pattern p, abilu_dtype
     return s;
 }
 
-extern "C" abilu_status abilu_factors_create(abilu_pattern p, abilu_dtype dtype, abilu_factors *out) {
+namespace abilu {
+
+// A handle without the pinned solve status, for factors that no solve is given
+// (an allocation of pinned memory with its release costs tens of microseconds)
+abilu_status factors_create_bare(abilu_pattern p, abilu_dtype dtype, abilu_factors *out) {
     if (!p || !out) return fail(ABILU_EINVAL, "factors_create: NULL argument");
     *out = nullptr;
     size_t esz;
@@ -143,6 +143,23 @@ extern "C" abilu_status abilu_factors_create(abilu_pattern p, abilu_dtype dtype,
     f->cur = 0;
     *out = f;
     return ABILU_OK;
+}
+
+abilu_status factors_add_status(abilu_factors f) {
+    ABILU_CUDA(cudaHostAlloc(&f->host_status, host_status_bytes(), cudaHostAllocMapped));
+    memset(f->host_status, 0, host_status_bytes());
+    return ABILU_OK;
+}
+
+}  // namespace abilu
+
+extern "C" abilu_status abilu_factors_create(abilu_pattern p, abilu_dtype dtype, abilu_factors *out) {
+    abilu_status s = factors_create_bare(p, dtype, out);
+    if (s == ABILU_OK && (s = factors_add_status(*out)) != ABILU_OK) {
+        factors_free(*out);
+        *out = nullptr;
+    }
+    return s;
 }
 
 extern "C" abilu_status abilu_build(abilu_factors f, const double *A, int nsweeps, abilu_mode mode,

@@ -31,6 +31,8 @@ namespace abilu {
 abilu_status build_dispatch(abilu_factors f, const double *A, int nsweeps, abilu_mode mode,
                             abilu_init init, cudaStream_t st);
 abilu_status export_dispatch(abilu_factors f, double *X, double *Dinv, cudaStream_t st);
+abilu_status factors_create_bare(abilu_pattern p, abilu_dtype dtype, abilu_factors *out);
+abilu_status factors_add_status(abilu_factors f);
 abilu_status scan_i32(const int32_t *in, int32_t *out, int n, long long *scratch, unsigned *err,
                       cudaStream_t st);
 abilu_status form_scaled_upper(abilu_factors f, cudaStream_t st);
@@ -297,7 +299,7 @@ static int grid_rows(int n, int per_cta) { return (n + per_cta - 1) / per_cta; }
 static abilu_status factors_from(abilu_pattern p, const double *X, const double *Dinv,
                                  const double *Ap, int sweeps, cudaStream_t st, abilu_factors *out) {
     abilu_factors f = nullptr;
-    abilu_status s = abilu_factors_create(p, ABILU_F64, &f);
+    abilu_status s = factors_create_bare(p, ABILU_F64, &f);
     if (s != ABILU_OK) return s;
     const int c = f->cur;
     k_import<double><<<counted(grid_rows(p->v.n, PLU_THREADS / 4)), PLU_THREADS, 0, st>>>(
@@ -338,7 +340,7 @@ static abilu_status store_as(abilu_factors f64, abilu_dtype dtype, double *X, do
     abilu_status s = export_dispatch(f64, X, D, st);
     if (s != ABILU_OK) return s;
     abilu_factors f = nullptr;
-    if ((s = abilu_factors_create(p, dtype, &f)) != ABILU_OK) return s;
+    if ((s = factors_create_bare(p, dtype, &f)) != ABILU_OK) return s;
     const int c = f->cur;
     k_import<T><<<counted(grid_rows(p->v.n, PLU_THREADS / 4)), PLU_THREADS, 0, st>>>(
         p->v, X, D, static_cast<T *>(f->L[c]), static_cast<T *>(f->U[c]), static_cast<T *>(f->D[c]),
@@ -418,13 +420,13 @@ extern "C" abilu_status abilu_parilut(abilu_pattern pA, const double *A,
     PatternGuard pcur;   // the current pattern when owned (NULL: A's)
     {
         FactorsGuard f0;
-        if ((s = abilu_factors_create(pA, ABILU_F64, &f0.f)) != ABILU_OK) return s;
+        if ((s = factors_create_bare(pA, ABILU_F64, &f0.f)) != ABILU_OK) return s;
         if ((s = build_dispatch(f0.f, A, o->sweeps, ABILU_SYNC, ABILU_INIT_FROM_A, st)) != ABILU_OK) return s;
         if (o->iters == 0) {
             PatternGuard pc;
             if ((s = abilu_pattern_create(n, VA.nnzb, VA.rowptr, VA.colind, stream, &pc.p)) != ABILU_OK) return s;
             FactorsGuard fo;
-            if ((s = abilu_factors_create(pc.p, ABILU_F64, &fo.f)) != ABILU_OK) return s;
+            if ((s = factors_create_bare(pc.p, ABILU_F64, &fo.f)) != ABILU_OK) return s;
             if ((s = build_dispatch(fo.f, A, o->sweeps, ABILU_SYNC, ABILU_INIT_FROM_A, st)) != ABILU_OK) return s;
             if (o->factor_dtype != ABILU_F64) {
                 double *Xs = nullptr;
@@ -436,6 +438,7 @@ extern "C" abilu_status abilu_parilut(abilu_pattern pA, const double *A,
                 if (s != ABILU_OK) return s;
                 std::swap(fo.f, fn.f);
             }
+            if ((s = factors_add_status(fo.f)) != ABILU_OK) return s;
             ABILU_CUDA(cudaStreamSynchronize(st));
             *pattern_out = pc.p;
             *factors_out = fo.f;
@@ -519,6 +522,7 @@ extern "C" abilu_status abilu_parilut(abilu_pattern pA, const double *A,
                 if (s != ABILU_OK) return s;
                 std::swap(f3.f, fn.f);   // the FP64 factors are released with fn
             }
+            if ((s = factors_add_status(f3.f)) != ABILU_OK) return s;
             ABILU_CUDA(cudaStreamSynchronize(st));
             *pattern_out = p3.p;
             *factors_out = f3.f;
