@@ -792,7 +792,8 @@ k_copy_segs(const __grid_constant__ CopySegs c) {
 
 // The copies of one call, launched together.  Arrays the kernel cannot take
 // (not on a 16-byte boundary; host memory, or another device's) go through
-// cudaMemcpyAsync at once, in the same stream.
+// cudaMemcpyAsync at once, in the same stream, behind the queued copies when
+// their destinations overlap one of them.
 struct Copies {
     CopySegs c;
     int dev, grid;
@@ -825,17 +826,18 @@ struct Copies {
         const long long n2 = (long long)(doubles / 2);
         if (n2 == 0) return ABILU_OK;
         const long long tiles = (n2 + COPY_TILE - 1) / COPY_TILE;
-        if (!here(src) || !here(dst) || tiles > (1 << 30)) {
-            ABILU_CUDA(cudaMemcpyAsync(dst, src, sizeof(double) * doubles, kind, st));
-            return ABILU_OK;
-        }
-        bool full = c.count == COPY_SEGS || c.tile0[c.count] + tiles > (1ll << 30);
+        const bool direct = here(src) && here(dst) && tiles <= (1 << 30);
+        bool full = direct && (c.count == COPY_SEGS || c.tile0[c.count] + tiles > (1ll << 30));
         for (int k = 0; k < c.count; k++)   // a destination given twice: in order
             full |= reinterpret_cast<double *>(c.dst[k]) < dst + doubles &&
                     dst < reinterpret_cast<double *>(c.dst[k] + c.n2[k]);
         if (full) {
             abilu_status s = flush();
             if (s != ABILU_OK) return s;
+        }
+        if (!direct) {
+            ABILU_CUDA(cudaMemcpyAsync(dst, src, sizeof(double) * doubles, kind, st));
+            return ABILU_OK;
         }
         c.src[c.count] = reinterpret_cast<const double2 *>(src);
         c.dst[c.count] = reinterpret_cast<double2 *>(dst);
