@@ -463,16 +463,16 @@ k_b_update_scale(const double *__restrict__ V, size_t nv, int j, const double *_
     }
 }
 
-// y = R^{-1} g, a CTA per system: R's upper triangle, g and the reciprocals of
-// R's diagonal in shared memory by the whole CTA, the back substitution by one
-// thread from there (a thread per system reading them as it went took 12 us for
-// four systems).  Also resets the cycle flags {all done, active count} for the
-// residual kernel that starts the next cycle.
+// y = R^{-1} g, a CTA per system: R's upper triangle and g in shared memory by
+// the whole CTA, the back substitution by one thread from there (a thread per
+// system reading them as it went took 12 us for four systems).  Also resets the
+// cycle flags {all done, active count} for the residual kernel that starts the
+// next cycle.
 __global__ void __launch_bounds__(128)
 k_b_ysolve(BState *S, int *bflag) {
     pdl_wait();
     pdl_trigger();
-    __shared__ double sR[BMAXM * (BMAXM + 1) / 2], sg[BMAXM], sinv[BMAXM];
+    __shared__ double sR[BMAXM * (BMAXM + 1) / 2], sg[BMAXM];
     BState *St = S + blockIdx.x;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         bflag[0] = 1;
@@ -483,17 +483,14 @@ k_b_ysolve(BState *S, int *bflag) {
         const int i = t / kd, k = t % kd;
         if (k >= i) sR[i * kd - i * (i - 1) / 2 + (k - i)] = St->H[i * BMAXM + k];
     }
-    for (int t = threadIdx.x; t < kd; t += blockDim.x) {
-        sg[t] = St->g[t];
-        sinv[t] = 1.0 / St->H[t * BMAXM + t];
-    }
+    for (int t = threadIdx.x; t < kd; t += blockDim.x) sg[t] = St->g[t];
     __syncthreads();
     if (threadIdx.x == 0) {
         for (int i = kd - 1; i >= 0; i--) {
             const double *Ri = sR + i * kd - i * (i - 1) / 2 - i;   // Ri[k] = R[i][k], k >= i
             double v = sg[i];
             for (int k = i + 1; k < kd; k++) v -= Ri[k] * sg[k];
-            sg[i] = v * sinv[i];
+            sg[i] = v / Ri[i];
         }
     }
     __syncthreads();
