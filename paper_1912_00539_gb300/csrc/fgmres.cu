@@ -94,7 +94,8 @@ __device__ __forceinline__ void publish_counters(HostStatus *hs, const CtrList &
 }
 
 // In the first CTA of the kernel after a Gram-Schmidt step or a residual: that
-// kernel's status to the host-mapped mirror (see givens_column)
+// kernel's status to the host-mapped mirror, off that kernel's serial tail (the
+// system-scope fence of the host-mapped stores overlaps this kernel's work)
 __device__ __forceinline__ void publish_early(SolveState *S) {
     if (blockIdx.x == 0 && threadIdx.x == 0) publish(S);
 }
@@ -349,13 +350,10 @@ __device__ __forceinline__ void dots_tile(const double2 *__restrict__ V2, long l
 
 // The Givens update of column j of the Hessenberg matrix (from the
 // Gram-Schmidt coefficients h, plus h2 after a second pass) with
-// h_{j+1,j} = hn, the residual estimate and the end-of-cycle test.  One
-// thread of the last CTA.  With `pub` the status goes to the host-mapped
-// mirror here; otherwise the next kernel's first CTA publishes it at its start
-// (publish_early), off this kernel's serial tail: the system-scope fence of
-// the host-mapped stores then overlaps that kernel's work.
-__device__ __forceinline__ void givens_column(SolveState *S, int j, int two_pass, double hn,
-                                              bool pub = true) {
+// h_{j+1,j} = hn, the residual estimate and the end-of-cycle test, for the forms
+// whose norm needs the updated w (the single-reduction form: givens_update).  One
+// thread of the last CTA.
+__device__ __forceinline__ void givens_column(SolveState *S, int j, int two_pass, double hn) {
     // the previous rotations, i = 0 .. j-1, each mixing entries i and i+1 of
     // the new column: entry i+1 is still the Gram-Schmidt coefficient when
     // rotation i reaches it, so one carried value replaces a column array
@@ -384,7 +382,7 @@ __device__ __forceinline__ void givens_column(SolveState *S, int j, int two_pass
                S->iters >= S->max_iters || j + 1 >= S->m) ? 1 : 0;
     S->hn_inv = hn != 0.0 ? 1.0 / hn : 0.0;
     S->counter = 0;
-    if (pub) publish(S);
+    publish(S);
 }
 
 // The last CTA of a dot-product pass: h[k] = sum over CTAs of the partials of
