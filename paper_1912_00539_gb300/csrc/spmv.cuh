@@ -26,12 +26,16 @@ namespace abilu {
 //
 // Precision: each product of two 53-bit significands, aligned to the largest
 // product's exponent, is kept to 2^-58 of the largest product (off by at most
-// three such units) and added exactly in 64 bits; the sum is rounded once.
-// Eight FP64 FMAs round eight times, to 2^-53 of the running sum.  On random
-// products its error was half of theirs (rms 6.5e-17 against 1.4e-16 of the
-// largest product, largest 5.8e-16 against 1.4e-15), and a whole product of the
-// 512x512 grid is 1.1e-16 from the exact one where FMAs gave 1.5e-16.  Sums of
-// integers below 2^26 stay exact.
+// three such units) and added exactly in 64 bits; the sum is rounded once: at most
+// 24 2^-58 of the largest product and half an ulp of the sum away.  Eight FP64 FMAs
+// round eight times, to 2^-53 of the running sum.  On random products its error was
+// half of theirs (rms 6.5e-17 against 1.4e-16 of the largest product, largest 5.8e-16
+// against 1.4e-15), and a whole product of the 512x512 grid is 1.1e-16 from the
+// exact one where FMAs gave 1.5e-16.  The bound is relative to the largest product,
+// not to the sum: where large products cancel before small ones are added, FMAs
+// keep the small ones (1e20, -1e20, 1 in this order: 1) and this sum does not (0), as
+// FMAs in another order would not.  Sums of integers stay exact while every partial sum
+// of FMAs would be (operands up to 2^25: eight products of 2^50).
 //
 // Range: taken when every operand is below 2^478 in magnitude and the largest
 // product is at least 2^-446: then a zero's or subnormal's product (exponent

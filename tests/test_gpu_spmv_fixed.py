@@ -103,6 +103,58 @@ def test_integers_are_exact():
             assert y[i, q] == float(s)
 
 
+def _only_integer_part(n, seed):
+    """Rows 4 .. n-1 of blocks in columns 0, 1, 2 and the diagonal, x zero in columns
+    0 and 1: the sum is that of the third and fourth block alone."""
+    rng = np.random.default_rng(seed)
+    cols = [sorted({i}) if i < 4 else [0, 1, 2, i] for i in range(n)]
+    rowptr = np.cumsum([0] + [len(c) for c in cols]).astype(np.int32)
+    return rng, rowptr, np.concatenate(cols).astype(np.int32)
+
+
+def _exact_rows(rowptr, A, x, colind, rows):
+    for i in rows:
+        for q in range(4):
+            t = [Fraction(float(A[p, q, c])) * Fraction(float(x[colind[p], c]))
+                 for p in range(rowptr[i], rowptr[i + 1]) for c in range(4)]
+            yield i, q, sum(t), max(abs(v) for v in t)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("gap", [0, 20, 45, 70])
+def test_cancelling_products_keep_the_bound_of_the_largest(gap):
+    """Two products of 2^gap and its negative ahead of six of about 1: each product is
+    kept to 3 units of 2^-58 of the largest, and one rounding follows.  (FMAs in this
+    order would keep the small ones whatever the gap.)"""
+    n = 40
+    rng, rowptr, colind = _only_integer_part(n, gap)
+    A = rng.standard_normal((rowptr[-1], 4, 4))
+    x = rng.standard_normal((n, 4))
+    x[:2] = 0.0
+    x[2, 0] = x[2, 1] = 1.75 * 2.0**(gap // 2)
+    third = rowptr[4:-1] + 2
+    A[third, :, 0] *= 2.0**(gap - gap // 2)
+    A[third, :, 1] = -A[third, :, 0]
+    y = _run(rowptr, colind, A, x)
+    for i, q, s, m in _exact_rows(rowptr, A, x, colind, range(4, n)):
+        got = Fraction(float(y[i, q]))
+        assert abs(got - s) <= 24 * m / 2**58 + abs(got) / 2**53, (i, q)
+
+
+@pytest.mark.gpu
+def test_integers_up_to_2_25_are_exact():
+    n = 60
+    rng, rowptr, colind = _only_integer_part(n, 1)
+    A = rng.integers(-2**25, 2**25 + 1, (rowptr[-1], 4, 4)).astype(np.float64)
+    x = rng.integers(-2**25, 2**25 + 1, (n, 4)).astype(np.float64)
+    x[:2] = 0.0
+    x[2], x[7] = 2.0**25, 2.0**25
+    A[rowptr[7] + 2:rowptr[7] + 4] = 2.0**25   # eight products of 2^50
+    y = _run(rowptr, colind, A, x)
+    for i, q, s, _ in _exact_rows(rowptr, A, x, colind, range(4, n)):
+        assert y[i, q] == float(s) and Fraction(float(y[i, q])) == s, (i, q)
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("n,blocks", [(119999, 4), (120000, 4), (120001, 7), (121599, 3), (121601, 5),
                                       (120001, 9), (250000, 9)])
