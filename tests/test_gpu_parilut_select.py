@@ -30,13 +30,16 @@ def test_kept_blocks(nx, ny, fill):
 
 @pytest.mark.gpu
 @pytest.mark.parametrize("fill", [0.0, 0.3, 0.75])
-@pytest.mark.parametrize("scale", [1.0, 1e-170])
+@pytest.mark.parametrize("scale", [1.0, 1e-160, 1e-170])
 def test_ties(fill, scale):
     """Off-diagonal blocks of three distinct norms, so the wanted rank falls among
-    equal keys; and keys that are subnormal or zero (norms squared of 1e-340)."""
+    equal keys (squared norms): normal; subnormal and still distinct (4, 16 and 36
+    times 1e-320); all zero (1e-340)."""
     s = gen.small_system(13, 9, seed=6)
     vals = s.vals.copy()
     rows = np.repeat(np.arange(s.n), np.diff(s.rowptr))
     off = rows != s.colind
     vals[off] = np.eye(4) * scale * (1.0 + (s.colind[off] % 3))[:, None, None]
+    keys = np.unique((vals[off] * vals[off]).sum(axis=(1, 2)))
+    assert len(keys) == (1 if scale == 1e-170 else 3)
     _compare(s, vals, fill)
