@@ -249,7 +249,8 @@ abilu_status abilu_factors_set_spin_limit(abilu_factors f, int64_t limit);
 /* Launch shape of the asynchronous block build (FP32/BF16 factors): the work
  * blocks a warp takes per ticket from the build's queue (a multiple of 32 in
  * 32..512; 0 restores the default: 128, or at most 64 consecutive blocks
- * for work lists that give each resident warp no more).  A ticket is made of sub-chunks of
+ * for work lists that give each resident warp no more; exactly 64 of them where
+ * most rows are coupled to the row before them).  A ticket is made of sub-chunks of
  * 64 consecutive blocks (32 for sizes that are not multiples of 64) spread
  * evenly over the work list, so the blocks in flight cover one short span in
  * each part of the list.  Any value gives a legal asynchronous iteration

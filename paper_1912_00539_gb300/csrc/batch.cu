@@ -1274,7 +1274,7 @@ __global__ void k_relocate(PatternView s, Reloc o, int32_t *__restrict__ rowptr,
 struct SrvMember {
     int id;
     abilu_pattern p;                       // local analysis, owned
-    int n, nnzb, np, nl, nu, npairs, nwork, max_row;
+    int n, nnzb, np, nl, nu, npairs, nwork, max_row, line_rows;
     int R, B, Lb, Ub, Pb, Wb;              // offsets in the current layout
     int laid;                              // placed in the current layout
     int warm;                              // its factors in the arena are a previous update's
@@ -1561,6 +1561,7 @@ static abilu_status server_admit(abilu_server sv, abilu_pattern p, int32_t *id) 
     m.npairs = (int)p->v.npairs;
     m.nwork = p->v.nwork;
     m.max_row = p->max_row;
+    m.line_rows = p->line_rows;
     if (t[2] + m.nl > c.nl || t[3] + m.nu > c.nu || t[4] + m.npairs > c.pairs ||
         t[5] + m.work_p() > c.work)
         return fail(ABILU_ENOMEM, "server_add: the arena has no room for the system's L/U blocks, "
@@ -1592,7 +1593,7 @@ static abilu_status server_relayout(abilu_server sv, const std::vector<int> &ord
     const int k = (int)order.size();
     std::vector<Reloc> rel(k);
     long long R = 0, B = 0, Lb = 0, Ub = 0, Pb = 0, Wb = 0;
-    int maxrow = 0;
+    int maxrow = 0, lines = 0;
     for (int q = 0; q < k; q++) {
         const SrvMember &m = sv->mem[order[q]];
         rel[q] = Reloc{(int)R, m.n, m.np, (int)B, m.nnzb, (int)Lb, m.nl, (int)Ub, m.nu, (int)Pb,
@@ -1604,6 +1605,7 @@ static abilu_status server_relayout(abilu_server sv, const std::vector<int> &ord
         Pb += m.npairs;
         Wb += m.work_p();
         maxrow = m.max_row > maxrow ? m.max_row : maxrow;
+        lines += m.line_rows;
     }
     // the warm factors of continuing systems: current buffer, old place ->
     // other buffer, new place
@@ -1686,6 +1688,7 @@ static abilu_status server_relayout(abilu_server sv, const std::vector<int> &ord
     v.npairs = Pb;
     v.nwork = (int32_t)Wb;
     P->max_row = maxrow;
+    P->line_rows = lines;
     abilu_status sst = batch_super_chunks(b, sv->staging + 2 * (sv->cap.rows / 64) + sv->cap.sys + 1,
                                           st);
     if (sst != ABILU_OK) return sst;

@@ -462,7 +462,7 @@ k_build_blocks_sync(PatternView P, const float *__restrict__ A32, const T *__res
 // falls as the blocks in flight (resident warps x blocks per ticket) span
 // fewer consecutive blocks, because then more of the rows a block reads were
 // already updated in the current sweep (the in-place iteration's Gauss-Seidel
-// effect).  At 512x512 (1.31 M work blocks, 6,080 warps), 6 sweeps, tickets
+// effect).  At 512x512 (1.31 M work blocks, 40 warps per SM then), 6 sweeps, tickets
 // of 128 consecutive blocks left an ILU residual of 44 in 437.7 us, of 64
 // blocks 4.1 in 442-444 us (twice the atomics on the one contended counter).
 // A 128-block ticket made of two 64-block sub-chunks half the list apart (the
@@ -491,23 +491,29 @@ __host__ __device__ __forceinline__ long long build_tickets(int nwork, int wchun
 }
 
 // Lists of at most SMALL_TICKET blocks per resident warp (7,296 warps at 48 per
-// SM: 467k blocks, 187k grid cells) take the smallest ticket, a multiple of 8
-// consecutive blocks (SUB = 8), that gives no more tickets than warps, so a sweep
-// is at most one ticket per warp.  Such lists are bound by the serial steps of a
-// ticket: with 128-block tickets a 20k-block list kept 160 warps busy for 16
-// dependent steps per sweep.  Measured, 4 sweeps with the prepare pass, 40 warps
-// per SM (us, 128-block tickets -> this rule): 2.4k blocks 80 -> 30, 20k 91 -> 34,
-// 82k 96 -> 53, 144k 105 -> 68, 327k 149 -> 124.  Above the line the 64-block groups
-// win: 737k blocks 253 against 286.  Consecutive blocks, not the strided ones
-// of the large lists: on wall-normal lines (coupling 100x along the line) a
-// warp that updates a piece of a line in order carries it as Gauss-Seidel does;
-// FGMRES on 182k cells in line order took 3 iterations (587 us per solve), 5.3
-// with 8-block pieces half the list apart (848), 3 with 128-block tickets (682).
-// Whole solves over 26 drawn grids of 3k to 435k cells, both orderings: all
-// faster than with 128-block tickets, iterations the same in RCM order, up to
-// one more (3 -> 4) on the smallest lines.  Fixing each warp's blocks for all
-// sweeps (no tickets, no flags) was faster still (20k: 22) but lets warps drift
-// apart by sweeps: FGMRES took 24 iterations where the ordered tickets take 7.
+// SM: 467k blocks, 187k grid cells) take tickets of consecutive blocks (a multiple of
+// 8, SUB = 8), at most one per warp and sweep: the smallest that gives no more
+// tickets than warps, or SMALL_TICKET blocks where most rows are coupled to the
+// row before them (lines).  Small lists are bound by the serial steps of a ticket:
+// with 128-block tickets a 20k-block list kept 160 warps busy for 16 dependent
+// steps per sweep.  4 sweeps with the prepare pass, RCM order (us, 128-block tickets
+// -> the smallest): 2k blocks 78 -> 24, 20k 88 -> 28, 81k 121 -> 49, 144k 120 -> 62, 264k
+// 145 -> 95, 450k 186 -> 144; above the line 544k 217 -> 175, 648k 236 -> 209, 800k 259 -> 249,
+// 1.0M equal, 1.3M 378 -> 388, not taken (tickets of more than 64 blocks in one piece lose the
+// shorter span that the strided ones keep).
+//
+// Lines: a warp that updates a piece of a line in order carries it as Gauss-Seidel
+// does, so a coupling of 100x along lines wants long pieces.  FGMRES, line order,
+// 128-block tickets / the smallest / 64 blocks (iterations, us): 8k cells 4.0, 291 / 5.9,
+// 252 / 4.0, 245; 33k 4.5, 356 / 7.9, 404 / 4.5, 318; 45k 5.0, 427 / 15.2, 546 / 5.0, 364; 106k 5.5,
+// 588 / 9.3, 684 / 5.5, 543.  (48 blocks: 238, 294, 337, 492 us, but up to half an iteration
+// more.)  RCM and one-way dissection orders take the same iterations with any ticket,
+// up to two more where the coupling is 100x (33k cells 7.0, 463 / 7.6, 406; 58k 7.5, 552
+// / 9.8, 561, the worst of nine grids).  Pieces half
+// the list apart: 182k cells in line order 5.3 iterations where consecutive ones take 3.
+// Fixing each warp's blocks for all sweeps (no tickets, no flags) was faster still (20k: 22)
+// but lets warps drift apart by sweeps: FGMRES took 24 iterations where the ordered
+// tickets take 7.
 constexpr int SMALL_TICKET = 64;
 
 template <typename T, bool ORDERED, int SUB>
@@ -911,6 +917,7 @@ static abilu_status async_plan(abilu_factors f, AsyncPlan *plan) {
     int wc = f->build_chunk ? f->build_chunk : WARP_CHUNK, sub = build_sub(wc);
     if (!f->build_chunk && (long long)P.nwork <= (long long)SMALL_TICKET * resident) {
         wc = (int)(((long long)P.nwork + 8LL * resident - 1) / (8LL * resident)) * 8;
+        if (2LL * f->p->line_rows > P.n) wc = SMALL_TICKET;
         sub = 8;
     }
     const int wchunks = (int)build_tickets(P.nwork, wc, sub);

@@ -77,8 +77,12 @@ constexpr int WORK_CHUNK = 64;  // work blocks per CTA of the build kernels (<= 
 struct abilu_pattern_s {
     abilu::PatternView v;
     int32_t max_row;
+    // rows coupled to the row before them: a fifth of them in RCM and one-way
+    // dissection orders of a triangulated grid, 0.6 in the natural order, nearly
+    // all where cells follow one another along lines
+    int32_t line_rows;
     int device;
-    void *mem;                 // one allocation holding every array
+    void *mem;                 // its device allocations
 };
 
 struct abilu_factors_s {

@@ -132,7 +132,7 @@ enum : unsigned {
 __global__ void k_pat_rows(int n, int nnzb, const int32_t *__restrict__ rowptr,
                            const int32_t *__restrict__ colind, int32_t *__restrict__ diagpos,
                            int32_t *__restrict__ lcnt, int32_t *__restrict__ ucnt,
-                           unsigned *err, int *max_row) {
+                           unsigned *err, int *max_row, int *line_rows) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     int p0 = rowptr[i], p1 = rowptr[i + 1];
@@ -143,13 +143,16 @@ __global__ void k_pat_rows(int n, int nnzb, const int32_t *__restrict__ rowptr,
     }
     int dp = -1, prev = -1;
     unsigned e = 0;
+    bool next = false;
     for (int p = p0; p < p1; p++) {
         int j = colind[p];
         if (j < 0 || j >= n) e |= PAT_BAD_COL;
         if (j <= prev) e |= PAT_UNSORTED;
         if (j == i) dp = p;
+        next |= j == i - 1;
         prev = j;
     }
+    if (next) atomicAdd(line_rows, 1);
     if (dp < 0) e |= PAT_NO_DIAG;
     if (e) atomicOr(err, e);
     if (dp < 0) dp = p0;
@@ -355,7 +358,7 @@ extern "C" abilu_status abilu_pattern_create(int32_t n, int32_t nnzb, const int3
     int32_t *pair_cnt = i32(o_pcnt), *pair_ptr = i32(o_pptr), *wptr = i32(o_wptr), *wpos = i32(o_wpos);
     long long *scratch = reinterpret_cast<long long *>(m + o_scratch);
     unsigned *err = reinterpret_cast<unsigned *>(m + o_err);
-    int *max_row = reinterpret_cast<int *>(err + 2);
+    int *max_row = reinterpret_cast<int *>(err + 2), *line_rows = max_row + 1;
     auto cu = [&](cudaError_t e, const char *w) -> abilu_status {
         return e == cudaSuccess ? ABILU_OK : cuda_fail(e, w);
     };
@@ -363,7 +366,8 @@ extern "C" abilu_status abilu_pattern_create(int32_t n, int32_t nnzb, const int3
     TRY(cu(cudaMemcpyAsync(d_colind, colind, sizeof(int32_t) * nnzb, cudaMemcpyDeviceToDevice, st), "copy colind"));
     TRY(cu(cudaMemsetAsync(err, 0, sizeof(unsigned) * 4, st), "memset"));
     int gb = (n + 255) / 256;
-    k_pat_rows<<<counted(gb), 256, 0, st>>>(n, nnzb, d_rowptr, d_colind, diagpos, lcnt, ucnt, err, max_row);
+    k_pat_rows<<<counted(gb), 256, 0, st>>>(n, nnzb, d_rowptr, d_colind, diagpos, lcnt, ucnt, err, max_row,
+                                          line_rows);
     TRY(cu(cudaGetLastError(), "k_pat_rows"));
     unsigned herr[4];
     TRY(cu(cudaMemcpyAsync(herr, err, sizeof herr, cudaMemcpyDeviceToHost, st), "read err"));
@@ -448,6 +452,7 @@ extern "C" abilu_status abilu_pattern_create(int32_t n, int32_t nnzb, const int3
     p->v.work = items;
     p->v.wpos = wpos;
     p->max_row = (int)herr[2];
+    p->line_rows = (int)herr[3];
     *out = p;
     return ABILU_OK;
 }
