@@ -133,33 +133,35 @@ __global__ void k_pat_rows(int n, int nnzb, const int32_t *__restrict__ rowptr,
                            const int32_t *__restrict__ colind, int32_t *__restrict__ diagpos,
                            int32_t *__restrict__ lcnt, int32_t *__restrict__ ucnt,
                            unsigned *err, int *max_row, int *line_rows) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    int p0 = rowptr[i], p1 = rowptr[i + 1];
-    if ((i == 0 && p0 != 0) || (i == n - 1 && p1 != nnzb) || p0 < 0 || p1 < p0 || p1 > nnzb) {
-        atomicOr(err, PAT_BAD_ROWPTR);
-        diagpos[i] = 0; lcnt[i] = 0; ucnt[i] = 0;
-        return;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    bool next = false;   // coupled to the row before
+    if (i < n) {
+        const int p0 = rowptr[i], p1 = rowptr[i + 1];
+        if ((i == 0 && p0 != 0) || (i == n - 1 && p1 != nnzb) || p0 < 0 || p1 < p0 || p1 > nnzb) {
+            atomicOr(err, PAT_BAD_ROWPTR);
+            diagpos[i] = 0; lcnt[i] = 0; ucnt[i] = 0;
+        } else {
+            int dp = -1, prev = -1;
+            unsigned e = 0;
+            for (int p = p0; p < p1; p++) {
+                const int j = colind[p];
+                if (j < 0 || j >= n) e |= PAT_BAD_COL;
+                if (j <= prev) e |= PAT_UNSORTED;
+                if (j == i) dp = p;
+                next |= j == i - 1;
+                prev = j;
+            }
+            if (dp < 0) e |= PAT_NO_DIAG;
+            if (e) atomicOr(err, e);
+            if (dp < 0) dp = p0;
+            diagpos[i] = dp;
+            lcnt[i] = dp - p0;
+            ucnt[i] = p1 - dp - (dp < p1 ? 1 : 0);
+            atomicMax(max_row, p1 - p0);
+        }
     }
-    int dp = -1, prev = -1;
-    unsigned e = 0;
-    bool next = false;
-    for (int p = p0; p < p1; p++) {
-        int j = colind[p];
-        if (j < 0 || j >= n) e |= PAT_BAD_COL;
-        if (j <= prev) e |= PAT_UNSORTED;
-        if (j == i) dp = p;
-        next |= j == i - 1;
-        prev = j;
-    }
-    if (next) atomicAdd(line_rows, 1);
-    if (dp < 0) e |= PAT_NO_DIAG;
-    if (e) atomicOr(err, e);
-    if (dp < 0) dp = p0;
-    diagpos[i] = dp;
-    lcnt[i] = dp - p0;
-    ucnt[i] = p1 - dp - (dp < p1 ? 1 : 0);
-    atomicMax(max_row, p1 - p0);
+    const int c = __syncthreads_count(next);   // one atomic per CTA
+    if (threadIdx.x == 0 && c) atomicAdd(line_rows, c);
 }
 
 __global__ void k_pat_cols(int n, const int32_t *__restrict__ rowptr,
