@@ -17,8 +17,8 @@
 // update of every unknown with every read seeing the zero initial guess, one
 // of the orders an asynchronous sweep may run in, and the in-place sweeps then
 // perform the remaining n_L - 1 and n_U - 1 updates of each unknown.  With
-// FP32/BF16 factors the FP64 right-hand side is converted to FP32 once per
-// application (FGMRES hands over the FP32 copy it already wrote).  With FP32
+// FP32/BF16 factors the FP64 right-hand side is converted to FP32 by the
+// first kernel that reads it or by a pass (FGMRES hands over the copy it already wrote).  With FP32
 // factors the upper sweeps run on the Dinv-scaled blocks Us_ij = Dinv_i U_ij
 // formed once per build: x_i = yh_i - sum_{j>i} Us_ij x_j with yh = Dinv y (formed where
 // x^1 = Dinv y is formed), the same iteration without re-reading Dinv in every
@@ -342,7 +342,8 @@ k_upper_async(PatternView P, const T *__restrict__ U, const T *__restrict__ D,
 // volatile, Algorithm 5; SYNC: from the previous iterate `vin`, written to
 // `v`), so each mode computes exactly what its unstaged form computes; only
 // the latency of the ticket, the row pointers and the factor rows leaves the
-// critical path.  A chunk with more than PIPE_CAP factor blocks reads them
+// critical path.  Triangles whose chunks do not fit a stage run the kernels above
+// instead (staged_rows); a single chunk with more than PIPE_CAP factor blocks reads them
 // from global memory.  Lower (UPPER = false): y_i = b_i - sum L_ij y_j; the
 // last update of a row also forms x^1 = Dinv_i y_i into x1 / yh / z.  Upper:
 // x_i = rhs_i - sum Us_ij x_j (SCALED) or Dinv_i (rhs_i - sum U_ij x_j),

@@ -364,7 +364,7 @@ __device__ __forceinline__ void b_dots_norm_last(BState *St, int s, int j, const
 }
 
 // w = A z for the super-chunk's rows (a quad of threads per block row, one
-// 64-row chunk per pass, the SpMV kernel's FMA chain, spmv.cuh) and, from the
+// 64-row chunk per pass, the SpMV kernel's row product, spmv.cuh) and, from the
 // same registers, the dots with V_0..V_{KF-1} and, with NORM, ||w||^2; w is
 // stored once.  The same value-to-thread map as the dot tiles (value e =
 // chunk * 256 + thread), so a later tile of the same kernel re-reads only

@@ -510,7 +510,7 @@ __device__ __forceinline__ void rows_dots_tile(int n, const double *__restrict__
 // w is written once and not read back by a second kernel, and one launch ramp
 // and tail go per step.  Both halves are bound by the FP64 pipe (two lanes
 // per SM), which they now share.  A quad of threads per block row as in the
-// SpMV kernel (row q of each 4x4 block, the same FMA chain, spmv.cuh), rows
+// SpMV kernel (row q of each 4x4 block, the same row product, spmv.cuh), rows
 // in a grid stride.  KF = j + 1 <= SPMV_DOTS_MAX; WIDE (KF = SPMV_DOTS_MAX,
 // any wider step): the tiles of V_KF..V_j follow in the same kernel, each a
 // pass over the thread's own rows that re-reads its entries of w through L2.

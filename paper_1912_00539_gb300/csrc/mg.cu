@@ -31,7 +31,7 @@
 //   pre_smooth smoothing steps, b_c = P^T (b - A x), the cycle on level l+1,
 //   x += P x_c, post_smooth steps; the coarsest level takes coarse_smooth
 //   steps.  The first step from x = 0 is x = M^{-1} b (no residual pass).
-//   Kernels: the residual (the SpMV's FMA chain, spmv.cuh; a quad per row,
+//   Kernels: the residual (the SpMV's row product, spmv.cuh; a quad per row,
 //   coalesced), the restriction (a quad per aggregate summing its cells'
 //   residuals in ascending order), the prolongation; x += z happens in the
 //   application's last sweep.
@@ -83,11 +83,11 @@ k_block_norm2(const double *__restrict__ A, long long nnzb, double *__restrict__
 // the gathers of a coarse block overlap instead of forming a chain.
 //
 // The records are sorted by list length, longest first (a long list started last
-// ran alone at the end; stable, so neighbours in memory stay close): an FP64 add holds this GPU's FP64 pipe for 16 cycles whatever lanes
-// are active, and with the coarse blocks in storage order the eight quads of a
+// ran alone at the end; stable, so neighbours in memory stay close): an FP64 add
+// holds this GPU's FP64 pipe for 16 cycles whatever lanes are active, and with the coarse blocks in storage order the eight quads of a
 // warp waited for its one diagonal block's ten or so entries.  The first entry
 // starts the sum (one add per entry fewer).  512x512 cells x 2, finest level
-// (274 MB read, 26 M adds): 347 us in storage order, 124 sorted (level 2: 112 -> 53).
+// (274 MB read, 26 M adds): 347 us in storage order, 115 sorted (level 2: 112 -> 53).
 __global__ void __launch_bounds__(MG_THREADS)
 k_galerkin(long long nnzb_c, const int4 *__restrict__ grec, const int *__restrict__ gidx,
            const double *__restrict__ A, double *__restrict__ Ac) {

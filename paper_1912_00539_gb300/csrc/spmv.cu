@@ -14,8 +14,8 @@
 // any arithmetic so each thread keeps up to 8 independent 16-byte loads in
 // flight.  Half of a row's products are FP64 FMAs, half integer sums
 // (spmv.cuh).  Large systems stream the rows through shared memory, one CTA
-// per SM: 512x512 51.0 us, 6.1 TB/s (65.7 with FMAs alone, 60.8 before the
-// streamed form).
+// per SM: 512x512 51.0 us, 6.1 TB/s (65.7 with FMAs alone, 62.9 in the direct
+// form).
 #include "common.cuh"
 #include "spmv.cuh"
 
